@@ -33,7 +33,7 @@
 
 #include "internal.cuh"
 #include "jfa_dev.cuh"
-#include "trace_dev.cuh"
+#include "front_dev.cuh"
 #include "vox_dev.cuh"
 
 namespace rtsdf {
@@ -284,92 +284,48 @@ __device__ __forceinline__ void batch_ray_prefix(const BatchArgs& b, unsigned lo
     __syncthreads();
 }
 
-// Stage 5: all scenes' rays from one dynamic counter (the per-scene
-// tracer's persistent-warp traversal; each lane remembers its ray's scene).
-// TEX: node fetches split between the load and texture pipes.
+// Stage 5: all scenes' rays from one dynamic counter, in units that stay
+// within a scene (a fetched range that crosses into the next scene makes two
+// units), traced by the per-scene tracer's warp loop.
+struct BatchUnits {
+    const BatchArgs& b;
+    const unsigned long long* rp;   // ray prefix over scenes
+    int ns;
+    __device__ __forceinline__ const TraceArgs& args(int s) const { return b.sc[s].t; }
+    // the scene's root in the concatenated tree
+    __device__ __forceinline__ int root(int s) const {
+        const SceneDesc& d = b.sc[s];
+        return d.t.nt > 1 ? d.wide_off : (d.t.nt == 1 ? ~d.tri_off : WIDE_EMPTY);
+    }
+    __device__ __forceinline__ bool next(WarpTrace& w, uint32_t unit, unsigned lane, int& scene) const {
+        unsigned long long c0 = w.cnext, end = w.cend;
+        if (c0 == end) {
+            c0 = 0;
+            if (lane == 0) c0 = atomicAdd(b.next_ray, (unsigned long long)unit);
+            c0 = __shfl_sync(0xFFFFFFFFu, c0, 0);
+            if (c0 >= rp[ns]) return false;
+            end = min(c0 + (unsigned long long)unit, rp[ns]);
+        }
+        scene = find_scene(rp, ns, c0);
+        const unsigned long long stop = min(end, rp[scene + 1]);
+        __syncwarp();
+        if (lane == 0) {
+            w.g0 = c0 - rp[scene];
+            w.len = (uint32_t)(stop - c0);
+            w.cnext = stop;
+            w.cend = end;
+        }
+        __syncwarp();
+        return true;
+    }
+};
+
 template <bool TEX>
 __device__ __forceinline__ void batch_trace_rays(const BatchArgs& b, const unsigned long long* s_rp, int ns) {
-    __shared__ int2 s_stack[SMEM_STACK][TRACE_THREADS];
-    // per-warp chunk state, kept in shared memory (read only at refills) so
-    // that the traversal loop keeps its registers
-    __shared__ unsigned long long s_cnext[TRACE_THREADS / 32], s_cend[TRACE_THREADS / 32];
-    __shared__ unsigned long long s_csend[TRACE_THREADS / 32];
-    __shared__ int s_cscene[TRACE_THREADS / 32];
-    __shared__ uint8_t s_scene[TRACE_THREADS];   // scene of each lane's ray (< MAX_BATCH; read at setup and commit)
-    const unsigned lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-    const unsigned lt = (1u << lane) - 1u;
-    int2 deep[TRACE_STACK - SMEM_STACK];
-    Stack stk{&s_stack[0][threadIdx.x], deep};
-    Ray r;
-    bool active = false;
-    bool exhausted = false;
-    uint32_t dummy_v = 0, dummy_t = 0, dummy_l = 0;
-    if (lane == 0) s_cnext[wi] = s_cend[wi] = 0;
-    __syncwarp();
-    for (;;) {
-        unsigned idle = __ballot_sync(0xFFFFFFFFu, !active);
-        while (idle && !exhausted) {
-            unsigned long long cn = s_cnext[wi];
-            if (cn == s_cend[wi]) {
-                unsigned long long c0 = 0;
-                if (lane == 0) c0 = atomicAdd(b.next_ray, (unsigned long long)b.ray_chunk);
-                c0 = __shfl_sync(0xFFFFFFFFu, c0, 0);
-                const unsigned long long total = s_rp[ns];
-                if (c0 >= total) {
-                    exhausted = true;
-                    break;
-                }
-                cn = c0;
-                __syncwarp();
-                if (lane == 0) {
-                    // scene of the chunk's first ray and where that scene ends
-                    const int cs = find_scene(s_rp, ns, c0);
-                    s_cscene[wi] = cs;
-                    s_csend[wi] = s_rp[cs + 1];
-                    s_cend[wi] = min(c0 + (unsigned long long)b.ray_chunk, total);
-                }
-                __syncwarp();
-            }
-            const uint32_t avail = (uint32_t)(s_cend[wi] - cn);
-            const uint32_t want = __popc(idle);
-            const uint32_t take = min(avail, want);
-            if (!active) {
-                const uint32_t rank = __popc(idle & lt);
-                if (rank < take) {
-                    const unsigned long long g = cn + rank;
-                    const int scene = g < s_csend[wi] ? s_cscene[wi] : find_scene(s_rp, ns, g);
-                    s_scene[threadIdx.x] = (uint8_t)scene;
-                    const TraceArgs& ta = b.sc[scene].t;
-                    setup_ray(ta, g - s_rp[scene], r);
-                    // enter the scene's root in the concatenated tree
-                    const SceneDesc& sd = b.sc[scene];
-                    r.node = ta.nt > 1 ? sd.wide_off : WIDE_EMPTY;
-                    r.leaf = ta.nt == 1 ? sd.tri_off : WIDE_EMPTY;
-                    active = true;
-                }
-            }
-            __syncwarp();
-            if (lane == 0) s_cnext[wi] = cn + take;
-            __syncwarp();
-            idle = __ballot_sync(0xFFFFFFFFu, !active);
-        }
-        if (__ballot_sync(0xFFFFFFFFu, active) == 0) break;
-        for (;;) {
-            const bool done = warp_step<false, TEX>(b.bvh, r, stk, active, b.leaf_min, dummy_v, dummy_t, dummy_l);
-            const unsigned fin = __ballot_sync(0xFFFFFFFFu, done);
-            if (fin && done) {
-                const int scene = (int)s_scene[threadIdx.x];
-                const unsigned long long key = ((unsigned long long)scene << 32) | r.slot;
-                const unsigned peers = __match_any_sync(fin, key);
-                const TraceArgs& st = b.sc[scene].t;
-                commit_ray(r, st.nearest != 0, peers, lt, st.ray_min, st.ray_cnt);
-                active = false;
-            }
-            const unsigned act = __ballot_sync(0xFFFFFFFFu, active);
-            if (act == 0) break;
-            if (!exhausted && (32 - __popc(act)) >= b.refill_min) break;
-        }
-    }
+    __shared__ BlockTrace s_trace;
+    BatchUnits src{b, s_rp, ns};
+    const uint32_t unit = unit_rays(s_rp[ns], (uint32_t)b.params->rays, (uint32_t)b.ray_chunk);
+    trace_units<false, TEX>(src, b.bvh, unit, b.refill_min, b.leaf_min, s_trace, nullptr);
 }
 
 // Stage 6: one grid-stride loop over every scene's slots (slot prefix = ray

@@ -306,36 +306,44 @@ ShadowArgs make_args(rtsdf_ctx* c, const float* sdf, const float* pos, const flo
 // blocked point gets visibility 0; the others keep the march's value.
 // TEX: node fetches split between the load and texture pipes, as in the
 // tracer.
+constexpr int SHADOW_STACK = 24;   // entries in shared memory
+struct ShadowStack : dev::Stack<SHADOW_STACK> {
+    float3 o, d;   // the ray
+    __device__ __forceinline__ float3 origin() const { return o; }
+    __device__ __forceinline__ float3 direction() const { return d; }
+    __device__ __forceinline__ bool below(float, int&) { return false; }   // nothing lies below the stack
+};
 template <bool TEX>
 __global__ void __launch_bounds__(dev::TRACE_THREADS) k_shadow_exact(dev::TraceArgs t, const float* __restrict__ pos,
                                                                      const float* __restrict__ nrm, long long npix,
                                                                      float Lx, float Ly, float Lz, float two_eps,
                                                                      float* vis, uint8_t* blocked) {
-    __shared__ int2 s_stack[dev::SMEM_STACK][dev::TRACE_THREADS];
-    int2 deep[TRACE_STACK - dev::SMEM_STACK];
-    dev::Stack stk{&s_stack[0][threadIdx.x], deep};
+    __shared__ int2 s_stack[SHADOW_STACK][dev::TRACE_THREADS];
+    int2 deep[TRACE_STACK - SHADOW_STACK];
+    ShadowStack stk;
+    stk.e = &s_stack[0][threadIdx.x];
+    stk.deep = deep;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= npix) return;                      // no barrier below
     dev::Ray r;
-    r.o = make_float3(fmaf(nrm[3 * i], two_eps, pos[3 * i]), fmaf(nrm[3 * i + 1], two_eps, pos[3 * i + 1]),
-                      fmaf(nrm[3 * i + 2], two_eps, pos[3 * i + 2]));
-    r.d = make_float3(Lx, Ly, Lz);
+    stk.o = make_float3(fmaf(nrm[3 * i], two_eps, pos[3 * i]), fmaf(nrm[3 * i + 1], two_eps, pos[3 * i + 1]),
+                        fmaf(nrm[3 * i + 2], two_eps, pos[3 * i + 2]));
+    stk.d = make_float3(Lx, Ly, Lz);
     r.id = make_float3(dev::safe_inv(Lx), dev::safe_inv(Ly), dev::safe_inv(Lz));
-    r.oid = make_float3(r.o.x * r.id.x, r.o.y * r.id.y, r.o.z * r.id.z);
+    r.oid = make_float3(stk.o.x * r.id.x, stk.o.y * r.id.y, stk.o.z * r.id.z);
     r.bt = CUDART_INF_F;
     r.bidx = 0x7FFFFFFF;
     r.bfront = false;
     r.node = t.nt > 1 ? 0 : WIDE_EMPTY;
     r.leaf = t.nt == 1 ? 0 : WIDE_EMPTY;
     r.sp = 0;
-    r.slot = 0;
     r.steps = 0;
     uint32_t nv = 0, ntest = 0;
     // every step enters a node or tests a leaf (bounded by the step guard);
     // the loop ends at the first hit or when nothing is left
-    while (r.bidx == 0x7FFFFFFF && !dev::ray_done(r)) {
-        dev::node_step<false, TEX>(t, r, stk, nv);
-        if (r.leaf != WIDE_EMPTY) dev::leaf_step<false>(t, r, stk, nv, ntest);
+    while (r.bidx == 0x7FFFFFFF && !(r.node == WIDE_EMPTY && r.leaf == WIDE_EMPTY)) {
+        if (dev::node_step<false, TEX>(t, r, stk, nv)) dev::advance(r, stk);
+        if (r.leaf != WIDE_EMPTY && dev::leaf_step<false>(t, r, stk, nv, ntest)) dev::advance(r, stk);
         dev::step_guard(t, r);
     }
     const bool b = r.bidx != 0x7FFFFFFF;

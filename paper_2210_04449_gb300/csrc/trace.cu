@@ -8,21 +8,22 @@
 //     counter (draw, ray, frame, texel) and key (seed lo, seed hi), mapped to
 //     the sphere by Marsaglia's (1972) rejection method -- integer accept
 //     test, fp32 map, so every direction is bit-reproducible;
-//   * the closest hit comes from a stack traversal of the 4-wide BVH (one
-//     128-byte node fetch tests four child boxes; the nearest hit child is
-//     entered next, the others pushed farthest-first with their entry
-//     distance and skipped on pop once they cannot hold a closer hit),
-//     leaves tested with Moller-Trumbore in fp32 with the operation
-//     order written out (explicit fma / rounding intrinsics); equal
-//     distances keep the smaller original triangle index.
+//   * the closest hit comes from a traversal of the 4-wide BVH that starts
+//     from a front of it, shared by the rays of neighbouring texels
+//     (front_dev.cuh); one 128-byte node fetch tests four child boxes, the
+//     nearest hit child is entered next, the others pushed farthest-first
+//     with their entry distance and skipped on pop once they cannot hold a
+//     closer hit; leaves are tested with Moller-Trumbore in fp32 with the
+//     operation order written out (explicit fma / rounding intrinsics);
+//     equal distances keep the smaller original triangle index.
 // Rays of very different lengths would leave most lanes of a lock-step warp
-// idle, so warps are persistent and refill idle lanes with new ray ids from
-// a warp-local chunk once enough lanes are idle.  The traversal runs in two
+// idle, so warps are persistent and refill idle lanes with new rays once
+// enough lanes are idle.  The traversal runs in two
 // phases (a lane parks the leaf it reaches and keeps descending; the warp
 // tests triangles when enough lanes hold a parked leaf), two node steps per
-// phase decision.  A finished ray commits its distance (atomicMin on the
-// float bits, t >= 0) and its front/back hit into per-slot scratch with
-// warp-aggregated atomics; k_trace_finalize then applies Eq. 1 per texel:
+// phase decision.  A finished ray commits its distance (minimum of the
+// float bits, t >= 0) and its front/back hit to its warp's shared memory, a
+// finished texel to per-slot scratch; k_trace_finalize then applies Eq. 1 per texel:
 // u_t = min(u, r_t) (the alpha decay was applied by the mask kernel), the
 // counts, and f_t = +-u_t (c_t while no ray has hit), negative when back
 // hits outnumber front hits.  In the nearest-face sign mode a ray starts
@@ -30,107 +31,47 @@
 #include <math_constants.h>
 
 #include "internal.cuh"
-#include "trace_dev.cuh"
+#include "front_dev.cuh"
 
 namespace rtsdf {
 namespace {
 
 using namespace dev;
 
-// Persistent warps: each lane traces one ray at a time and takes a new one
-// as soon as it finishes (from a warp-local chunk of consecutive ray ids, so
-// the lanes of a warp mostly share a texel and its origin).  Finished rays
-// commit (min distance, front/back) per texel slot with warp-aggregated
-// atomics; k_trace_finalize then applies Eq. 1 per texel.
-template <bool COUNT, bool TEX>
-__global__ void __launch_bounds__(TRACE_THREADS, 8) k_trace(TraceArgs a) {
-    uint32_t n_visits = 0, n_tests = 0, n_rays = 0;
-    uint32_t n_slots = 0, n_leaf_slots = 0;   // COUNT: traversal iterations, leaf phases run
-    const uint64_t total = (uint64_t)(*a.count) * 8u * (uint64_t)a.rays;
-    const unsigned lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    // traversal stack: the first SMEM_STACK (node, distance) entries in shared
-    // memory laid out [entry][thread], deeper entries in local memory
-    __shared__ int2 s_stack[SMEM_STACK][TRACE_THREADS];
-    int2 deep[TRACE_STACK - SMEM_STACK];
-    Stack stk{&s_stack[0][threadIdx.x], deep};
-    // per-warp chunk of ray ids, kept in shared memory (read only at refills)
-    // so that the traversal loop keeps its registers
-    __shared__ unsigned long long s_cnext[TRACE_THREADS / 32], s_cend[TRACE_THREADS / 32];
-    const unsigned wi = threadIdx.x >> 5;
-    if (lane == 0) s_cnext[wi] = s_cend[wi] = 0;
-    __syncwarp();
-    Ray r;
-    bool active = false;
-    bool exhausted = false;                    // warp-uniform
-    for (;;) {
-        // hand out rays to idle lanes
-        unsigned idle = __ballot_sync(0xFFFFFFFFu, !active);
-        while (idle && !exhausted) {
-            uint64_t cn = s_cnext[wi];
-            if (cn == s_cend[wi]) {
-                unsigned long long b = 0;
-                if (lane == 0) b = atomicAdd(a.next_ray, (unsigned long long)a.ray_chunk);
-                b = __shfl_sync(0xFFFFFFFFu, b, 0);
-                if (b >= total) {
-                    exhausted = true;
-                    break;
-                }
-                cn = b;
-                __syncwarp();
-                if (lane == 0) s_cend[wi] = min((uint64_t)b + (uint64_t)a.ray_chunk, total);
-                __syncwarp();
-            }
-            const uint32_t avail = (uint32_t)(s_cend[wi] - cn);
-            const uint32_t want = __popc(idle);
-            const uint32_t take = min(avail, want);
-            if (!active) {
-                const uint32_t rank = __popc(idle & lt);
-                if (rank < take) {
-                    setup_ray(a, cn + rank, r);
-                    active = true;
-                    if (COUNT) n_rays++;
-                }
-            }
-            __syncwarp();
-            if (lane == 0) s_cnext[wi] = cn + take;
-            __syncwarp();
-            idle = __ballot_sync(0xFFFFFFFFu, !active);
-        }
-        if (__ballot_sync(0xFFFFFFFFu, active) == 0) break;
-        // trace until enough lanes are idle to be worth a refill
-        for (;;) {
-            const bool done = warp_step<COUNT, TEX>(a, r, stk, active, a.leaf_min, n_visits, n_tests, n_leaf_slots);
-            if (COUNT) n_slots += NODE_STEPS;   // lane slots of the node steps
-            const unsigned fin = __ballot_sync(0xFFFFFFFFu, done);
-            if (fin && done) {
-                const unsigned peers = __match_any_sync(fin, r.slot);
-                commit_ray(r, a.nearest != 0, peers, lt, a.ray_min, a.ray_cnt);
-                active = false;
-            }
-            const unsigned act = __ballot_sync(0xFFFFFFFFu, active);
-            if (act == 0) break;
-            if (!exhausted && (32 - __popc(act)) >= a.refill_min) break;
-        }
-    }
-    if (COUNT) {
-        // summed over the warp's lanes, the iteration counts become lane slots
-        unsigned long long rr = n_rays, v = n_visits, t = n_tests, sl = n_slots, ls = n_leaf_slots;
-        for (int off = 16; off >= 1; off >>= 1) {
-            rr += __shfl_xor_sync(0xFFFFFFFFu, rr, off);
-            v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
-            t += __shfl_xor_sync(0xFFFFFFFFu, t, off);
-            sl += __shfl_xor_sync(0xFFFFFFFFu, sl, off);
-            ls += __shfl_xor_sync(0xFFFFFFFFu, ls, off);
-        }
+#ifndef TRACE_MIN_BLOCKS
+#define TRACE_MIN_BLOCKS 8
+#endif
+
+// Units of one scene's rays, handed out in order from the frame's counter.
+struct SceneUnits {
+    const TraceArgs& a;
+    unsigned long long total;
+    __device__ __forceinline__ const TraceArgs& args(int) const { return a; }
+    __device__ __forceinline__ int root(int) const { return a.nt > 1 ? 0 : (a.nt == 1 ? ~0 : WIDE_EMPTY); }
+    __device__ __forceinline__ bool next(WarpTrace& w, uint32_t unit, unsigned lane, int& scene) const {
+        unsigned long long c0 = 0;
+        if (lane == 0) c0 = atomicAdd(a.next_ray, (unsigned long long)unit);
+        c0 = __shfl_sync(0xFFFFFFFFu, c0, 0);
+        if (c0 >= total) return false;
         if (lane == 0) {
-            atomicAdd(&a.counters->rays, rr);
-            atomicAdd(&a.counters->visits, v);
-            atomicAdd(&a.counters->tests, t);
-            atomicAdd(&a.counters->slots, sl);
-            atomicAdd(&a.counters->leaf_slots, ls);
+            w.g0 = c0;
+            w.len = (uint32_t)min((unsigned long long)unit, total - c0);
         }
+        __syncwarp();
+        scene = 0;
+        return true;
     }
+};
+
+template <bool COUNT, bool TEX>
+__global__ void __launch_bounds__(TRACE_THREADS, TRACE_MIN_BLOCKS) k_trace(TraceArgs a) {
+    __shared__ BlockTrace s_trace;
+    __shared__ TraceArgs s_args;   // for the parts that are called
+    if (threadIdx.x == 0) s_args = a;
+    __syncthreads();
+    SceneUnits src{s_args, (unsigned long long)(*a.count) * 8u * (unsigned long long)a.rays};
+    const uint32_t unit = unit_rays(src.total, (uint32_t)a.rays, (uint32_t)a.ray_chunk);
+    trace_units<COUNT, TEX>(src, a, unit, a.refill_min, a.leaf_min, s_trace, a.counters);
 }
 
 // Eq. 1 per traced texel slot (see finalize_slot): a grid-stride loop over

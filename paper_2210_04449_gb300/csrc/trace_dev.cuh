@@ -141,68 +141,35 @@ __device__ __forceinline__ float fmin3(float a, float b, float c) {
     return r;
 }
 
-// Per-lane ray state of the persistent tracer.
+// Per-lane ray state of a traversal.
 struct Ray {
-    float3 o, d, id, oid;
+    float3 id, oid;    // reciprocal direction, origin times it
     float bt;          // closest hit distance so far
     int bidx;          // its original triangle index (0x7FFFFFFF: none)
     bool bfront;
     int node;          // next node to enter (>= 0 internal, < 0 ~leaf, WIDE_EMPTY none)
     int leaf;          // parked leaf waiting for the leaf phase (WIDE_EMPTY none)
     int sp;
-    uint32_t slot;     // texel slot = 8 * (masked-list position) + child
     uint32_t steps;    // nodes entered; a tree of 2 nt - 1 nodes bounds it
 };
 
-__device__ __forceinline__ void setup_ray(const TraceArgs& a, uint64_t g, Ray& r) {
-    const uint32_t slot = (uint32_t)(g >> a.log2_rays);
-    const uint32_t ray = (uint32_t)(g & (uint64_t)(a.rays - 1));
-    const uint32_t parent = a.masked[slot >> 3];
-    const uint32_t ch = slot & 7u;
-    const uint32_t nc = (uint32_t)a.nc, nf = 2u * nc;
-    const uint32_t pq = __umulhi(parent, a.nc_mag), pz = __umulhi(pq, a.nc_mag);
-    const uint32_t px = parent - pq * nc, py = pq - pz * nc;
-    const uint32_t jx = 2 * px + (ch & 1), jy = 2 * py + ((ch >> 1) & 1), jz = 2 * pz + (ch >> 2);
-    const uint32_t texel = jx + nf * (jy + nf * jz);
-    // nearest-face variant: no hit beyond the texel's accumulated distance
-    // can change its result, so the ray starts with that distance as its
-    // best hit (hits at exactly that distance still count: bidx is unset)
-    const float cap = a.nearest ? a.accum[texel] : CUDART_INF_F;
-    r.o = make_float3(__fadd_rn(a.bx, __fmul_rn(__fadd_rn((float)jx, 0.5f), a.hf)),
-                      __fadd_rn(a.by, __fmul_rn(__fadd_rn((float)jy, 0.5f), a.hf)),
-                      __fadd_rn(a.bz, __fmul_rn(__fadd_rn((float)jz, 0.5f), a.hf)));
-    r.d = sphere_dir(a.key0, a.key1, texel, a.frame, ray);
-    r.id = make_float3(safe_inv(r.d.x), safe_inv(r.d.y), safe_inv(r.d.z));
-    r.oid = make_float3(r.o.x * r.id.x, r.o.y * r.id.y, r.o.z * r.id.z);
-    r.bt = cap;
-    r.bidx = 0x7FFFFFFF;
-    r.bfront = false;
-    // the root; a one-triangle mesh has no node, so its leaf starts parked
-    // (a ray with neither a node nor a parked leaf is done)
-    r.node = a.nt > 1 ? 0 : WIDE_EMPTY;
-    r.leaf = a.nt == 1 ? 0 : WIDE_EMPTY;
-    r.sp = 0;
-    r.slot = slot;
-    r.steps = 0;
-}
-
 constexpr int TRACE_THREADS = 128;
-constexpr int SMEM_STACK = 24;
 
 // Traversal stack of one lane: (node, entry distance) pairs, the first
-// SMEM_STACK in shared memory laid out [entry][thread] (a push or pop of a
+// SMEM in shared memory laid out [entry][thread] (a push or pop of a
 // warp is one 64-bit access per lane over distinct banks), deeper entries
 // in local memory.
+template <int SMEM>
 struct Stack {
     int2* e;      // &s_stack[0][thread], stride TRACE_THREADS
     int2* deep;   // local overflow
     __device__ __forceinline__ void push(int sp, int node, float t0) {
         const int2 v = make_int2(node, __float_as_int(t0));
-        if (sp < SMEM_STACK) e[sp * TRACE_THREADS] = v;
-        else deep[sp - SMEM_STACK] = v;
+        if (sp < SMEM) e[sp * TRACE_THREADS] = v;
+        else deep[sp - SMEM] = v;
     }
     __device__ __forceinline__ void pop(int sp, int& node, float& t0) const {
-        const int2 v = sp < SMEM_STACK ? e[sp * TRACE_THREADS] : deep[sp - SMEM_STACK];
+        const int2 v = sp < SMEM ? e[sp * TRACE_THREADS] : deep[sp - SMEM];
         node = v.x;
         t0 = __int_as_float(v.y);
     }
@@ -218,14 +185,20 @@ struct Stack {
 
 // Pop the next entry that can still hold a hit at distance <= bt, parking
 // leaves while the lane's slot is free; stops at an internal node, at a leaf
-// behind the parked one, or with the stack empty (r.node = WIDE_EMPTY).
-__device__ __forceinline__ void advance(Ray& r, Stack& stack) {
+// behind the parked one, or with the stack (and what lies below it) empty
+// (r.node = WIDE_EMPTY).
+template <class S>
+__device__ __forceinline__ void advance(Ray& r, S& stack) {
     int nx = WIDE_EMPTY;
-    while (r.sp > 0) {
+    for (;;) {
         int cand;
-        float te;
-        stack.pop(--r.sp, cand, te);
-        if (te > r.bt) continue;
+        if (r.sp > 0) {
+            float te;
+            stack.pop(--r.sp, cand, te);
+            if (te > r.bt) continue;
+        } else if (!stack.below(r.bt, cand)) {
+            break;
+        }
         if (cand < 0 && r.leaf == WIDE_EMPTY) {
             r.leaf = ~cand;
             continue;
@@ -235,8 +208,6 @@ __device__ __forceinline__ void advance(Ray& r, Stack& stack) {
     }
     r.node = nx;
 }
-
-__device__ __forceinline__ bool ray_done(const Ray& r) { return r.node == WIDE_EMPTY && r.leaf == WIDE_EMPTY; }
 
 // A damaged tree (a cycle) would make a walk endless: a lane whose walk has
 // taken more node and leaf steps than a tree of 2 nt - 1 nodes allows stops,
@@ -251,11 +222,12 @@ __device__ __forceinline__ void step_guard(const A& a, Ray& r) {
 
 // Enter r.node if it is an internal node (A: any argument block with the BVH
 // fields wide, wtex, tri, nt and err).  TEX: the child ids come through the
-// texture pipe (wtex), the box planes through the load pipe.
-template <bool COUNT, bool TEX, class A>
-__device__ __forceinline__ void node_step(const A& a, Ray& r, Stack& stack, uint32_t& visits) {
+// texture pipe (wtex), the box planes through the load pipe.  Returns true
+// when no child is left to enter: the caller advances the ray.
+template <bool COUNT, bool TEX, class A, class S>
+__device__ __forceinline__ bool node_step(const A& a, Ray& r, S& stack, uint32_t& visits) {
     const int node = r.node;
-    if (node < 0) return;   // none, or a leaf waiting behind the parked one
+    if (node < 0) return false;   // none, or a leaf waiting behind the parked one
     r.steps++;
     if (COUNT) visits++;
     // 4-wide node: test the four child boxes, visit the nearest hit child
@@ -321,15 +293,17 @@ __device__ __forceinline__ void node_step(const A& a, Ray& r, Stack& stack, uint
     }
     // a directly entered leaf always waits behind the parked one; only a
     // pop can bring a leaf to park
-    if (first < nh) r.node = first ? val[1] : val[0];
-    else advance(r, stack);
+    if (first >= nh) return true;
+    r.node = first ? val[1] : val[0];
+    return false;
 }
 
-// Test the parked leaf, if any.
-template <bool COUNT, class A>
-__device__ __forceinline__ void leaf_step(const A& a, Ray& r, Stack& stack, uint32_t& visits, uint32_t& tests) {
+// Test the parked leaf, if any.  Returns true when the ray's next node was
+// a leaf waiting behind it, which is parked now: the caller advances the ray.
+template <bool COUNT, class A, class S>
+__device__ __forceinline__ bool leaf_step(const A& a, Ray& r, const S& stack, uint32_t& visits, uint32_t& tests) {
     const int leaf = r.leaf;
-    if (leaf == WIDE_EMPTY) return;
+    if (leaf == WIDE_EMPTY) return false;
     r.steps++;
     if (COUNT) {
         visits++;
@@ -341,7 +315,7 @@ __device__ __forceinline__ void leaf_step(const A& a, Ray& r, Stack& stack, uint
     ldg256(&a.tri[TRI_F4 * leaf + 2], p2, pad);
     float t;
     bool fr;
-    if (ray_tri(r.o, r.d, make_float3(p0.x, p0.y, p0.z), make_float3(p1.x, p1.y, p1.z),
+    if (ray_tri(stack.origin(), stack.direction(), make_float3(p0.x, p0.y, p0.z), make_float3(p1.x, p1.y, p1.z),
                 make_float3(p2.x, p2.y, p2.z), t, fr)) {
         const int idx = __float_as_int(p0.w);
         if (t < r.bt || (t == r.bt && idx < r.bidx)) {
@@ -351,49 +325,9 @@ __device__ __forceinline__ void leaf_step(const A& a, Ray& r, Stack& stack, uint
         }
     }
     r.leaf = WIDE_EMPTY;
-    if (r.node != WIDE_EMPTY && r.node < 0) {
-        r.leaf = ~r.node;
-        advance(r, stack);
-    }
-}
-
-// One warp iteration of the two-phase traversal for every lane (active or
-// not: call it convergently): NODE_STEPS node steps, then the leaf phase if
-// enough lanes wait on a parked leaf.  Two node steps per iteration halve
-// the cost of the phase decision (three ballots) per node visit; measured on
-// the 1M-triangle frame: 1 step 525 ms, 2 steps 497 ms, 3 steps 517 ms,
-// 4 steps 499 ms.  Returns true for a lane whose ray finished.
-constexpr int NODE_STEPS = 2;
-
-// COUNT: visits / tests count this lane's node visits and triangle tests,
-// leaf_slots the leaf rounds the warp ran (one or two per leaf phase).
-template <bool COUNT, bool TEX, class A>
-__device__ __forceinline__ bool warp_step(const A& a, Ray& r, Stack& stack, bool active, int leaf_min,
-                                          uint32_t& visits, uint32_t& tests, uint32_t& leaf_slots) {
-    if (active) {
-#pragma unroll
-        for (int i = 0; i < NODE_STEPS; i++) node_step<COUNT, TEX>(a, r, stack, visits);
-    }
-    const bool parked = active && r.leaf != WIDE_EMPTY;
-    const bool blocked = parked && r.node < 0;             // cannot go on before its leaf
-    const unsigned pm = __ballot_sync(0xFFFFFFFFu, parked);
-    const unsigned bm = __ballot_sync(0xFFFFFFFFu, blocked);
-    const unsigned im = __ballot_sync(0xFFFFFFFFu, active && r.node >= 0);
-    if (pm && (__popc(pm) >= leaf_min || 2 * __popc(bm) >= leaf_min || im == 0)) {
-        if (COUNT) leaf_slots++;
-        if (parked) leaf_step<COUNT>(a, r, stack, visits, tests);
-        // a lane whose next node was a leaf waiting behind the tested one has
-        // parked it now and tests it in a second round of this phase (any
-        // lane: measured slightly faster than waiting for several)
-        const bool again = parked && r.leaf != WIDE_EMPTY;
-        const unsigned am = __ballot_sync(0xFFFFFFFFu, again);
-        if (am) {
-            if (COUNT) leaf_slots++;
-            if (again) leaf_step<COUNT>(a, r, stack, visits, tests);
-        }
-    }
-    if (active) step_guard(a, r);
-    return active && ray_done(r);
+    if (r.node == WIDE_EMPTY || r.node >= 0) return false;
+    r.leaf = ~r.node;
+    return true;
 }
 
 // L2 policy for data that streams past the tracer (the per-slot scratch of
@@ -409,31 +343,6 @@ __device__ __forceinline__ void red_min_stream(uint32_t* p, uint32_t v, uint64_t
 }
 __device__ __forceinline__ void red_add_stream(uint32_t* p, uint32_t v, uint64_t pol) {
     asm volatile("red.relaxed.gpu.global.add.L2::cache_hint.u32 [%0], %1, %2;" ::"l"(p), "r"(v), "l"(pol) : "memory");
-}
-
-// Commit of finished rays that share a texel slot (peers: the lanes of the
-// same slot among those finishing now; lt: lanes below this one).  Vote:
-// the minimum distance bits and the front | back << 16 hit counts.
-// Nearest face: the minimum of (distance bits << 1 | back), ties -> front.
-__device__ __forceinline__ void commit_ray(const Ray& r, bool nearest, unsigned peers, unsigned lt,
-                                           uint32_t* ray_min, uint32_t* ray_cnt) {
-    const bool hit = r.bidx != 0x7FFFFFFF;
-    const uint32_t tbits = __float_as_uint(r.bt) & 0x7FFFFFFFu;
-    if (nearest) {
-        const uint32_t key = hit ? ((tbits << 1) | (r.bfront ? 0u : 1u)) : 0xFFFFFFFFu;
-        const uint32_t mn = __reduce_min_sync(peers, key);
-        if ((peers & lt) == 0 && mn != 0xFFFFFFFFu) red_min_stream(ray_min + r.slot, mn, l2_evict_first());
-        return;
-    }
-    const uint32_t tb = hit ? tbits : 0x7F800000u;
-    const uint32_t cv = hit ? (r.bfront ? 1u : 0x10000u) : 0u;
-    const uint32_t mn = __reduce_min_sync(peers, tb);
-    const uint32_t sum = __reduce_add_sync(peers, cv);
-    if ((peers & lt) == 0) {
-        const uint64_t pol = l2_evict_first();
-        if (mn != 0x7F800000u) red_min_stream(ray_min + r.slot, mn, pol);
-        if (sum) red_add_stream(ray_cnt + r.slot, sum, pol);
-    }
 }
 
 // Eq. 1 for one texel slot after its rays committed: u_t = min(u, r_t) (the
