@@ -16,8 +16,8 @@
 // 512^3 reads a few hundred MB of texels from L2/L1, not HBM.
 //
 // Backward: the march is re-run per point (nothing is stored by the forward
-// pass), its (t_i, h_i) kept in per-thread local memory, then the single
-// penumbra term that produced the visibility (its arg-min step i*) is
+// pass), the t_i of the steps that carry a derivative kept in per-thread local
+// memory, then the single penumbra term that produced the visibility (its arg-min step i*) is
 // differentiated and swept back to step 0 through h_j = S(o + t_j L) and
 // t_{j+1} = t_j + min(h_j, step_max):
 //   dsdf[texel] += hbar_j w_texel(q_j)            (fp32 atomics)
@@ -33,6 +33,8 @@
 
 namespace rtsdf {
 namespace {
+
+constexpr int SHADOW_THREADS = 128;
 
 struct ShadowArgs {
     const float* sdf;
@@ -63,39 +65,38 @@ struct Taps {
     float grad[3];   // d S / d q
 };
 
+// S at offset (dx, dy, dz) from the lower corner of the scene cube.  The fine
+// grid has n = 2 N >= 2 texels per axis, so a cell's upper neighbour is always
+// the next texel, and the eight taps are four rows of two.
 template <bool GRAD>
-__device__ __forceinline__ float sample(const ShadowArgs& a, float qx, float qy, float qz, Taps* tp) {
+__device__ __forceinline__ float sample(const ShadowArgs& a, float dx_, float dy_, float dz_, Taps* tp) {
     const int n = a.n;
-    const float q[3] = {qx, qy, qz};
-    const float b[3] = {a.bx, a.by, a.bz};
-    int i0[3], i1[3];
+    const float d[3] = {dx_, dy_, dz_};
+    const float top = (float)(n - 1);
+    int i0[3];
     float fr[3], dg[3];
 #pragma unroll
     for (int ax = 0; ax < 3; ax++) {
-        float g = __fsub_rn(__fmul_rn(__fsub_rn(q[ax], b[ax]), a.inv_h), 0.5f);
-        dg[ax] = a.inv_h;
-        if (!(g > 0.f)) { g = 0.f; dg[ax] = 0.f; }
-        if (g >= (float)(n - 1)) { g = (float)(n - 1); dg[ax] = 0.f; }
-        int base = (int)floorf(g);
-        base = min(base, n - 2);
-        base = max(base, 0);
-        i0[ax] = base;
-        i1[ax] = n > 1 ? base + 1 : 0;
-        fr[ax] = n > 1 ? g - (float)base : 0.f;
+        const float g0 = __fsub_rn(__fmul_rn(d[ax], a.inv_h), 0.5f);
+        if (GRAD) dg[ax] = g0 > 0.f && !(g0 >= top) ? a.inv_h : 0.f;
+        const float g = fminf(fmaxf(g0, 0.f), top);   // NaN goes to 0
+        i0[ax] = min((int)g, n - 2);
+        fr[ax] = g - (float)i0[ax];
     }
+    const int id0 = i0[0] + n * (i0[1] + n * i0[2]);
+    const float* p = a.sdf + id0;
     float val = 0.f;
     float gx = 0.f, gy = 0.f, gz = 0.f;
 #pragma unroll
     for (int c = 0; c < 8; c++) {
         const int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
-        const int x = dx ? i1[0] : i0[0], y = dy ? i1[1] : i0[1], z = dz ? i1[2] : i0[2];
         const float wx = dx ? fr[0] : 1.f - fr[0], wy = dy ? fr[1] : 1.f - fr[1], wz = dz ? fr[2] : 1.f - fr[2];
-        const int id = x + n * (y + n * z);
-        const float fv = __ldg(a.sdf + id);
+        const int off = dx + n * (dy + n * dz);
+        const float fv = __ldg(p + off);
         const float w = wx * wy * wz;
         val = fmaf(w, fv, val);
         if (GRAD) {
-            tp->idx[c] = id;
+            tp->idx[c] = id0 + off;
             tp->w[c] = w;
             gx = fmaf((dx ? 1.f : -1.f) * wy * wz, fv, gx);
             gy = fmaf(wx * (dy ? 1.f : -1.f) * wz, fv, gy);
@@ -110,11 +111,41 @@ __device__ __forceinline__ float sample(const ShadowArgs& a, float qx, float qy,
     return val;
 }
 
-__device__ __forceinline__ bool inside(const ShadowArgs& a, float x, float y, float z) {
-    return x >= a.bx && x <= a.bx + a.ext && y >= a.by && y <= a.by + a.ext && z >= a.bz && z <= a.bz + a.ext;
+// Whether the penumbra term of a step, k dd / (t - y), may be below res (or
+// anything is not finite).  The march's divisions and root cost a third of a
+// step, and in most steps the term is far above res: it is bounded from below
+// here with an approximate reciprocal and squares (relative errors below 1e-6,
+// taken as 1e-5), and only evaluated where the bound does not settle it, so the
+// result keeps every bit.  r: 1 / (2 ph), approximate.
+__device__ __forceinline__ bool may_lower(float k, float h, float t, float r, float res) {
+    const float h2 = h * h, y = h2 * r;
+    const float a2 = fmaf(-1e-5f, h2, fmaf(-y, y, h2));                // at most h^2 - y^2
+    const float den = fmaf(1e-5f, t + y, t - y);                       // at least t - y
+    const float rd = res * den * 1.00001f, rd2 = rd * rd;
+    // (squares near the underflow are left to the exact form)
+    return !(den < 0.f || ((k * k) * a2 >= rd2 && fminf(a2, rd2) > 1e-30f));
 }
 
-__global__ void __launch_bounds__(256) k_shadow(ShadowArgs a, float* __restrict__ vis) {
+__device__ __forceinline__ float approx_half_rcp(float ph) { return 0.5f * __fdividef(1.f, ph); }
+
+// The bounds of the scene cube as the march tests them: x >= b, by the sign of
+// x - b (exact), and x <= b + ext.
+struct Inside {
+    float hx, hy, hz;
+    __device__ __forceinline__ explicit Inside(const ShadowArgs& a) : hx(a.bx + a.ext), hy(a.by + a.ext), hz(a.bz + a.ext) {}
+    __device__ __forceinline__ bool operator()(float qx, float qy, float qz, float dx, float dy, float dz) const {
+        return dev::fmin3(dx, dy, dz) >= 0.f && qx <= hx && qy <= hy && qz <= hz;
+    }
+};
+
+// Bound by the taps: a step waits for its eight loads (63 % of the L1 pipe's
+// wavefronts, 3.2 a load: neighbouring marches drift apart) and issues 118
+// instructions (73 % of the issue slots).  1920 x 1080 points, 256^3 grid, 64
+// steps: 350 us with every penumbra term evaluated and per-axis clamps, 261 us
+// now; blocks of 128 instead of 256 take 2 % off (10 % for 427 x 240 points).
+// Tried, no change: floor without the conversion unit, 32 registers (64 warps
+// an SM), two steps unrolled.
+__global__ void __launch_bounds__(SHADOW_THREADS) k_shadow(ShadowArgs a, float* __restrict__ vis) {
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= a.npix) return;
     const float two_eps = 2.f * a.eps;
@@ -127,64 +158,87 @@ __global__ void __launch_bounds__(256) k_shadow(ShadowArgs a, float* __restrict_
         oy = fmaf(sh, a.Ly, oy);
         oz = fmaf(sh, a.Lz, oz);
     }
+    const Inside inside(a);
     float t = 0.f, res = 1.f, ph = 1e20f;
     for (int s = 0; s < a.steps; s++) {
         const float qx = fmaf(t, a.Lx, ox), qy = fmaf(t, a.Ly, oy), qz = fmaf(t, a.Lz, oz);
-        if (!inside(a, qx, qy, qz)) break;
-        const float h = sample<false>(a, qx, qy, qz, nullptr);
+        const float dx = __fsub_rn(qx, a.bx), dy = __fsub_rn(qy, a.by), dz = __fsub_rn(qz, a.bz);
+        if (!inside(qx, qy, qz, dx, dy, dz)) break;
+        const float h = sample<false>(a, dx, dy, dz, nullptr);
         if (h < a.eps) {
             res = 0.f;
             break;
         }
-        const float y = h * h / (2.f * ph);
-        const float dd = sqrtf(fmaxf(h * h - y * y, 0.f));
-        if (t - y > 0.f) res = fminf(res, a.k * dd / (t - y));
+        if (may_lower(a.k, h, t, approx_half_rcp(ph), res)) {
+            const float y = h * h / (2.f * ph);
+            const float dd = sqrtf(fmaxf(h * h - y * y, 0.f));
+            if (t - y > 0.f) res = fminf(res, a.k * dd / (t - y));
+        }
         ph = h;
         t += fminf(h, a.smax);
     }
     vis[i] = fminf(fmaxf(res, 0.f), 1.f);
 }
 
-__global__ void __launch_bounds__(128) k_shadow_bwd(ShadowArgs a, const float* __restrict__ dvis,
+// Bound by the latency of the re-marched steps (49 % of the issue slots, 52 %
+// of the warps): 42 registers let 12 blocks of 128 reside.  1024^2 points,
+// 512^3 grid: 439 us with (t, h) of every step in local memory and every step
+// swept back, 210 us now (221 us at 56 registers).
+__global__ void __launch_bounds__(128, 12) k_shadow_bwd(ShadowArgs a, const float* __restrict__ dvis,
                                                    float* __restrict__ dsdf, float* __restrict__ dlight,
                                                    float inv_norm) {
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     float lbx = 0.f, lby = 0.f, lbz = 0.f;
     if (i < a.npix && dvis[i] != 0.f) {
-        float ts[MAX_SHADOW_STEPS], hs[MAX_SHADOW_STEPS];
+        // The sweep back visits step j < s - 1 only through t_{j+1} = t_j +
+        // min(h_j, step_max), so only steps with h_j < step_max matter to it:
+        // their t_j are kept (and, with the sign set, those of steps whose h_j
+        // is not finite, which pass on what 0 times their taps gives).
+        float ts[MAX_SHADOW_STEPS];
         const float two_eps = 2.f * a.eps;
         const float ox = fmaf(a.nrm[3 * i], two_eps, a.pos[3 * i]);
         const float oy = fmaf(a.nrm[3 * i + 1], two_eps, a.pos[3 * i + 1]);
         const float oz = fmaf(a.nrm[3 * i + 2], two_eps, a.pos[3 * i + 2]);
-        float t = 0.f, res = 1.f, ph = 1e20f;
-        int am = -1;
+        const Inside inside(a);
+        float t = 0.f, res = 1.f, ph = 1e20f, tprev = 0.f;
+        int kept = 0, kept_prev = 0;           // kept steps before this one, before the previous one
+        // the arg-min step: index, t, h, the previous step's h and t, kept steps before that
+        int am = -1, am_kept = 0;
+        float am_t = 0.f, am_h = 0.f, am_p = 0.f, am_tp = 0.f;
         bool term = false;
         for (int s = 0; s < a.steps; s++) {
             const float qx = fmaf(t, a.Lx, ox), qy = fmaf(t, a.Ly, oy), qz = fmaf(t, a.Lz, oz);
-            if (!inside(a, qx, qy, qz)) break;
-            const float h = sample<false>(a, qx, qy, qz, nullptr);
-            ts[s] = t;
-            hs[s] = h;
+            const float dx = __fsub_rn(qx, a.bx), dy = __fsub_rn(qy, a.by), dz = __fsub_rn(qz, a.bz);
+            if (!inside(qx, qy, qz, dx, dy, dz)) break;
+            const float h = sample<false>(a, dx, dy, dz, nullptr);
             if (h < a.eps) {
                 term = true;
                 break;
             }
-            const float y = h * h / (2.f * ph);
-            const float dd = sqrtf(fmaxf(h * h - y * y, 0.f));
-            if (t - y > 0.f) {
-                const float g = a.k * dd / (t - y);
-                if (g < res) {
-                    res = g;
-                    am = s;
+            if (may_lower(a.k, h, t, approx_half_rcp(ph), res)) {
+                const float y = h * h / (2.f * ph);
+                const float dd = sqrtf(fmaxf(h * h - y * y, 0.f));
+                if (t - y > 0.f) {
+                    const float g = a.k * dd / (t - y);
+                    if (g < res) {
+                        res = g;
+                        am = s;
+                        am_kept = kept_prev;
+                        am_t = t;
+                        am_h = h;
+                        am_p = ph;
+                        am_tp = tprev;
+                    }
                 }
             }
+            kept_prev = kept;
+            if (!(h >= a.smax && h < CUDART_INF_F)) ts[kept++] = h < a.smax ? t : -t;
             ph = h;
+            tprev = t;
             t += fminf(h, a.smax);
         }
         if (!term && am >= 0) {
-            const int s = am;
-            const float h = hs[s], tt = ts[s];
-            const float p = s > 0 ? hs[s - 1] : 1e20f;
+            const float h = am_h, tt = am_t, p = am_p;
             const float y = h * h / (2.f * p);
             const float a2 = h * h - y * y;
             if (a2 > 0.f) {
@@ -194,12 +248,15 @@ __global__ void __launch_bounds__(128) k_shadow_bwd(ShadowArgs a, const float* _
                 const float gb = dvis[i];
                 const float kd = a.k / den, kd2 = a.k * dd / (den * den);
                 float hbar = gb * (kd * ddd_dh + kd2 * dy_dh);
-                const float pbar = s > 0 ? gb * (kd * ddd_dp + kd2 * dy_dp) : 0.f;
+                const float pbar = am > 0 ? gb * (kd * ddd_dp + kd2 * dy_dp) : 0.f;
                 float tbar = -gb * kd2;
-                for (int j = s; j >= 0; j--) {
-                    const float tj = ts[j];
+                float tj = tt;
+                // the arg-min step, the one before it, then the kept ones
+                for (int j = am_kept + 1; j >= -1; j--) {
                     Taps tp;
-                    sample<true>(a, fmaf(tj, a.Lx, ox), fmaf(tj, a.Ly, oy), fmaf(tj, a.Lz, oz), &tp);
+                    const float dx = __fsub_rn(fmaf(tj, a.Lx, ox), a.bx), dy = __fsub_rn(fmaf(tj, a.Ly, oy), a.by),
+                                dz = __fsub_rn(fmaf(tj, a.Lz, oz), a.bz);
+                    sample<true>(a, dx, dy, dz, &tp);
 #pragma unroll
                     for (int c = 0; c < 8; c++) atomicAdd(dsdf + tp.idx[c], hbar * tp.w[c]);
                     const float qbx = hbar * tp.grad[0], qby = hbar * tp.grad[1], qbz = hbar * tp.grad[2];
@@ -207,9 +264,17 @@ __global__ void __launch_bounds__(128) k_shadow_bwd(ShadowArgs a, const float* _
                     lbx = fmaf(qbx, tj, lbx);
                     lby = fmaf(qby, tj, lby);
                     lbz = fmaf(qbz, tj, lbz);
-                    if (j == 0) break;
-                    hbar = (j - 1 == s - 1) ? pbar : 0.f;
-                    if (hs[j - 1] < a.smax) hbar += tbar;
+                    if (j == am_kept + 1) {
+                        if (am == 0) break;
+                        tj = am_tp;
+                        hbar = pbar;
+                        if (p < a.smax) hbar += tbar;
+                    } else {
+                        if (j == 0) break;
+                        const float e = ts[j - 1];
+                        tj = fabsf(e);
+                        hbar = signbit(e) ? 0.f : tbar;
+                    }
                 }
             }
         }
@@ -360,7 +425,7 @@ cudaError_t launch_shadow(rtsdf_ctx* c, const float* sdf, const float* pos, cons
     ShadowArgs a = make_args(c, sdf, pos, nrm, npix, L, k, steps, smax, eps);
     a.jitter = jitter;
     a.frame = (uint32_t)frame;
-    RTSDF_LAUNCH(c, k_shadow, (unsigned)((npix + 255) / 256), 256, 0, a, vis);
+    RTSDF_LAUNCH(c, k_shadow, (unsigned)((npix + SHADOW_THREADS - 1) / SHADOW_THREADS), SHADOW_THREADS, 0, a, vis);
     return cudaGetLastError();
 }
 
