@@ -96,10 +96,9 @@ void free_all(rtsdf_ctx* c) {
     dfree(c->bin_count); dfree(c->bin_start); dfree(c->bin_cursor); dfree(c->bin_items); dfree(c->bin_overflow);
     drop_texture(c->bvh.wtex);
     dfree(c->bvh.nodes); dfree(c->bvh.wide); dfree(c->bvh.nbox); dfree(c->bvh.lbox); dfree(c->bvh.tri); dfree(c->bvh.leaf_tri); dfree(c->bvh.leaf_parent); dfree(c->bvh.flags);
-    dfree(c->bvh.col_fb); dfree(c->bvh.col_fslot); dfree(c->bvh.col_nb); dfree(c->bvh.col_nslot);
-    dfree(c->bvh.col_kids); dfree(c->bvh.col_nint); dfree(c->bvh.col_total);
+    dfree(c->bvh.col_from); dfree(c->bvh.col_lev);
     dfree(c->bvh.root); dfree(c->bvh.mk0); dfree(c->bvh.mk1); dfree(c->bvh.mv0); dfree(c->bvh.mv1);
-    dfree(c->bvh.hist); dfree(c->bvh.d_depth); dfree(c->bvh.sah);
+    dfree(c->bvh.hist); dfree(c->bvh.sah);
     dfree(c->bvh.top_child); dfree(c->bvh.top_ids); dfree(c->bvh.top_box); dfree(c->bvh.top_scratch);
     dfree(c->bvh.obj_count);
     dfree(c->d_err);

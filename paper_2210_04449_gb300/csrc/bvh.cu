@@ -15,6 +15,7 @@
 #include <math_constants.h>
 #include <string.h>
 
+#include <algorithm>
 #include <utility>
 #include <vector>
 
@@ -293,27 +294,6 @@ __global__ void k_top_up(const int32_t* __restrict__ child, int32_t n, const int
     climb(nodes, flags, nbox, c, c >= 0 ? nodes[c].d.z : leaf_parent[~c], lo, hi, nt);
 }
 
-// Child boxes of the 4-wide nodes from the (re)fitted binary boxes.
-__global__ void k_wide_boxes(WNode* __restrict__ wide, int64_t n_wide, const float* __restrict__ nbox,
-                             const float* __restrict__ lbox) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n_wide * 4) return;
-    const int64_t w = i >> 2;
-    const int k = (int)(i & 3);
-    const int src = (&wide[w].src.x)[k];
-    float b[6] = {CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
-    if (src != WIDE_EMPTY) {
-        const float* p = src >= 0 ? nbox + 6 * (int64_t)src : lbox + 6 * (int64_t)(~src);
-        for (int a = 0; a < 6; a++) b[a] = p[a];
-    }
-    (&wide[w].lox.x)[k] = b[0];
-    (&wide[w].hix.x)[k] = b[3];
-    (&wide[w].loy.x)[k] = b[1];
-    (&wide[w].hiy.x)[k] = b[4];
-    (&wide[w].loz.x)[k] = b[2];
-    (&wide[w].hiz.x)[k] = b[5];
-}
-
 __global__ void k_depth(const int32_t* __restrict__ leaf_parent, const BNode* __restrict__ nodes, int64_t n,
                         int32_t* depth) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -424,14 +404,17 @@ __global__ void k_transform(float* __restrict__ verts, const int32_t* __restrict
 }  // namespace
 
 // Collapse the binary tree into 4-wide nodes, on the device, one tree level
-// at a time: every frontier node (a binary node that roots a wide node)
+// at a time: every node of a level (a binary node that roots a wide node)
 // starts from its two children and replaces the internal child of largest
 // surface area by its two children until four are collected (or only
 // leaves remain); each internal child roots a wide node of the next level.
-// Slots are handed out in frontier order by an exclusive scan of the
-// internal-child counts, so the layout is breadth-first with the children
-// of a node contiguous.
+// The layout is breadth-first with the children of a node contiguous; within
+// a level, slots are handed out as the warps come.  A level's size stays on
+// the device, so that no level waits for the host.
 namespace {
+
+constexpr int COL_BATCH = 30;   // levels enqueued without a look from the host
+constexpr int COL_WORDS = 2 * (COL_BATCH + 1) + 1;   // the levels, then the binary tree's depth
 
 __device__ __forceinline__ float half_area(const float* __restrict__ nbox, int node) {
     const float* p = nbox + 6 * (int64_t)node;
@@ -439,93 +422,121 @@ __device__ __forceinline__ float half_area(const float* __restrict__ nbox, int n
     return dx * dy + dy * dz + dz * dx;
 }
 
-__global__ void k_collapse_expand(const int32_t* __restrict__ fb, int32_t cnt, const BNode* __restrict__ bn,
-                                  const float* __restrict__ nbox, int4* __restrict__ kids,
-                                  uint32_t* __restrict__ nint) {
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= cnt) return;
-    const int4 d = bn[fb[i]].d;
-    int kid[4] = {d.x, d.y, WIDE_EMPTY, WIDE_EMPTY};
-    int nk = 2;
-    while (nk < 4) {
-        int best = -1;
-        float ba = -1.f;
-        for (int k = 0; k < nk; k++)
-            if (kid[k] >= 0) {
-                const float ar = half_area(nbox, kid[k]);
-                if (ar > ba) {
-                    ba = ar;
-                    best = k;
-                }
-            }
-        if (best < 0) break;
-        const int4 od = bn[kid[best]].d;
-        kid[best] = od.x;
-        kid[nk++] = od.y;
+// The wide node's child boxes from the (re)fitted binary boxes.
+__device__ __forceinline__ void wide_box(WNode* w, int k, int src, const float* __restrict__ nbox,
+                                         const float* __restrict__ lbox) {
+    float b[6] = {CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
+    if (src != WIDE_EMPTY) {
+        const float* p = src >= 0 ? nbox + 6 * (int64_t)src : lbox + 6 * (int64_t)(~src);
+        for (int a = 0; a < 6; a++) b[a] = p[a];
     }
-    kids[i] = make_int4(kid[0], kid[1], kid[2], kid[3]);
-    nint[i] = (kid[0] >= 0) + (kid[1] >= 0) + (kid[2] >= 0) + (kid[3] >= 0);
+    (&w->lox.x)[k] = b[0];
+    (&w->hix.x)[k] = b[3];
+    (&w->loy.x)[k] = b[1];
+    (&w->hiy.x)[k] = b[4];
+    (&w->loz.x)[k] = b[2];
+    (&w->hiz.x)[k] = b[5];
 }
 
-__global__ void k_collapse_write(const int32_t* __restrict__ fslot, int32_t cnt, const int4* __restrict__ kids,
-                                 const uint32_t* __restrict__ off, int32_t base, int64_t cap, WNode* __restrict__ wide,
-                                 int32_t* __restrict__ nb, int32_t* __restrict__ nslot, int32_t* __restrict__ total) {
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= cnt) return;
-    const int4 kv = kids[i];
-    const int kid[4] = {kv.x, kv.y, kv.z, kv.w};
-    const uint32_t o = off[i];
-    uint32_t j = 0;
-    int child[4], src[4];
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-        src[k] = kid[k];
-        if (kid[k] == WIDE_EMPTY) {
-            child[k] = WIDE_EMPTY;
-        } else if (kid[k] >= 0) {
-            const int32_t slot = base + (int32_t)(o + j);
-            if ((int64_t)slot >= cap) {   // only a damaged tree gets here: drop the child, the host stops
-                child[k] = src[k] = WIDE_EMPTY;
-                j++;
-                continue;
+__global__ void k_wide_boxes(WNode* __restrict__ wide, int64_t n_wide, const float* __restrict__ nbox,
+                             const float* __restrict__ lbox) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n_wide * 4) return;
+    const int k = (int)(i & 3);
+    wide_box(wide + (i >> 2), k, (&wide[i >> 2].src.x)[k], nbox, lbox);
+}
+
+// Level l: the nodes of slots [lev[2 l], + lev[2 l + 1]), whose binary roots
+// are in `from`.  Writes lev[2 l + 2] (the next level's first slot) and counts
+// its nodes in lev[2 l + 3].
+__global__ void __launch_bounds__(128) k_collapse_level(int32_t* lev, int l, int64_t cap,
+                                                        const BNode* __restrict__ bn,
+                                                        const float* __restrict__ nbox,
+                                                        const float* __restrict__ lbox, int32_t* from,
+                                                        WNode* __restrict__ wide) {
+    const int32_t first = lev[2 * l];
+    const int32_t cnt = min(lev[2 * l + 1], max((int32_t)(cap - first), 0));   // (all of it, unless the tree is damaged)
+    const int32_t next = first + cnt;
+    if (blockIdx.x == 0 && threadIdx.x == 0) lev[2 * l + 2] = next;
+    const int lane = (int)(threadIdx.x & 31);
+    for (int32_t w0 = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x) - lane; w0 < cnt;
+         w0 += (int32_t)(gridDim.x * blockDim.x)) {
+        const int32_t i = w0 + lane;
+        int kid[4] = {WIDE_EMPTY, WIDE_EMPTY, WIDE_EMPTY, WIDE_EMPTY};
+        int nint = 0;
+        if (i < cnt) {
+            const int4 d = bn[from[first + i]].d;
+            kid[0] = d.x;
+            kid[1] = d.y;
+            float area[4];
+            area[0] = kid[0] >= 0 ? half_area(nbox, kid[0]) : -1.f;
+            area[1] = kid[1] >= 0 ? half_area(nbox, kid[1]) : -1.f;
+            for (int nk = 2; nk < 4; nk++) {
+                int best = -1;
+                float ba = -1.f;
+                for (int k = 0; k < nk; k++)
+                    if (kid[k] >= 0 && area[k] > ba) {
+                        ba = area[k];
+                        best = k;
+                    }
+                if (best < 0) break;
+                const int4 od = bn[kid[best]].d;
+                kid[best] = od.x;
+                kid[nk] = od.y;
+                area[best] = od.x >= 0 ? half_area(nbox, od.x) : -1.f;
+                area[nk] = od.y >= 0 ? half_area(nbox, od.y) : -1.f;
             }
-            child[k] = slot;
-            nb[o + j] = kid[k];
-            nslot[o + j] = slot;
-            j++;
-        } else {
-            child[k] = kid[k];   // ~leaf
+            nint = (kid[0] >= 0) + (kid[1] >= 0) + (kid[2] >= 0) + (kid[3] >= 0);
         }
+        int sum = nint;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xFFFFFFFFu, sum, o);
+            if (lane >= o) sum += u;
+        }
+        int at = 0;
+        if (lane == 31 && sum) at = atomicAdd(lev + 2 * l + 3, sum);
+        at = __shfl_sync(0xFFFFFFFFu, at, 31) + next + sum - nint;
+        if (i >= cnt) continue;
+        WNode* w = wide + first + i;
+        int child[4];
+        for (int k = 0; k < 4; k++) {
+            child[k] = kid[k];   // ~leaf, or none
+            if (kid[k] >= 0) {
+                if ((int64_t)at >= cap) {   // only a damaged tree gets here: drop the child, the host stops
+                    child[k] = kid[k] = WIDE_EMPTY;
+                } else {
+                    child[k] = at;
+                    from[at] = kid[k];
+                }
+                at++;
+            }
+            wide_box(w, k, kid[k], nbox, lbox);
+        }
+        w->child = make_int4(child[0], child[1], child[2], child[3]);
+        w->src = make_int4(kid[0], kid[1], kid[2], kid[3]);
     }
-    const int32_t w = fslot[i];
-    wide[w].child = make_int4(child[0], child[1], child[2], child[3]);
-    wide[w].src = make_int4(src[0], src[1], src[2], src[3]);
-    if (i == cnt - 1) *total = (int32_t)(o + j);
 }
 
-__global__ void k_collapse_root(const int32_t* root, int32_t* fb, int32_t* fslot) {
-    fb[0] = *root;
-    fslot[0] = 0;
+__global__ void k_collapse_root(const int32_t* root, int32_t* from, int32_t* lev) {
+    if (threadIdx.x == 0) from[0] = *root;
+    if (threadIdx.x < COL_WORDS) lev[threadIdx.x] = threadIdx.x == 1 ? 1 : 0;   // (64 threads)
 }
 
 }  // namespace
 
-static cudaError_t collapse_wide(rtsdf_ctx* c) {
+// depth: where the binary tree's depth goes (nullptr: not wanted).
+static cudaError_t collapse_wide(rtsdf_ctx* c, int* depth) {
     Bvh& b = c->bvh;
     const int64_t n = b.nt;                  // n >= 2: n - 1 binary internal nodes
     const int64_t cap = n - 1;               // every wide node roots a distinct binary node
     cudaError_t e;
     if (b.col_cap < cap) {
-        cudaFree(b.col_fb); cudaFree(b.col_fslot); cudaFree(b.col_nb); cudaFree(b.col_nslot);
-        cudaFree(b.col_kids); cudaFree(b.col_nint); cudaFree(b.col_total);
-        b.col_fb = b.col_fslot = b.col_nb = b.col_nslot = b.col_total = nullptr;
-        b.col_kids = nullptr;
-        b.col_nint = nullptr;
+        cudaFree(b.col_from); cudaFree(b.col_lev);
+        b.col_from = b.col_lev = nullptr;
         b.col_cap = 0;
-        if ((e = cudaMalloc(&b.col_fb, sizeof(int32_t) * cap)) || (e = cudaMalloc(&b.col_fslot, sizeof(int32_t) * cap)) ||
-            (e = cudaMalloc(&b.col_nb, sizeof(int32_t) * cap)) || (e = cudaMalloc(&b.col_nslot, sizeof(int32_t) * cap)) ||
-            (e = cudaMalloc(&b.col_kids, sizeof(int4) * cap)) || (e = cudaMalloc(&b.col_nint, sizeof(uint32_t) * cap)) ||
-            (e = cudaMalloc(&b.col_total, sizeof(int32_t))))
+        if ((e = cudaMalloc(&b.col_from, sizeof(int32_t) * cap)) ||
+            (e = cudaMalloc(&b.col_lev, sizeof(int32_t) * COL_WORDS)))
             return e;
         b.col_cap = cap;
     }
@@ -540,28 +551,43 @@ static cudaError_t collapse_wide(rtsdf_ctx* c) {
         b.wide_cap = cap;
         b.wtex = make_int4_texture(b.wide, (sizeof(WNode) / 16) * (size_t)cap, c->device);
     }
-    int32_t *fb = b.col_fb, *fs = b.col_fslot, *nb = b.col_nb, *ns = b.col_nslot;
-    RTSDF_LAUNCH(c, k_collapse_root, 1, 1, 0, b.root, fb, fs);
-    int32_t base = 1, cnt = 1;
-    while (cnt > 0) {
-        const unsigned g = (unsigned)((cnt + 255) / 256);
-        RTSDF_LAUNCH(c, k_collapse_expand, g, 256, 0, fb, cnt, b.nodes, b.nbox, b.col_kids, b.col_nint);
-        RTSDF_LAUNCH(c, k_scan, 1, 1024, 0, b.col_nint, (int64_t)cnt);
-        RTSDF_LAUNCH(c, k_collapse_write, g, 256, 0, fs, cnt, b.col_kids, b.col_nint, base, cap, b.wide, nb, ns,
-                     b.col_total);
-        int32_t next = 0;
-        e = cudaMemcpyAsync(&next, b.col_total, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        if (e != cudaSuccess) return e;
-        if (next < 0 || (int64_t)base + next > cap) return cudaErrorUnknown;   // only a damaged tree gets here
-        base += next;
-        cnt = next;
-        int32_t* t = fb; fb = nb; nb = t;
-        t = fs; fs = ns; ns = t;
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+    const int64_t most = 16 * (int64_t)(sms > 0 ? sms : 132);
+    RTSDF_LAUNCH(c, k_collapse_root, 1, 64, 0, b.root, b.col_from, b.col_lev);
+    if (depth)
+        RTSDF_LAUNCH(c, k_depth, (unsigned)((n + 255) / 256), 256, 0, b.leaf_parent, b.nodes, n,
+                     b.col_lev + COL_WORDS - 1);
+    // a batch of levels for a tree whose leaves are a few levels apart; a
+    // deeper one takes more batches
+    int levels = 6;
+    while (levels < COL_BATCH && (1ll << (2 * (levels - 6))) < n) levels++;
+    int64_t nodes = 1;
+    for (int batch = 0;; batch++) {
+        if (batch >= (1 << 24)) return cudaErrorUnknown;
+        for (int l = 0; l < levels; l++) {
+            RTSDF_LAUNCH(c, k_collapse_level, (unsigned)std::min<int64_t>((std::min(nodes, cap) + 127) / 128, most), 128,
+                         0, b.col_lev, l, cap, b.nodes, b.nbox, b.lbox, b.col_from, b.wide);
+            if (nodes < cap) nodes *= 4;
+        }
+        int32_t h[COL_WORDS];
+        if ((e = cudaGetLastError())) return e;
+        if ((e = cudaMemcpyAsync(h, b.col_lev, sizeof(h), cudaMemcpyDeviceToHost, c->stream))) return e;
+        if ((e = cudaStreamSynchronize(c->stream))) return e;
+        const int64_t done = h[2 * levels], left = h[2 * levels + 1];
+        if (left < 0 || done + left > cap) return cudaErrorUnknown;   // only a damaged tree gets here
+        if (depth && batch == 0) *depth = h[COL_WORDS - 1];
+        if (left == 0) {
+            b.n_wide = done;
+            return cudaSuccess;
+        }
+        int32_t r[COL_WORDS] = {0};
+        r[0] = (int32_t)done;
+        r[1] = (int32_t)left;
+        if ((e = cudaMemcpyAsync(b.col_lev, r, sizeof(r), cudaMemcpyHostToDevice, c->stream))) return e;
+        if ((e = cudaStreamSynchronize(c->stream))) return e;   // r is a local buffer
+        levels = 8;
     }
-    b.n_wide = base;
-    RTSDF_LAUNCH(c, k_wide_boxes, (unsigned)((4 * b.n_wide + 255) / 256), 256, 0, b.wide, b.n_wide, b.nbox, b.lbox);
-    return cudaGetLastError();
 }
 
 // Two-level topology: triangles sorted by object (stable), one SAH subtree
@@ -690,7 +716,6 @@ cudaError_t launch_bvh_build(rtsdf_ctx* c) {
         b.cap_nt = n;
     }
     if (!b.root && (e = cudaMalloc(&b.root, sizeof(int32_t)))) return e;
-    if (!b.d_depth && (e = cudaMalloc(&b.d_depth, sizeof(int32_t)))) return e;
     if (sah && b.sah_bytes < sah_scratch_bytes(n)) {
         cudaFree(b.sah);
         b.sah = nullptr;
@@ -731,17 +756,10 @@ cudaError_t launch_bvh_build(rtsdf_ctx* c) {
     RTSDF_LAUNCH(c, k_leaves_up, g, 256, 0, c->verts, c->tris, order, n, b.tri, b.leaf_tri, b.leaf_parent, b.nodes,
                  b.flags, pad, b.lbox, b.nbox);
     if (two && (e = build_top(c))) return e;
-    if ((e = cudaMemsetAsync(b.d_depth, 0, sizeof(int32_t), c->stream))) return e;
-    RTSDF_LAUNCH(c, k_depth, g, 256, 0, b.leaf_parent, b.nodes, n, b.d_depth);
-    if (n > 1) {
-        if ((e = cudaGetLastError())) return e;
-        if ((e = collapse_wide(c))) return e;
-    }
     if ((e = cudaGetLastError())) return e;
-    int32_t hd = 0;
-    if ((e = cudaMemcpyAsync(&hd, b.d_depth, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream))) return e;
-    if ((e = cudaStreamSynchronize(c->stream))) return e;
-    b.depth = hd;
+    b.depth = 1;
+    if (n > 1 && (e = collapse_wide(c, &b.depth))) return e;   // waits for the stream
+    if (n == 1 && (e = cudaStreamSynchronize(c->stream))) return e;
     b.built = true;
     return cudaSuccess;
 }
@@ -760,7 +778,7 @@ cudaError_t launch_bvh_refit(rtsdf_ctx* c) {
         RTSDF_LAUNCH(c, k_leaves_up, (unsigned)((n + 255) / 256), 256, 0, c->verts, c->tris, b.leaf_tri, n, b.tri,
                      b.leaf_tri, b.leaf_parent, b.nodes, b.flags, pad, b.lbox, b.nbox);
         if ((e = build_top(c))) return e;
-        return collapse_wide(c);
+        return collapse_wide(c, nullptr);
     }
     RTSDF_LAUNCH(c, k_leaves_up, (unsigned)((n + 255) / 256), 256, 0, c->verts, c->tris, b.leaf_tri, n, b.tri,
                  b.leaf_tri, b.leaf_parent, b.nodes, b.flags, pad, b.lbox, b.nbox);

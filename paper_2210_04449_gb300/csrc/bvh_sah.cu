@@ -11,13 +11,14 @@
 // belongs to exactly one node), so the tree has the layout of the Morton
 // tree: [nt - 1] nodes, [nt] leaves, any node may be the root.
 //
-// Three tiers by range size m:
-//  * m > SAH_CH: level-synchronous over chunks of SAH_CH positions.
+// Three tiers by range size m (blk: 256, or 1024 for large meshes):
+//  * m > blk: level-synchronous over chunks of SAH_CH positions, the levels'
+//    sizes kept on the device so that no level waits for the host.
 //    k_sah_bin bins a chunk in shared memory and merges into the range's
 //    bins with global atomics (and keeps the chunk's histogram);
 //    k_sah_split (a warp per range) picks the split and every chunk's output
 //    offset; k_sah_partition scatters stably into the other order buffer.
-//  * 32 < m <= SAH_CH: one block per range (k_sah_block), boxes in shared
+//  * 32 < m <= blk: one block per range (k_sah_block), boxes in shared
 //    memory, the same binned split down to ranges of 32;
 //  * 2 <= m <= 32: one warp per range, the exact heuristic over every split
 //    of the centroids sorted along each axis (bitonic sort in registers).
@@ -46,12 +47,27 @@ constexpr int SAH_WARPS = SAH_THREADS / 32;
 constexpr int WARP_MAX = 32;                  // largest range of the exact warp build
 constexpr int BLK_STACK = 48;                 // disjoint ranges > 32 in 1024: at most 31
 constexpr int WLIST_CAP = SAH_CH / 2;         // disjoint ranges >= 2 in 1024
-constexpr int WSTACK = 32;                    // disjoint ranges >= 2 in 32: at most 16
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
 static_assert(SAH_ITEMS * SAH_THREADS == SAH_CH, "one chunk per block pass");
 
-// big range (m > SAH_CH) of one level
+// Largest range of the block tier.  A block splits its range one node after
+// another, so a small mesh, whose few ranges leave most SMs idle, is split
+// further by the levels (each of which costs three launches).  Whole build
+// with 256 against 1024: 2.2k triangles 403 / 505 us, 104k 908 / 1270 us, 1M
+// 2587 / 2389 us (300k: 1103 / 1166 us).
+constexpr int SAH_BLK_SMALL = 256;
+constexpr int64_t SAH_SMALL_MESH = 400000;
+__host__ __device__ constexpr int blk_of(int64_t n) { return n <= SAH_SMALL_MESH ? SAH_BLK_SMALL : SAH_CH; }
+
+// Device-side counters of a build: block ranges listed, a capacity guard that
+// fired, block ranges taken, then (tasks, chunks) of each level of a batch.
+constexpr int CT_BLOCKS = 0, CT_BAD = 1, CT_TAKEN = 2, CT_LEVELS = 4;
+constexpr int LEVEL_BATCH = 28;               // levels enqueued without a look from the host, at most
+constexpr int CT_WORDS = CT_LEVELS + 2 * (LEVEL_BATCH + 1);
+static_assert(CT_WORDS <= 64, "counters fit 256 bytes");
+
+// big range (m > blk_of(n)) of one level
 struct SahTask {
     int32_t b, e, parent, side;
     int32_t buf, chunk0, nchunk, axis;   // buf: order buffer holding the range
@@ -243,7 +259,8 @@ __device__ __forceinline__ int block_excl(int v, int* s_warp, int& total) {
 
 // ------------------------------------------------------------- setup
 
-__global__ void k_sah_root(SahTask* t, int4* chunks, uint32_t* bins, SahRange* blist, int32_t n) {
+__global__ void k_sah_root(SahTask* t, int4* chunks, uint32_t* bins, SahRange* blist, int32_t n, int blk,
+                           int32_t* counters) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int nch = (n + SAH_CH - 1) / SAH_CH;
     if (i == 0) {
@@ -257,9 +274,12 @@ __global__ void k_sah_root(SahTask* t, int4* chunks, uint32_t* bins, SahRange* b
         }
         r.pad[0] = r.pad[1] = 0;
         t[0] = r;
-        if (n <= SAH_CH) blist[0] = SahRange{0, n, -1, 0};
+        if (n <= blk) blist[0] = SahRange{0, n, -1, 0};
+        counters[CT_BLOCKS] = n <= blk ? 1 : 0;
+        counters[CT_LEVELS] = n <= blk ? 0 : 1;
+        counters[CT_LEVELS + 1] = n <= blk ? 0 : nch;
     }
-    if (n > SAH_CH) {
+    if (n > blk) {
         if (i < nch) chunks[i] = make_int4(0, i * SAH_CH, min(SAH_CH, n - i * SAH_CH), 0);
         if (i < SAH_BIN_WORDS) bins[i] = bin_init(i);
     }
@@ -368,8 +388,10 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_bin(const int4* __restrict_
                                                          const int32_t* __restrict__ ord0,
                                                          const int32_t* __restrict__ ord1,
                                                          const float4* __restrict__ pbox, uint32_t* bins,
-                                                         uint32_t* __restrict__ hist) {
+                                                         uint32_t* __restrict__ hist,
+                                                         const int32_t* counters, int lev) {
     __shared__ uint32_t sb[SAH_BIN_WORDS];
+    if ((int)blockIdx.x >= counters[lev + 1] || counters[CT_BAD]) return;
     const int4 ch = chunks[blockIdx.x];        // (task, start, length)
     const SahTask& T = tasks[ch.x];
     for (int i = threadIdx.x; i < SAH_BIN_WORDS; i += SAH_THREADS) sb[i] = bin_init(i);
@@ -412,17 +434,16 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_bin(const int4* __restrict_
 
 // One warp per big range: split choice, node links, chunk output offsets,
 // and the children (leaf, block range or next-level big range).
-// counters: [0] next tasks, [1] next chunks, [2] block ranges, [3] overflow.
-__global__ void __launch_bounds__(SAH_THREADS) k_sah_split(SahTask* tasks, int32_t ntask, const uint32_t* bins,
+__global__ void __launch_bounds__(SAH_THREADS) k_sah_split(SahTask* tasks, int lev, const uint32_t* bins,
                                                            const uint32_t* __restrict__ hist,
                                                            const int4* __restrict__ chunks,
                                                            int32_t* __restrict__ left_off, Links L, SahTask* next,
                                                            int4* next_chunks, uint32_t* next_bins, SahRange* blist,
                                                            int32_t* counters, int32_t cap_task, int32_t cap_chunk,
-                                                           int32_t cap_blist) {
+                                                           int32_t cap_blist, int blk) {
     const int w = (int)((blockIdx.x * (unsigned)SAH_THREADS + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
-    if (w >= ntask) return;                    // warp-uniform
+    if (w >= counters[lev] || counters[CT_BAD]) return;   // warp-uniform
     SahTask& T = tasks[w];
     const int b = T.b, e = T.e, m = e - b;
     const Choice ch = warp_choose(bins + (size_t)w * SAH_BIN_WORDS, lane);
@@ -456,18 +477,18 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_split(SahTask* tasks, int32
         const int cb = s ? b + nl : b, ce = s ? e : b + nl, cm = ce - cb;
         if (cm == 1) {
             if (lane == 0) make_leaf(L, id, s, cb, -1);
-        } else if (cm <= SAH_CH) {
+        } else if (cm <= blk) {
             if (lane == 0) {
-                const int q = atomicAdd(counters + 2, 1);
+                const int q = atomicAdd(counters + CT_BLOCKS, 1);
                 if (q < cap_blist) blist[q] = SahRange{cb, ce, id, s | ((T.buf ^ 1) << 1)};
-                else atomicOr(counters + 3, 1);
+                else atomicOr(counters + CT_BAD, 1);
             }
         } else {
             const int nch = (cm + SAH_CH - 1) / SAH_CH;
             int q = 0, c0 = 0;
             if (lane == 0) {
-                q = atomicAdd(counters, 1);
-                c0 = atomicAdd(counters + 1, nch);
+                q = atomicAdd(counters + lev + 2, 1);
+                c0 = atomicAdd(counters + lev + 3, nch);
             }
             q = __shfl_sync(FULL, q, 0);
             c0 = __shfl_sync(FULL, c0, 0);
@@ -489,7 +510,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_split(SahTask* tasks, int32
                     next_chunks[c0 + k] = make_int4(q, cb + k * SAH_CH, min(SAH_CH, ce - (cb + k * SAH_CH)), 0);
                 for (int i = lane; i < SAH_BIN_WORDS; i += 32) next_bins[(size_t)q * SAH_BIN_WORDS + i] = bin_init(i);
             } else if (lane == 0) {
-                atomicOr(counters + 3, 1);
+                atomicOr(counters + CT_BAD, 1);
             }
         }
     }
@@ -509,9 +530,11 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_partition(const int4* __res
                                                                const SahTask* __restrict__ tasks,
                                                                const int32_t* __restrict__ left_off, int32_t* ord0,
                                                                int32_t* ord1, const float4* __restrict__ pbox,
-                                                               int32_t* __restrict__ order_final, SahTask* next) {
+                                                               int32_t* __restrict__ order_final, SahTask* next,
+                                                               const int32_t* counters, int lev) {
     __shared__ int s_warp[SAH_WARPS];
     __shared__ uint32_t s_cb[2][6];
+    if ((int)blockIdx.x >= counters[lev + 1] || counters[CT_BAD]) return;
     const int4 ch = chunks[blockIdx.x];
     const SahTask& T = tasks[ch.x];
     const int32_t* src = T.buf ? ord1 : ord0;
@@ -588,53 +611,52 @@ struct BlockSmem {
     uint32_t bins[SAH_BIN_WORDS];
     SahRange stack[BLK_STACK];
     SahRange wlist[WLIST_CAP];
-    SahRange wstack[SAH_WARPS][WSTACK];
     float red[SAH_WARPS][6];
     int scan[SAH_WARPS];
     Choice choice;
-    int top, nw, bad;
+    int top, nw, bad, take;
 };
 
-// Exact heuristic for a range of <= 32 positions, one warp; sub-ranges on a
-// warp-private stack.  Positions are local to the block's range (global
-// position = gb + local).
-__device__ void warp_exact(BlockSmem& S, SahRange r0, int gb, const Links& L, int lane, SahRange* st) {
-    int top = 1;
-    if (lane == 0) st[0] = r0;
-    __syncwarp();
-    for (int guard = 0; top > 0 && guard < 2 * WARP_MAX; guard++) {
-        const SahRange r = st[top - 1];
-        top--;
-        __syncwarp();
-        const int lb = r.b, mm = r.e - r.b;
-        int nl = 1;
-        if (mm > 2) {
-            const int slot = lane < mm ? (int)S.perm[lb + lane] : 0;
-            float c[3], lo[3], hi[3];
+// Exact heuristic for a range of <= 32 positions, one warp, one item per lane:
+// all sub-ranges of a tree level are split at once (segmented sorts, scans and
+// minima), so that a range takes as many steps as its subtree is deep, not as
+// many as it has nodes (a step is a long chain of shuffles, and a block's
+// warps are too few to hide it; node by node, the block tier of 1M triangles
+// took 1.7 ms, and that of 2.2k 0.5 ms).  Positions are local to the block's range
+// (global position = gb + local).
+__device__ void warp_exact(BlockSmem& S, SahRange r0, int gb, const Links& L, int lane) {
+    const int lb = r0.b, m = r0.e - r0.b;
+    int slot = lane < m ? (int)S.perm[lb + lane] : 0;
+    float lo[3], hi[3];
 #pragma unroll
-            for (int k = 0; k < 3; k++) {
-                lo[k] = lane < mm ? S.lo[k][slot] : CUDART_INF_F;
-                hi[k] = lane < mm ? S.hi[k][slot] : -CUDART_INF_F;
-                c[k] = lane < mm ? cen(lo[k], hi[k]) : CUDART_INF_F;
-            }
-            float bestc = CUDART_INF_F;
-            int bestj = 0, bestidx = lane;
+    for (int k = 0; k < 3; k++) {
+        lo[k] = S.lo[k][slot];
+        hi[k] = S.hi[k][slot];
+    }
+    // this lane's segment: first lane, size (a lane without an item: itself, 0)
+    int sb = lane < m ? 0 : lane, sm = lane < m ? m : 0;
+    int parent = r0.parent, side = r0.sb & 1;
+    // every level splits every segment of two or more: at most 31 levels
+    for (int level = 0; level < WARP_MAX && __any_sync(FULL, sm >= 2); level++) {
+        const int end = sb + sm - 1;                     // last lane of the segment
+        float bestc = CUDART_INF_F;
+        int bestj = sb, bestidx = lane;
+        if (__any_sync(FULL, sm >= 3)) {
             for (int a = 0; a < 3; a++) {
-                float key = c[a];
-                int idx = lane;
+                // sort by (segment, centroid, lane); a pair keeps its order
+                const uint32_t key = sm >= 3 ? f2o(cen(a == 0 ? lo[0] : (a == 1 ? lo[1] : lo[2]),
+                                                       a == 0 ? hi[0] : (a == 1 ? hi[1] : hi[2]))) : 0u;
+                unsigned long long v = ((unsigned long long)sb << 37) | ((unsigned long long)key << 5) |
+                                       (unsigned long long)lane;
 #pragma unroll
                 for (int k = 2; k <= 32; k <<= 1)
 #pragma unroll
                     for (int j = k >> 1; j > 0; j >>= 1) {
-                        const float ok = __shfl_xor_sync(FULL, key, j);
-                        const int oi = __shfl_xor_sync(FULL, idx, j);
-                        const bool other_less = ok < key || (ok == key && oi < idx);
+                        const unsigned long long o = __shfl_xor_sync(FULL, v, j);
                         const bool keep_min = ((lane & j) == 0) == ((lane & k) == 0);
-                        if (keep_min ? other_less : !other_less) {
-                            key = ok;
-                            idx = oi;
-                        }
+                        v = keep_min == (o < v) ? o : v;
                     }
+                const int idx = (int)(v & 31ull);
                 float plo[3], phi[3], slo[3], shi[3];
 #pragma unroll
                 for (int k = 0; k < 3; k++) {
@@ -647,11 +669,11 @@ __device__ void warp_exact(BlockSmem& S, SahRange r0, int gb, const Links& L, in
                     for (int k = 0; k < 3; k++) {
                         const float ul = __shfl_up_sync(FULL, plo[k], o), uh = __shfl_up_sync(FULL, phi[k], o);
                         const float dl = __shfl_down_sync(FULL, slo[k], o), dh = __shfl_down_sync(FULL, shi[k], o);
-                        if (lane >= o) {
+                        if (lane - o >= sb) {
                             plo[k] = fminf(plo[k], ul);
                             phi[k] = fmaxf(phi[k], uh);
                         }
-                        if (lane + o < 32) {
+                        if (lane + o <= end) {
                             slo[k] = fminf(slo[k], dl);
                             shi[k] = fmaxf(shi[k], dh);
                         }
@@ -663,50 +685,49 @@ __device__ void warp_exact(BlockSmem& S, SahRange r0, int gb, const Links& L, in
                     rhi[k] = __shfl_down_sync(FULL, shi[k], 1);
                 }
                 float cost = CUDART_INF_F;
-                if (lane < mm - 1)
-                    cost = half_area3(plo, phi) * (float)(lane + 1) + half_area3(rlo, rhi) * (float)(mm - 1 - lane);
+                if (lane < end)
+                    cost = half_area3(plo, phi) * (float)(lane - sb + 1) + half_area3(rlo, rhi) * (float)(end - lane);
                 // equal costs: the split nearest the middle, then the smaller one
                 float bc = cost;
                 int bl = lane;
 #pragma unroll
-                for (int o = 16; o >= 1; o >>= 1) {
-                    const float c2 = __shfl_xor_sync(FULL, bc, o);
-                    const int l2 = __shfl_xor_sync(FULL, bl, o);
-                    const int d1 = abs(2 * bl + 2 - mm), d2 = abs(2 * l2 + 2 - mm);
-                    if (c2 < bc || (c2 == bc && (d2 < d1 || (d2 == d1 && l2 < bl)))) {
+                for (int o = 1; o < 32; o <<= 1) {
+                    const float c2 = __shfl_up_sync(FULL, bc, o);
+                    const int l2 = __shfl_up_sync(FULL, bl, o);
+                    const int d1 = abs(2 * (bl - sb) + 2 - sm), d2 = abs(2 * (l2 - sb) + 2 - sm);
+                    if (lane - o >= sb && (c2 < bc || (c2 == bc && (d2 < d1 || (d2 == d1 && l2 < bl))))) {
                         bc = c2;
                         bl = l2;
                     }
                 }
-                if (bc < bestc) {
+                bc = __shfl_sync(FULL, bc, max(end, 0) & 31);
+                bl = __shfl_sync(FULL, bl, max(end, 0) & 31);
+                if (sm >= 3 && bc < bestc) {
                     bestc = bc;
                     bestj = bl;
                     bestidx = idx;
                 }
             }
-            nl = bestj + 1;
-            // position lb + lane takes the slot that sorted to rank `lane`
-            const int ns = __shfl_sync(FULL, slot, bestidx);
-            if (lane < mm) S.perm[lb + lane] = (uint16_t)ns;
-            __syncwarp();
         }
-        const int id = L.node_ids ? L.node_ids[lb + nl - 1] : gb + lb + nl - 1;
-        if (lane == 0) make_node(L, id, r.parent, r.sb & 1);
-        for (int s = 0; s < 2; s++) {
-            const int cb = s ? lb + nl : lb, ce = s ? r.e : lb + nl;
-            if (ce - cb == 1) {
-                if (lane == 0) make_leaf(L, id, s, gb + cb, S.tri[S.perm[cb]]);
-            } else {
-                if (lane == 0 && top < WSTACK) st[top] = SahRange{cb, ce, id, s};
-                top++;
-            }
+        // position lb + lane takes the item that sorted to this lane
+        slot = __shfl_sync(FULL, slot, bestidx);
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            lo[k] = __shfl_sync(FULL, lo[k], bestidx);
+            hi[k] = __shfl_sync(FULL, hi[k], bestidx);
         }
-        if (top > WSTACK) {                   // cannot happen: disjoint ranges of >= 2 in 32
-            if (lane == 0) S.bad = 1;
-            top = WSTACK;
+        if (sm >= 2) {
+            const int nl = bestj - sb + 1;
+            const int id = L.node_ids ? L.node_ids[lb + sb + nl - 1] : gb + lb + sb + nl - 1;
+            if (lane == sb) make_node(L, id, parent, side);
+            parent = id;
+            side = lane < sb + nl ? 0 : 1;
+            sm = side ? sm - nl : nl;
+            if (side) sb += nl;
+            if (sm == 1) make_leaf(L, id, side, gb + lb + lane, S.tri[slot]);
         }
-        __syncwarp();
     }
+    if (lane < m) S.perm[lb + lane] = (uint16_t)slot;
 }
 
 __global__ void __launch_bounds__(SAH_THREADS) k_sah_block(const SahRange* __restrict__ blist,
@@ -717,7 +738,14 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_block(const SahRange* __res
                                                            int32_t* counters) {
     extern __shared__ __align__(16) unsigned char sah_smem[];
     BlockSmem& S = *reinterpret_cast<BlockSmem*>(sah_smem);
-    const SahRange R = blist[blockIdx.x];
+    // the ranges are on the device; blocks take them from a counter
+    const int count = counters[CT_BLOCKS];
+    for (;;) {
+    if (threadIdx.x == 0) S.take = atomicAdd(counters + CT_TAKEN, 1);
+    __syncthreads();
+    const int mine = S.take;
+    if (mine >= count) return;                 // block-uniform
+    const SahRange R = blist[mine];
     const int gb = R.b, m = R.e - R.b;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int32_t* ord = (R.sb >> 1) ? ord1 : ord0;
@@ -843,22 +871,24 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_block(const SahRange* __res
         }
         __syncthreads();
     }
-    for (int q = warp; q < S.nw; q += SAH_WARPS) warp_exact(S, S.wlist[q], gb, L, lane, S.wstack[warp]);
+    for (int q = warp; q < S.nw; q += SAH_WARPS) warp_exact(S, S.wlist[q], gb, L, lane);
     __syncthreads();
     if (order_final)
         for (int i = tid; i < m; i += SAH_THREADS) order_final[gb + i] = S.tri[S.perm[i]];
-    if (tid == 0 && (S.bad || S.top != 0)) atomicOr(counters + 3, 2);
+    if (tid == 0 && (S.bad || S.top != 0)) atomicOr(counters + CT_BAD, 2);
+    __syncthreads();                           // the next range reuses S
+    }
 }
 
 }  // namespace
 
 size_t sah_scratch_bytes(int64_t n) {
-    const int64_t cap_task = n / (SAH_CH + 1) + 2;
-    const int64_t cap_chunk = 2 * (n / SAH_CH) + 4;
+    const int64_t cap_task = n / (blk_of(n) + 1) + 2;
+    const int64_t cap_chunk = n / SAH_CH + cap_task + 4;
     const int64_t cap_blist = n / 2 + 2;
     return sizeof(float4) * 2 * n + sizeof(int32_t) * 3 * n + sizeof(uint32_t) * 3 * NB * cap_chunk +
            sizeof(int32_t) * cap_chunk + sizeof(SahTask) * 2 * cap_task + sizeof(int4) * 2 * cap_chunk +
-           sizeof(uint32_t) * SAH_BIN_WORDS * 2 * cap_task + sizeof(SahRange) * cap_blist + 16 * sizeof(int32_t) +
+           sizeof(uint32_t) * SAH_BIN_WORDS * 2 * cap_task + sizeof(SahRange) * cap_blist + CT_WORDS * sizeof(int32_t) +
            16 * 256;   // alignment slack
 }
 
@@ -876,8 +906,8 @@ struct SahArena {
 };
 
 cudaError_t carve(void* scratch, int32_t n, SahArena& A) {
-    A.cap_task = n / (SAH_CH + 1) + 2;
-    A.cap_chunk = 2 * (n / SAH_CH) + 4;
+    A.cap_task = n / (blk_of(n) + 1) + 2;
+    A.cap_chunk = n / SAH_CH + A.cap_task + 4;
     A.cap_blist = n / 2 + 2;
     unsigned char* p = (unsigned char*)scratch;
     auto take = [&](size_t bytes) {
@@ -894,7 +924,7 @@ cudaError_t carve(void* scratch, int32_t n, SahArena& A) {
     for (int k = 0; k < 2; k++) A.chunks[k] = (int4*)take(sizeof(int4) * (size_t)A.cap_chunk);
     for (int k = 0; k < 2; k++) A.bins[k] = (uint32_t*)take(sizeof(uint32_t) * SAH_BIN_WORDS * (size_t)A.cap_task);
     A.blist = (SahRange*)take(sizeof(SahRange) * (size_t)A.cap_blist);
-    A.counters = (int32_t*)take(16 * sizeof(int32_t));
+    A.counters = (int32_t*)take(CT_WORDS * sizeof(int32_t));
     return (size_t)(p - (unsigned char*)scratch) > sah_scratch_bytes(n) ? cudaErrorInvalidValue : cudaSuccess;
 }
 
@@ -910,40 +940,61 @@ cudaError_t block_attr(rtsdf_ctx* c) {
     return cudaSuccess;
 }
 
-// The level loop over big ranges, then the block ranges; ntask / nchunk /
-// nblock describe the first level (already in A).
-cudaError_t run_levels(rtsdf_ctx* c, SahArena& A, const Links& L, int32_t* order, int32_t ntask, int32_t nchunk,
-                       int32_t nblock) {
+// The levels over big ranges, then the block ranges; the first level (ntask
+// ranges of at most `largest` positions) is in A and its counts in A.counters.
+// Levels are enqueued in batches, each with the largest grid that it can need
+// and kernels that read the level's size on the device; the host looks once
+// per batch whether ranges are left (one batch nearly always does).  With a
+// look after every level, the host round trips were a third of a build.
+cudaError_t run_levels(rtsdf_ctx* c, SahArena& A, const Links& L, int32_t* order, int32_t n, int32_t ntask,
+                       int32_t largest) {
     cudaError_t e;
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+    const int blk = blk_of(n);
     int cur = 0;
-    for (int level = 0; ntask > 0; level++) {
-        if (level >= 4096) return cudaErrorUnknown;   // sizes shrink every level; only a fault gets here
-        if ((e = cudaMemsetAsync(A.counters, 0, 2 * sizeof(int32_t), c->stream))) return e;
-        RTSDF_LAUNCH(c, k_sah_bin, (unsigned)nchunk, SAH_THREADS, 0, A.chunks[cur], A.tasks[cur], A.ord0, A.ord1,
-                     A.pbox, A.bins[cur], A.hist);
-        RTSDF_LAUNCH(c, k_sah_split, (unsigned)((ntask + SAH_WARPS - 1) / SAH_WARPS), SAH_THREADS, 0, A.tasks[cur],
-                     ntask, A.bins[cur], A.hist, A.chunks[cur], A.loff, L, A.tasks[cur ^ 1], A.chunks[cur ^ 1],
-                     A.bins[cur ^ 1], A.blist, A.counters, A.cap_task, A.cap_chunk, A.cap_blist);
-        RTSDF_LAUNCH(c, k_sah_partition, (unsigned)nchunk, SAH_THREADS, 0, A.chunks[cur], A.tasks[cur], A.loff, A.ord0,
-                     A.ord1, A.pbox, order, A.tasks[cur ^ 1]);
-        int32_t h[4] = {0, 0, 0, 0};
+    // a binned split is rarely further off the middle than these allow for
+    int levels = 0;
+    if (ntask > 0) {
+        while (((int64_t)blk << levels) < largest) levels++;
+        levels = std::min(levels + 3, LEVEL_BATCH);
+    }
+    const int64_t block_grid = std::min<int64_t>(std::max<int64_t>(n / 64, 1), 4 * (int64_t)(sms > 0 ? sms : 132));
+    for (int batch = 0;; batch++) {
+        if (batch >= 4096) return cudaErrorUnknown;   // sizes shrink every level; only a fault gets here
+        int64_t tasks = ntask;
+        for (int l = 0; l < levels; l++) {
+            const int lev = CT_LEVELS + 2 * l;
+            const unsigned gt = (unsigned)((tasks + SAH_WARPS - 1) / SAH_WARPS);
+            const unsigned gc = (unsigned)std::min<int64_t>(n / SAH_CH + tasks + 1, A.cap_chunk);
+            RTSDF_LAUNCH(c, k_sah_bin, gc, SAH_THREADS, 0, A.chunks[cur], A.tasks[cur], A.ord0, A.ord1, A.pbox,
+                         A.bins[cur], A.hist, A.counters, lev);
+            RTSDF_LAUNCH(c, k_sah_split, gt, SAH_THREADS, 0, A.tasks[cur], lev, A.bins[cur], A.hist, A.chunks[cur],
+                         A.loff, L, A.tasks[cur ^ 1], A.chunks[cur ^ 1], A.bins[cur ^ 1], A.blist, A.counters,
+                         A.cap_task, A.cap_chunk, A.cap_blist, blk);
+            RTSDF_LAUNCH(c, k_sah_partition, gc, SAH_THREADS, 0, A.chunks[cur], A.tasks[cur], A.loff, A.ord0, A.ord1,
+                         A.pbox, order, A.tasks[cur ^ 1], A.counters, lev);
+            tasks = std::min<int64_t>(2 * tasks, A.cap_task);
+            cur ^= 1;
+        }
+        RTSDF_LAUNCH(c, k_sah_block, (unsigned)block_grid, SAH_THREADS, sizeof(BlockSmem), A.blist, A.ord0, A.ord1,
+                     A.pbox, order, L, A.counters);
+        int32_t h[CT_WORDS];
         if ((e = cudaGetLastError())) return e;
         if ((e = cudaMemcpyAsync(h, A.counters, sizeof(h), cudaMemcpyDeviceToHost, c->stream))) return e;
         if ((e = cudaStreamSynchronize(c->stream))) return e;
-        if (h[3] != 0 || h[0] > A.cap_task || h[1] > A.cap_chunk || h[2] > A.cap_blist) return cudaErrorUnknown;
-        ntask = h[0];
-        nchunk = h[1];
-        nblock = h[2];
-        cur ^= 1;
+        if (h[CT_BAD] != 0) return cudaErrorUnknown;   // a capacity guard fired: cannot happen for a valid range
+        ntask = h[CT_LEVELS + 2 * levels];
+        if (ntask == 0) return cudaSuccess;
+        // the ranges that are left become the first level of another batch
+        int32_t r[CT_WORDS] = {0};
+        r[CT_BLOCKS] = r[CT_TAKEN] = h[CT_BLOCKS];
+        r[CT_LEVELS] = ntask;
+        r[CT_LEVELS + 1] = h[CT_LEVELS + 2 * levels + 1];
+        if ((e = cudaMemcpyAsync(A.counters, r, sizeof(r), cudaMemcpyHostToDevice, c->stream))) return e;
+        if ((e = cudaStreamSynchronize(c->stream))) return e;   // r is a local buffer
+        levels = 4;
     }
-    if (nblock > 0)
-        RTSDF_LAUNCH(c, k_sah_block, (unsigned)nblock, SAH_THREADS, sizeof(BlockSmem), A.blist, A.ord0, A.ord1,
-                     A.pbox, order, L, A.counters);
-    if ((e = cudaGetLastError())) return e;
-    int32_t bad = 0;
-    if ((e = cudaMemcpyAsync(&bad, A.counters + 3, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream))) return e;
-    if ((e = cudaStreamSynchronize(c->stream))) return e;
-    return bad ? cudaErrorUnknown : cudaSuccess;   // a capacity guard fired: cannot happen for a valid range
 }
 
 }  // namespace
@@ -954,16 +1005,16 @@ cudaError_t sah_topology(rtsdf_ctx* c, void* scratch, int32_t* order) {
     SahArena A;
     cudaError_t e = carve(scratch, n, A);
     if (!e) e = block_attr(c);
-    if (!e) e = cudaMemsetAsync(A.counters, 0, 16 * sizeof(int32_t), c->stream);
+    if (!e) e = cudaMemsetAsync(A.counters, 0, CT_WORDS * sizeof(int32_t), c->stream);
     if (e) return e;
     const int nch0 = (n + SAH_CH - 1) / SAH_CH;
     const int init_threads = nch0 > SAH_BIN_WORDS ? nch0 : SAH_BIN_WORDS;
     RTSDF_LAUNCH(c, k_sah_root, (unsigned)((init_threads + 255) / 256), 256, 0, A.tasks[0], A.chunks[0], A.bins[0],
-                 A.blist, n);
+                 A.blist, n, blk_of(n), A.counters);
     RTSDF_LAUNCH(c, k_sah_prims, (unsigned)((n + SAH_THREADS - 1) / SAH_THREADS), SAH_THREADS, 0, c->verts, c->tris,
                  n, A.pbox, A.ord0, A.tasks[0]);
     const Links L{bv.nodes, bv.leaf_parent, bv.root, nullptr, nullptr, nullptr};
-    return run_levels(c, A, L, order, n > SAH_CH ? 1 : 0, nch0, n > SAH_CH ? 0 : 1);
+    return run_levels(c, A, L, order, n, n > blk_of(n) ? 1 : 0, n);
 }
 
 cudaError_t sah_segments(rtsdf_ctx* c, void* scratch, int32_t* order, const int32_t* order_in,
@@ -979,13 +1030,15 @@ cudaError_t sah_segments(rtsdf_ctx* c, void* scratch, int32_t* order, const int3
     std::vector<int4> chunks;
     std::vector<SahRange> blist;
     std::vector<int32_t> root0((size_t)nseg, 0);
+    int32_t largest = 0;
     for (int32_t k = 0; k < nseg; k++) {
         const int32_t b = bounds[k], en = bounds[k + 1], m = en - b;
         if (m == 1) {
             root0[(size_t)k] = ~b;                // a one-triangle segment is its own leaf
-        } else if (m <= SAH_CH) {
+        } else if (m <= blk_of(n)) {
             blist.push_back(SahRange{b, en, -2 - k, 0});
         } else {
+            largest = std::max(largest, m);
             SahTask t;
             memset(&t, 0, sizeof(t));
             t.b = b; t.e = en; t.parent = -2 - k; t.side = 0; t.buf = 0;
@@ -1000,8 +1053,10 @@ cudaError_t sah_segments(rtsdf_ctx* c, void* scratch, int32_t* order, const int3
     if ((int64_t)tasks.size() > A.cap_task || (int64_t)chunks.size() > A.cap_chunk ||
         (int64_t)blist.size() > A.cap_blist)
         return cudaErrorInvalidValue;   // cannot happen: the segments partition [0, n)
-    int32_t h0[16] = {0};
-    h0[2] = (int32_t)blist.size();
+    int32_t h0[CT_WORDS] = {0};
+    h0[CT_BLOCKS] = (int32_t)blist.size();
+    h0[CT_LEVELS] = (int32_t)tasks.size();
+    h0[CT_LEVELS + 1] = (int32_t)chunks.size();
     if ((e = cudaMemcpyAsync(A.counters, h0, sizeof(h0), cudaMemcpyHostToDevice, c->stream))) return e;
     if ((e = cudaMemcpyAsync(seg_root, root0.data(), sizeof(int32_t) * (size_t)nseg, cudaMemcpyHostToDevice,
                              c->stream)))
@@ -1026,7 +1081,7 @@ cudaError_t sah_segments(rtsdf_ctx* c, void* scratch, int32_t* order, const int3
         return e;
     const Links L{bv.nodes, bv.leaf_parent, bv.root, seg_root, nullptr, nullptr};
     // the host vectors must outlive the copies above: run_levels synchronises
-    return run_levels(c, A, L, order, (int32_t)tasks.size(), (int32_t)chunks.size(), (int32_t)blist.size());
+    return run_levels(c, A, L, order, n, (int32_t)tasks.size(), largest);
 }
 
 size_t sah_top_bytes(int32_t nseg) {
@@ -1036,6 +1091,7 @@ size_t sah_top_bytes(int32_t nseg) {
 cudaError_t sah_top_prepare(rtsdf_ctx* c, void* scratch, int32_t nseg) {
     if (nseg < 1 || nseg > SAH_CH) return cudaErrorInvalidValue;
     std::vector<unsigned char> h(sah_top_bytes(nseg), 0);
+    ((int32_t*)h.data())[CT_BLOCKS] = 1;
     SahRange r{0, nseg, -1, 0};
     memcpy(h.data() + 256, &r, sizeof(r));
     int32_t* list = (int32_t*)(h.data() + 512);
@@ -1061,6 +1117,7 @@ cudaError_t sah_top(rtsdf_ctx* c, void* scratch, int32_t nseg, const float4* box
     int32_t* list = (int32_t*)(p + 512);
     const Links L{bv.nodes, bv.leaf_parent, bv.root, nullptr, node_ids, child_of};
     // counters, the range {0, nseg} and the identity list come from sah_top_prepare
+    if ((e = cudaMemsetAsync(counters + CT_TAKEN, 0, sizeof(int32_t), c->stream))) return e;
     RTSDF_LAUNCH(c, k_sah_block, 1, SAH_THREADS, sizeof(BlockSmem), range, list, list, boxes, (int32_t*)nullptr, L,
                  counters);
     return cudaGetLastError();

@@ -59,11 +59,8 @@ struct Bvh {
     BNode* nodes = nullptr;        // [nt - 1]
     WNode* wide = nullptr;         // [n_wide] (capacity wide_cap = nt - 1)
     int64_t wide_cap = 0;
-    // device collapse scratch: frontier (binary node, wide slot) x 2, kids, counts
-    int32_t *col_fb = nullptr, *col_fslot = nullptr, *col_nb = nullptr, *col_nslot = nullptr;
-    int4* col_kids = nullptr;
-    uint32_t* col_nint = nullptr;
-    int32_t* col_total = nullptr;
+    // device collapse scratch: binary root of each wide node, (first slot, count) per level
+    int32_t *col_from = nullptr, *col_lev = nullptr;
     int64_t col_cap = 0;
     int64_t n_wide = 0;
     cudaTextureObject_t wtex = 0;  // the wide nodes as int4 texels (0: none; see make_int4_texture)
@@ -76,9 +73,9 @@ struct Bvh {
     int32_t* root = nullptr;       // [1] binary root node (device)
     int64_t cap_nt = 0;            // capacity of the per-triangle arrays above
     // build scratch, kept across builds: Morton keys / order x 2, radix
-    // histograms, depth, and the SAH builder's arena
+    // histograms, and the SAH builder's arena
     uint32_t *mk0 = nullptr, *mk1 = nullptr, *hist = nullptr;
-    int32_t *mv0 = nullptr, *mv1 = nullptr, *d_depth = nullptr;
+    int32_t *mv0 = nullptr, *mv1 = nullptr;
     void* sah = nullptr;
     size_t sah_bytes = 0;
     // two-level form (RTSDF_BVH_TWO_LEVEL): one subtree per object, kept

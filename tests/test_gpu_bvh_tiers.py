@@ -1,0 +1,43 @@
+"""The SAH build at the edges of its tiers (warp, block, levels) and on meshes
+whose splits are far off the middle, so that a build takes more than one batch
+of levels, top-down and in the 4-wide collapse: every tree is valid over all
+triangles, and the distances traced through it equal the oracle's."""
+import numpy as np
+import pytest
+
+import oracle
+from tests.test_gpu_bvh import _check_tree
+
+pytestmark = pytest.mark.gpu
+
+
+def _soup(n, seed=5):
+    rng = np.random.default_rng(seed)
+    c = rng.uniform(0.1, 0.9, (n, 1, 3))
+    return c + rng.uniform(-0.03, 0.03, (n, 3, 3))
+
+
+def _geometric(n):
+    """Triangles that shrink and close in on a corner by a constant factor."""
+    f = 0.993 ** np.arange(n)[:, None, None]
+    shape = np.array([[0.0, 0, 0], [0.02, 0, 0.01], [0, 0.02, 0.005]])[None]
+    return 0.1 + f * (0.8 * np.array([1.0, 0.6, 0.3])[None, None] + shape)
+
+
+@pytest.mark.parametrize("name, n", [("soup", n) for n in (2, 3, 31, 32, 33, 64, 255, 256, 257, 513, 1024, 1025, 4099)] +
+                         [("geometric", 700), ("geometric", 3000)])
+def test_tiers(name, n):
+    from paper_2210_04449_gb300 import RTSDF
+    v = (_soup(n) if name == "soup" else _geometric(n)).reshape(-1, 3).astype(np.float32)
+    t = np.arange(3 * n, dtype=np.int32).reshape(-1, 3)
+    nc, R = 8, 8
+    rt = RTSDF(nc, seed=2)
+    rt.upload_mesh(v, t)
+    rt.build_bvh()
+    ch, lt, root = rt.bvh_topology()
+    _check_tree(ch, lt, root, n)
+    rt.update(2.0, R, 0)
+    rt.sync()
+    pipe = oracle.FinePipeline(np.zeros(3, np.float32), 1.0, nc, 0.5, 2.0, 1.0, 2, accel="bvh")
+    pipe.frame(v, t, 0, R)
+    assert np.array_equal(rt.grids()["accum"].cpu().numpy().astype(np.float64), pipe.u)
