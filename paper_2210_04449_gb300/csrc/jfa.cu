@@ -64,6 +64,12 @@ __global__ void __launch_bounds__(128, 4) k_jfa_zblock(const uint32_t* __restric
     dev::jfa_zblock_column<FINAL, T>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
 }
 
+// Columns below which shorter ones are taken: a thread floods its column
+// serially.  All passes: 16^3 20.7 -> 16.6 us, 32^3 28.1 -> 20.7, 61^3 45.2 -> 40.0
+// (38.0 with 50,000 columns, but 75^3 66.9 instead of 64.9); from 96^3 on, more
+// columns cost more than they hide (98 instead of 88 us at 96^3 with 400,000).
+constexpr int64_t JFA_COLUMNS = 100000;
+
 template <int T>
 void launch_zblock(rtsdf_ctx* c, const uint32_t* in, uint32_t* out, int n, int k, bool final, float beta_h) {
     const int lat = (n + k - 1) / k;          // z-lattice members of the fullest residue class
@@ -100,9 +106,14 @@ cudaError_t launch_jfa(rtsdf_ctx* c) {
             case 2: launch_pass<128, 2>(c, in, out, n, k, k == 1, beta_h); break;
             case 3: launch_pass<32, 4>(c, in, out, n, k, k == 1, beta_h); break;
             case 4: {
+                // columns of up to 8 voxels, shorter where the lattice is or
+                // where the columns would be too few to fill the GPU
                 const int lat = (n + k - 1) / k;
-                if (lat <= 2) launch_zblock<2>(c, in, out, n, k, k == 1, beta_h);
-                else if (lat <= 4) launch_zblock<4>(c, in, out, n, k, k == 1, beta_h);
+                const int64_t cols = (int64_t)n * n * k;
+                int t = 8;
+                while (t > 2 && (t / 2 >= lat || cols * ((lat + t - 1) / t) < JFA_COLUMNS)) t /= 2;
+                if (t == 2) launch_zblock<2>(c, in, out, n, k, k == 1, beta_h);
+                else if (t == 4) launch_zblock<4>(c, in, out, n, k, k == 1, beta_h);
                 else launch_zblock<8>(c, in, out, n, k, k == 1, beta_h);
                 break;
             }
