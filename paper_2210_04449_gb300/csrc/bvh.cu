@@ -296,6 +296,7 @@ __global__ void k_top_up(const int32_t* __restrict__ child, int32_t n, const int
 
 __global__ void k_depth(const int32_t* __restrict__ leaf_parent, const BNode* __restrict__ nodes, int64_t n,
                         int32_t* depth) {
+    chain_begin();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     int d = 1;
@@ -454,6 +455,7 @@ __global__ void __launch_bounds__(128) k_collapse_level(int32_t* lev, int l, int
                                                         const float* __restrict__ nbox,
                                                         const float* __restrict__ lbox, int32_t* from,
                                                         WNode* __restrict__ wide) {
+    chain_begin();
     const int32_t first = lev[2 * l];
     const int32_t cnt = min(lev[2 * l + 1], max((int32_t)(cap - first), 0));   // (all of it, unless the tree is damaged)
     const int32_t next = first + cnt;
@@ -519,6 +521,7 @@ __global__ void __launch_bounds__(128) k_collapse_level(int32_t* lev, int l, int
 }
 
 __global__ void k_collapse_root(const int32_t* root, int32_t* from, int32_t* lev) {
+    chain_begin();
     if (threadIdx.x == 0) from[0] = *root;
     if (threadIdx.x < COL_WORDS) lev[threadIdx.x] = threadIdx.x == 1 ? 1 : 0;   // (64 threads)
 }
@@ -554,9 +557,9 @@ static cudaError_t collapse_wide(rtsdf_ctx* c, int* depth) {
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     const int64_t most = 16 * (int64_t)(sms > 0 ? sms : 132);
-    RTSDF_LAUNCH(c, k_collapse_root, 1, 64, 0, b.root, b.col_from, b.col_lev);
+    launch_chain(c, k_collapse_root, 1, 64, 0, b.root, b.col_from, b.col_lev);
     if (depth)
-        RTSDF_LAUNCH(c, k_depth, (unsigned)((n + 255) / 256), 256, 0, b.leaf_parent, b.nodes, n,
+        launch_chain(c, k_depth, (unsigned)((n + 255) / 256), 256, 0, b.leaf_parent, b.nodes, n,
                      b.col_lev + COL_WORDS - 1);
     // a batch of levels for a tree whose leaves are a few levels apart; a
     // deeper one takes more batches
@@ -566,7 +569,7 @@ static cudaError_t collapse_wide(rtsdf_ctx* c, int* depth) {
     for (int batch = 0;; batch++) {
         if (batch >= (1 << 24)) return cudaErrorUnknown;
         for (int l = 0; l < levels; l++) {
-            RTSDF_LAUNCH(c, k_collapse_level, (unsigned)std::min<int64_t>((std::min(nodes, cap) + 127) / 128, most), 128,
+            launch_chain(c, k_collapse_level, (unsigned)std::min<int64_t>((std::min(nodes, cap) + 127) / 128, most), 128,
                          0, b.col_lev, l, cap, b.nodes, b.nbox, b.lbox, b.col_from, b.wide);
             if (nodes < cap) nodes *= 4;
         }

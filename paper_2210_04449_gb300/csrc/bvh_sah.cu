@@ -391,6 +391,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_bin(const int4* __restrict_
                                                          uint32_t* __restrict__ hist,
                                                          const int32_t* counters, int lev) {
     __shared__ uint32_t sb[SAH_BIN_WORDS];
+    chain_begin();
     if ((int)blockIdx.x >= counters[lev + 1] || counters[CT_BAD]) return;
     const int4 ch = chunks[blockIdx.x];        // (task, start, length)
     const SahTask& T = tasks[ch.x];
@@ -441,6 +442,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_split(SahTask* tasks, int l
                                                            int4* next_chunks, uint32_t* next_bins, SahRange* blist,
                                                            int32_t* counters, int32_t cap_task, int32_t cap_chunk,
                                                            int32_t cap_blist, int blk) {
+    chain_begin();
     const int w = (int)((blockIdx.x * (unsigned)SAH_THREADS + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (w >= counters[lev] || counters[CT_BAD]) return;   // warp-uniform
@@ -534,6 +536,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_partition(const int4* __res
                                                                const int32_t* counters, int lev) {
     __shared__ int s_warp[SAH_WARPS];
     __shared__ uint32_t s_cb[2][6];
+    chain_begin();
     if ((int)blockIdx.x >= counters[lev + 1] || counters[CT_BAD]) return;
     const int4 ch = chunks[blockIdx.x];
     const SahTask& T = tasks[ch.x];
@@ -738,6 +741,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_block(const SahRange* __res
                                                            int32_t* counters) {
     extern __shared__ __align__(16) unsigned char sah_smem[];
     BlockSmem& S = *reinterpret_cast<BlockSmem*>(sah_smem);
+    chain_begin();
     // the ranges are on the device; blocks take them from a counter
     const int count = counters[CT_BLOCKS];
     for (;;) {
@@ -967,17 +971,17 @@ cudaError_t run_levels(rtsdf_ctx* c, SahArena& A, const Links& L, int32_t* order
             const int lev = CT_LEVELS + 2 * l;
             const unsigned gt = (unsigned)((tasks + SAH_WARPS - 1) / SAH_WARPS);
             const unsigned gc = (unsigned)std::min<int64_t>(n / SAH_CH + tasks + 1, A.cap_chunk);
-            RTSDF_LAUNCH(c, k_sah_bin, gc, SAH_THREADS, 0, A.chunks[cur], A.tasks[cur], A.ord0, A.ord1, A.pbox,
+            launch_chain(c, k_sah_bin, gc, SAH_THREADS, 0, A.chunks[cur], A.tasks[cur], A.ord0, A.ord1, A.pbox,
                          A.bins[cur], A.hist, A.counters, lev);
-            RTSDF_LAUNCH(c, k_sah_split, gt, SAH_THREADS, 0, A.tasks[cur], lev, A.bins[cur], A.hist, A.chunks[cur],
+            launch_chain(c, k_sah_split, gt, SAH_THREADS, 0, A.tasks[cur], lev, A.bins[cur], A.hist, A.chunks[cur],
                          A.loff, L, A.tasks[cur ^ 1], A.chunks[cur ^ 1], A.bins[cur ^ 1], A.blist, A.counters,
                          A.cap_task, A.cap_chunk, A.cap_blist, blk);
-            RTSDF_LAUNCH(c, k_sah_partition, gc, SAH_THREADS, 0, A.chunks[cur], A.tasks[cur], A.loff, A.ord0, A.ord1,
+            launch_chain(c, k_sah_partition, gc, SAH_THREADS, 0, A.chunks[cur], A.tasks[cur], A.loff, A.ord0, A.ord1,
                          A.pbox, order, A.tasks[cur ^ 1], A.counters, lev);
             tasks = std::min<int64_t>(2 * tasks, A.cap_task);
             cur ^= 1;
         }
-        RTSDF_LAUNCH(c, k_sah_block, (unsigned)block_grid, SAH_THREADS, sizeof(BlockSmem), A.blist, A.ord0, A.ord1,
+        launch_chain(c, k_sah_block, (unsigned)block_grid, SAH_THREADS, sizeof(BlockSmem), A.blist, A.ord0, A.ord1,
                      A.pbox, order, L, A.counters);
         int32_t h[CT_WORDS];
         if ((e = cudaGetLastError())) return e;

@@ -217,6 +217,38 @@ namespace rtsdf {
         (ctx)->launches++;                                                    \
     } while (0)
 
+// A chain of short dependent kernels is launched with programmatic stream
+// serialization: a kernel's blocks may be put on the SMs while the one before
+// it still runs, which hides most of the launch gap (1 to 2 us a kernel).
+// Every kernel launched this way begins with chain_begin(), before any access
+// to memory: it waits until the kernel before has finished and its writes are
+// visible (which has waited the same way, and so on back), and only then lets
+// the next one be launched, so that at most two kernels of a chain overlap and
+// none is started before all but its direct predecessor have ended.  Without
+// the attribute, or as the first of a chain, the wait is over at once.
+#ifdef __CUDACC__
+__device__ __forceinline__ void chain_begin() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
+template <class... P, class... A>
+inline cudaError_t launch_chain(rtsdf_ctx* c, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, A... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c->stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    c->launches++;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 // Stage launchers, one per translation unit; each returns a cudaError_t of
 // the launches (cudaGetLastError), never synchronises.
 cudaError_t launch_quantise(rtsdf_ctx* c);

@@ -57,6 +57,7 @@ template <bool FINAL, int T>
 __global__ void __launch_bounds__(128, 4) k_jfa_zblock(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
                                                       int n, int k, float* __restrict__ coarse, float hc,
                                                       float beta_h) {
+    chain_begin();
     const int x = blockIdx.x * 32 + threadIdx.x;
     const int y = blockIdx.y * 4 + threadIdx.y;
     const int rz = (int)(blockIdx.z % (unsigned)k), g = (int)(blockIdx.z / (unsigned)k);
@@ -75,8 +76,8 @@ void launch_zblock(rtsdf_ctx* c, const uint32_t* in, uint32_t* out, int n, int k
     const int lat = (n + k - 1) / k;          // z-lattice members of the fullest residue class
     const int groups = (lat + T - 1) / T;
     dim3 block(32, 4, 1), grid((n + 31) / 32, (n + 3) / 4, (unsigned)(groups * k));
-    if (final) RTSDF_LAUNCH(c, (k_jfa_zblock<true, T>), grid, block, 0, in, out, n, k, c->coarse, c->hc, beta_h);
-    else RTSDF_LAUNCH(c, (k_jfa_zblock<false, T>), grid, block, 0, in, out, n, k, c->coarse, c->hc, beta_h);
+    if (final) launch_chain(c, k_jfa_zblock<true, T>, grid, block, 0, in, out, n, k, c->coarse, c->hc, beta_h);
+    else launch_chain(c, k_jfa_zblock<false, T>, grid, block, 0, in, out, n, k, c->coarse, c->hc, beta_h);
 }
 
 // Coarse SDF without a pass (N = 1: no jump steps).
