@@ -91,8 +91,8 @@ void free_all(rtsdf_ctx* c) {
     dfree(c->verts); dfree(c->qverts); dfree(c->tris); dfree(c->vert_obj); dfree(c->obj_box);
     dfree(c->obj_trans); dfree(c->obj_xform); dfree(c->moved_list); dfree(c->d_moved_count);
     dfree(c->seeds[0]); dfree(c->seeds[1]); dfree(c->coarse); dfree(c->big_list); dfree(c->d_big_count);
-    dfree(c->accum); dfree(c->counts); dfree(c->fine); dfree(c->masked); dfree(c->d_masked_count);
-    dfree(c->ray_min); dfree(c->ray_cnt); dfree(c->d_next_ray);
+    dfree(c->accum); dfree(c->counts); dfree(c->fine); dfree(c->masked); dfree(c->d_frame_words);
+    dfree(c->ray_min); dfree(c->ray_cnt);
     dfree(c->bin_count); dfree(c->bin_start); dfree(c->bin_cursor); dfree(c->bin_items); dfree(c->bin_overflow);
     drop_texture(c->bvh.wtex);
     dfree(c->bvh.nodes); dfree(c->bvh.wide); dfree(c->bvh.nbox); dfree(c->bvh.lbox); dfree(c->bvh.tri); dfree(c->bvh.leaf_tri); dfree(c->bvh.leaf_parent); dfree(c->bvh.flags);
@@ -226,7 +226,6 @@ rtsdf_status rtsdf_create(const rtsdf_config* cfg, rtsdf_t* out) {
     if (!e) e = dalloc(&c->masked, c->nc3);
     if (!e) e = dalloc(&c->ray_min, 8 * c->nc3);
     if (!e) e = dalloc(&c->ray_cnt, 8 * c->nc3);
-    if (!e) e = dalloc(&c->d_next_ray, 1);
     {
         const size_t g = (size_t)(c->nc + 7) / 8, cells = g * g * g;
         c->bin_cap = 1u << 23;
@@ -237,14 +236,18 @@ rtsdf_status rtsdf_create(const rtsdf_config* cfg, rtsdf_t* out) {
         if (!e) e = dalloc(&c->bin_overflow, 1);
         if (!e) e = cudaMemsetAsync(c->bin_overflow, 0, sizeof(uint32_t), c->stream);
     }
-    if (!e) e = dalloc(&c->d_masked_count, 1);
+    if (!e) e = dalloc(&c->d_frame_words, FRAME_WORDS);
+    if (!e) {
+        c->d_masked_count = reinterpret_cast<uint32_t*>(c->d_frame_words);
+        c->d_next_ray = reinterpret_cast<unsigned long long*>(c->d_frame_words + 1);
+    }
     if (!e) e = dalloc(&c->d_big_count, 1);
     if (!e) e = dalloc(&c->d_moved_count, 1);
     if (!e) e = dalloc(&c->d_err, 1);
     if (!e) e = dalloc(&c->d_counters, 1);
     if (!e) e = cudaMemsetAsync(c->d_counters, 0, sizeof(TraceCounters), c->stream);
     if (!e) e = cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), c->stream);
-    if (!e) e = cudaMemsetAsync(c->d_masked_count, 0, sizeof(uint32_t), c->stream);
+    if (!e) e = cudaMemsetAsync(c->d_frame_words, 0, FRAME_WORDS * sizeof(uint64_t), c->stream);
     if (!e) e = cudaMemsetAsync(c->d_moved_count, 0, sizeof(int32_t), c->stream);
     if (!e) e = cudaMemsetAsync(c->seeds[0], 0xFF, c->nc3 * sizeof(uint32_t), c->stream);
     if (!e) e = cudaMemsetAsync(c->seeds[1], 0xFF, c->nc3 * sizeof(uint32_t), c->stream);

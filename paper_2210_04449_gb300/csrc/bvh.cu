@@ -224,6 +224,7 @@ __global__ void k_leaves_up(const float* __restrict__ verts, const int32_t* __re
                             const int32_t* order, int64_t n, float4* __restrict__ tri, int32_t* leaf_tri,
                             const int32_t* __restrict__ leaf_parent, BNode* nodes, uint32_t* flags, float pad,
                             float* __restrict__ lbox, float* __restrict__ nbox) {
+    chain_begin();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int32_t t = order[i];
@@ -309,14 +310,14 @@ __global__ void k_depth(const int32_t* __restrict__ leaf_parent, const BNode* __
 }
 
 // ---------------------------------------------------------------- motion
-__global__ void k_obj_boxes_init(float* boxes, int n_obj) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_obj) return;
-    for (int a = 0; a < 3; a++) {
-        boxes[6 * i + a] = CUDART_INF_F;
-        boxes[6 * i + 3 + a] = -CUDART_INF_F;
-    }
+// Rigid transforms, rows of [R | t] per object (12 floats).  An object is
+// moved unless its transform is exactly the identity.
+__device__ __forceinline__ bool xform_moves(const float* m) {
+    return m[0] != 1.f || m[1] != 0.f || m[2] != 0.f || m[3] != 0.f || m[4] != 0.f || m[5] != 1.f ||
+           m[6] != 0.f || m[7] != 0.f || m[8] != 0.f || m[9] != 0.f || m[10] != 1.f || m[11] != 0.f;
 }
+
+__device__ __forceinline__ bool trans_moves(const float* t) { return t[0] != 0.f || t[1] != 0.f || t[2] != 0.f; }
 
 __device__ __forceinline__ void atomic_min_f(float* a, float v) {
     if (v >= 0.f) atomicMin(reinterpret_cast<int*>(a), __float_as_int(v));
@@ -327,29 +328,68 @@ __device__ __forceinline__ void atomic_max_f(float* a, float v) {
     else atomicMin(reinterpret_cast<unsigned*>(a), __float_as_uint(v));
 }
 
-// Box of every moved object (before the move), then v += t[obj].
-__global__ void k_obj_boxes(const float* __restrict__ verts, const int32_t* __restrict__ vobj, int64_t nv,
-                            const float* __restrict__ trans, float* boxes) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= nv) return;
-    const int o = vobj[i];
-    const float* t = trans + 3 * o;
-    if (t[0] == 0.f && t[1] == 0.f && t[2] == 0.f) return;
+// Vertex i of object o (o < 0: none, or one that stays) into its object's box;
+// all 32 lanes call.  An object's vertices are mostly consecutive, so a warp
+// of one object sends one set of atomics (1M triangles: 173 us with one per
+// vertex, which queue up on 500 boxes).
+__device__ __forceinline__ void add_to_box(const float* __restrict__ verts, int64_t i, int o, float* boxes) {
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    const int o0 = __shfl_sync(FULL, o, 0);
+    if (__all_sync(FULL, o == o0)) {
+        if (o0 < 0) return;
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            float lo = verts[3 * i + a], hi = lo;
+#pragma unroll
+            for (int d = 16; d >= 1; d >>= 1) {
+                lo = fminf(lo, __shfl_xor_sync(FULL, lo, d));
+                hi = fmaxf(hi, __shfl_xor_sync(FULL, hi, d));
+            }
+            if ((threadIdx.x & 31) == 0) {
+                atomic_min_f(boxes + 6 * o0 + a, lo);
+                atomic_max_f(boxes + 6 * o0 + 3 + a, hi);
+            }
+        }
+        return;
+    }
+    if (o < 0) return;
     for (int a = 0; a < 3; a++) {
         atomic_min_f(boxes + 6 * o + a, verts[3 * i + a]);
         atomic_max_f(boxes + 6 * o + 3 + a, verts[3 * i + a]);
     }
 }
 
-__global__ void k_moved_list(const float* __restrict__ trans, int n_obj, int32_t* list, int32_t* count) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+// Empty boxes, and the list of the objects that move (XF: rigid transforms,
+// else translations).
+template <bool XF>
+__global__ void k_obj_init(const float* __restrict__ motion, int n_obj, float* boxes, int32_t* list, int32_t* count) {
+    chain_begin();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_obj) return;
-    const float* t = trans + 3 * i;
-    if (t[0] != 0.f || t[1] != 0.f || t[2] != 0.f) list[atomicAdd(count, 1)] = i;
+    for (int a = 0; a < 3; a++) {
+        boxes[6 * i + a] = CUDART_INF_F;
+        boxes[6 * i + 3 + a] = -CUDART_INF_F;
+    }
+    if (XF ? xform_moves(motion + 12 * i) : trans_moves(motion + 3 * i)) list[atomicAdd(count, 1)] = i;
+}
+
+// Box of every moved object (before the move), then v += t[obj].
+template <bool XF>
+__global__ void k_obj_boxes(const float* __restrict__ verts, const int32_t* __restrict__ vobj, int64_t nv,
+                            const float* __restrict__ motion, float* boxes) {
+    chain_begin();
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    int o = -1;
+    if (i < nv) {
+        o = vobj[i];
+        if (!(XF ? xform_moves(motion + 12 * o) : trans_moves(motion + 3 * o))) o = -1;
+    }
+    add_to_box(verts, i, o, boxes);
 }
 
 __global__ void k_translate(float* __restrict__ verts, const int32_t* __restrict__ vobj, int64_t nv,
                             const float* __restrict__ trans) {
+    chain_begin();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= nv * 3) return;
     const int64_t v = i / 3;
@@ -357,36 +397,11 @@ __global__ void k_translate(float* __restrict__ verts, const int32_t* __restrict
     verts[i] = __fadd_rn(verts[i], trans[3 * vobj[v] + a]);
 }
 
-// Rigid transforms, rows of [R | t] per object (12 floats).  An object is
-// moved unless its transform is exactly the identity.
-__device__ __forceinline__ bool xform_moves(const float* m) {
-    return m[0] != 1.f || m[1] != 0.f || m[2] != 0.f || m[3] != 0.f || m[4] != 0.f || m[5] != 1.f ||
-           m[6] != 0.f || m[7] != 0.f || m[8] != 0.f || m[9] != 0.f || m[10] != 1.f || m[11] != 0.f;
-}
-
-__global__ void k_moved_list_x(const float* __restrict__ xf, int n_obj, int32_t* list, int32_t* count) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_obj) return;
-    if (xform_moves(xf + 12 * i)) list[atomicAdd(count, 1)] = i;
-}
-
-// Box of every moved object before the transform.
-__global__ void k_obj_boxes_x(const float* __restrict__ verts, const int32_t* __restrict__ vobj, int64_t nv,
-                              const float* __restrict__ xf, float* boxes) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= nv) return;
-    const int o = vobj[i];
-    if (!xform_moves(xf + 12 * o)) return;
-    for (int a = 0; a < 3; a++) {
-        atomic_min_f(boxes + 6 * o + a, verts[3 * i + a]);
-        atomic_max_f(boxes + 6 * o + 3 + a, verts[3 * i + a]);
-    }
-}
-
 // v' = R v + t in fp32, each product and sum rounded in this order:
 // v'_a = ((R_a0 x + R_a1 y) + R_a2 z) + t_a  (no fused multiply-add).
 __global__ void k_transform(float* __restrict__ verts, const int32_t* __restrict__ vobj, int64_t nv,
                             const float* __restrict__ xf) {
+    chain_begin();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= nv) return;
     const float* m = xf + 12 * vobj[i];
@@ -756,7 +771,7 @@ cudaError_t launch_bvh_build(rtsdf_ctx* c) {
     }
     if ((e = cudaMemsetAsync(b.flags, 0, sizeof(uint32_t) * n, c->stream))) return e;
     const float pad = c->cfg.extent * 0x1p-16f;
-    RTSDF_LAUNCH(c, k_leaves_up, g, 256, 0, c->verts, c->tris, order, n, b.tri, b.leaf_tri, b.leaf_parent, b.nodes,
+    launch_chain(c, k_leaves_up, g, 256, 0, c->verts, c->tris, order, n, b.tri, b.leaf_tri, b.leaf_parent, b.nodes,
                  b.flags, pad, b.lbox, b.nbox);
     if (two && (e = build_top(c))) return e;
     if ((e = cudaGetLastError())) return e;
@@ -778,12 +793,12 @@ cudaError_t launch_bvh_refit(rtsdf_ctx* c) {
         // refit the objects' subtrees, then rebuild the top tree over them
         RTSDF_LAUNCH(c, k_top_detach, (unsigned)((b.top_n + 127) / 128), 128, 0, b.top_child, b.top_n, b.nodes,
                      b.leaf_parent);
-        RTSDF_LAUNCH(c, k_leaves_up, (unsigned)((n + 255) / 256), 256, 0, c->verts, c->tris, b.leaf_tri, n, b.tri,
+        launch_chain(c, k_leaves_up, (unsigned)((n + 255) / 256), 256, 0, c->verts, c->tris, b.leaf_tri, n, b.tri,
                      b.leaf_tri, b.leaf_parent, b.nodes, b.flags, pad, b.lbox, b.nbox);
         if ((e = build_top(c))) return e;
         return collapse_wide(c, nullptr);
     }
-    RTSDF_LAUNCH(c, k_leaves_up, (unsigned)((n + 255) / 256), 256, 0, c->verts, c->tris, b.leaf_tri, n, b.tri,
+    launch_chain(c, k_leaves_up, (unsigned)((n + 255) / 256), 256, 0, c->verts, c->tris, b.leaf_tri, n, b.tri,
                  b.leaf_tri, b.leaf_parent, b.nodes, b.flags, pad, b.lbox, b.nbox);
     if (b.n_wide > 0)
         RTSDF_LAUNCH(c, k_wide_boxes, (unsigned)((4 * b.n_wide + 255) / 256), 256, 0, b.wide, b.n_wide, b.nbox, b.lbox);
@@ -794,12 +809,12 @@ cudaError_t launch_move(rtsdf_ctx* c) {
     const int n_obj = c->n_obj;
     cudaError_t e = cudaMemsetAsync(c->d_moved_count, 0, sizeof(int32_t), c->stream);
     if (e != cudaSuccess) return e;
-    RTSDF_LAUNCH(c, k_obj_boxes_init, (n_obj + 127) / 128, 128, 0, c->obj_box, n_obj);
-    RTSDF_LAUNCH(c, k_moved_list, (n_obj + 127) / 128, 128, 0, c->obj_trans, n_obj, c->moved_list, c->d_moved_count);
+    launch_chain(c, k_obj_init<false>, (n_obj + 127) / 128, 128, 0, c->obj_trans, n_obj, c->obj_box, c->moved_list,
+                 c->d_moved_count);
     if (c->nv > 0) {
-        RTSDF_LAUNCH(c, k_obj_boxes, (unsigned)((c->nv + 255) / 256), 256, 0, c->verts, c->vert_obj, c->nv,
+        launch_chain(c, k_obj_boxes<false>, (unsigned)((c->nv + 255) / 256), 256, 0, c->verts, c->vert_obj, c->nv,
                      c->obj_trans, c->obj_box);
-        RTSDF_LAUNCH(c, k_translate, (unsigned)((c->nv * 3 + 255) / 256), 256, 0, c->verts, c->vert_obj, c->nv,
+        launch_chain(c, k_translate, (unsigned)((c->nv * 3 + 255) / 256), 256, 0, c->verts, c->vert_obj, c->nv,
                      c->obj_trans);
     }
     return cudaGetLastError();
@@ -809,13 +824,12 @@ cudaError_t launch_transform(rtsdf_ctx* c) {
     const int n_obj = c->n_obj;
     cudaError_t e = cudaMemsetAsync(c->d_moved_count, 0, sizeof(int32_t), c->stream);
     if (e != cudaSuccess) return e;
-    RTSDF_LAUNCH(c, k_obj_boxes_init, (n_obj + 127) / 128, 128, 0, c->obj_box, n_obj);
-    RTSDF_LAUNCH(c, k_moved_list_x, (n_obj + 127) / 128, 128, 0, c->obj_xform, n_obj, c->moved_list,
+    launch_chain(c, k_obj_init<true>, (n_obj + 127) / 128, 128, 0, c->obj_xform, n_obj, c->obj_box, c->moved_list,
                  c->d_moved_count);
     if (c->nv > 0) {
-        RTSDF_LAUNCH(c, k_obj_boxes_x, (unsigned)((c->nv + 255) / 256), 256, 0, c->verts, c->vert_obj, c->nv,
+        launch_chain(c, k_obj_boxes<true>, (unsigned)((c->nv + 255) / 256), 256, 0, c->verts, c->vert_obj, c->nv,
                      c->obj_xform, c->obj_box);
-        RTSDF_LAUNCH(c, k_transform, (unsigned)((c->nv + 255) / 256), 256, 0, c->verts, c->vert_obj, c->nv,
+        launch_chain(c, k_transform, (unsigned)((c->nv + 255) / 256), 256, 0, c->verts, c->vert_obj, c->nv,
                      c->obj_xform);
     }
     return cudaGetLastError();

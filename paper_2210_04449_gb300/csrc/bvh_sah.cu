@@ -261,6 +261,7 @@ __device__ __forceinline__ int block_excl(int v, int* s_warp, int& total) {
 
 __global__ void k_sah_root(SahTask* t, int4* chunks, uint32_t* bins, SahRange* blist, int32_t n, int blk,
                            int32_t* counters) {
+    chain_begin();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int nch = (n + SAH_CH - 1) / SAH_CH;
     if (i == 0) {
@@ -275,9 +276,13 @@ __global__ void k_sah_root(SahTask* t, int4* chunks, uint32_t* bins, SahRange* b
         r.pad[0] = r.pad[1] = 0;
         t[0] = r;
         if (n <= blk) blist[0] = SahRange{0, n, -1, 0};
-        counters[CT_BLOCKS] = n <= blk ? 1 : 0;
-        counters[CT_LEVELS] = n <= blk ? 0 : 1;
-        counters[CT_LEVELS + 1] = n <= blk ? 0 : nch;
+    }
+    if (i < CT_WORDS) {
+        int v = 0;
+        if (i == CT_BLOCKS) v = n <= blk ? 1 : 0;
+        if (i == CT_LEVELS) v = n <= blk ? 0 : 1;
+        if (i == CT_LEVELS + 1) v = n <= blk ? 0 : nch;
+        counters[i] = v;
     }
     if (n > blk) {
         if (i < nch) chunks[i] = make_int4(0, i * SAH_CH, min(SAH_CH, n - i * SAH_CH), 0);
@@ -293,6 +298,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_prims(const float* __restri
                                                            float4* __restrict__ pbox, int32_t* __restrict__ ord,
                                                            SahTask* root) {
     __shared__ float s_red[SAH_WARPS][6];
+    chain_begin();
     const int i = blockIdx.x * SAH_THREADS + threadIdx.x;
     float r[6] = {CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
     if (i < n) {
@@ -1009,13 +1015,12 @@ cudaError_t sah_topology(rtsdf_ctx* c, void* scratch, int32_t* order) {
     SahArena A;
     cudaError_t e = carve(scratch, n, A);
     if (!e) e = block_attr(c);
-    if (!e) e = cudaMemsetAsync(A.counters, 0, CT_WORDS * sizeof(int32_t), c->stream);
     if (e) return e;
     const int nch0 = (n + SAH_CH - 1) / SAH_CH;
     const int init_threads = nch0 > SAH_BIN_WORDS ? nch0 : SAH_BIN_WORDS;
-    RTSDF_LAUNCH(c, k_sah_root, (unsigned)((init_threads + 255) / 256), 256, 0, A.tasks[0], A.chunks[0], A.bins[0],
+    launch_chain(c, k_sah_root, (unsigned)((init_threads + 255) / 256), 256, 0, A.tasks[0], A.chunks[0], A.bins[0],
                  A.blist, n, blk_of(n), A.counters);
-    RTSDF_LAUNCH(c, k_sah_prims, (unsigned)((n + SAH_THREADS - 1) / SAH_THREADS), SAH_THREADS, 0, c->verts, c->tris,
+    launch_chain(c, k_sah_prims, (unsigned)((n + SAH_THREADS - 1) / SAH_THREADS), SAH_THREADS, 0, c->verts, c->tris,
                  n, A.pbox, A.ord0, A.tasks[0]);
     const Links L{bv.nodes, bv.leaf_parent, bv.root, nullptr, nullptr, nullptr};
     return run_levels(c, A, L, order, n, n > blk_of(n) ? 1 : 0, n);

@@ -48,7 +48,8 @@ constexpr float FRONT_STEP = 0.4f;   // each time no node is left to open, the b
 constexpr float FRONT_LAST = 0.3f;   // share of the unit's rays below which a node stays closed
 constexpr int UNIT_TEXELS = 32;      // texels of a unit, at most
 constexpr int UNIT_RAYS = 512;       // rays of a unit, at most (but one texel's always)
-constexpr int UNITS_PER_WARP = 8;    // units are made smaller until every warp gets this many
+constexpr int UNITS_PER_WARP = 2;    // units are made smaller until every warp gets this many (a front costs
+                                     // as much as some 30 rays: tiny frame 147 us with 8, 123 with 2)
 constexpr int FRONT_STACK = 8;       // stack entries in shared memory below a front
 
 // One warp's shared state.

@@ -23,6 +23,7 @@ constexpr int QSUB = 256;          // vertex quantisation steps per coarse voxel
 constexpr int MAX_N = 256;         // coarse voxels per axis
 constexpr int TRACE_STACK = 64;    // BVH traversal stack depth per ray
 constexpr int MAX_SHADOW_STEPS = 256;
+constexpr int FRAME_WORDS = 2;     // per-frame device counters of a context (rtsdf_ctx::d_frame_words)
 
 __host__ __device__ inline uint32_t pack_seed(uint32_t x, uint32_t y, uint32_t z) {
     return x | (y << 8) | (z << 16);
@@ -181,7 +182,8 @@ struct rtsdf_ctx {
     uint32_t* counts = nullptr;
     float* fine = nullptr;
     uint32_t* masked = nullptr;   // masked coarse voxels
-    uint32_t* d_masked_count = nullptr;
+    uint64_t* d_frame_words = nullptr;    // [FRAME_WORDS] cleared per frame: masked count, next ray
+    uint32_t* d_masked_count = nullptr;   // in d_frame_words
     int64_t last_masked = -1;
 
     // tracer scratch: per texel slot (8 per masked voxel) this frame's
@@ -189,7 +191,7 @@ struct rtsdf_ctx {
     // hit counts; cleared again by the finalize kernel
     uint32_t* ray_min = nullptr;
     uint32_t* ray_cnt = nullptr;
-    unsigned long long* d_next_ray = nullptr;
+    unsigned long long* d_next_ray = nullptr;   // in d_frame_words
     unsigned trace_grid = 0;
 
     // launch parameters (rtsdf_set_tuning / rtsdf_autotune)
@@ -225,10 +227,13 @@ namespace rtsdf {
 // visible (which has waited the same way, and so on back), and only then lets
 // the next one be launched, so that at most two kernels of a chain overlap and
 // none is started before all but its direct predecessor have ended.  Without
-// the attribute, or as the first of a chain, the wait is over at once.
+// the attribute, or as the first of a chain, the wait is over at once.  A
+// kernel that fills the GPU for long only waits (chain_wait()): the next one's
+// blocks would take places from its own.
 #ifdef __CUDACC__
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_begin() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    chain_wait();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 #endif

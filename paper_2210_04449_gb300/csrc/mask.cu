@@ -182,6 +182,7 @@ __device__ __forceinline__ bool near_moved_box(const MaskArgs& a, int cx, int cy
 }
 
 __global__ void __launch_bounds__(256) k_mask(MaskArgs a) {
+    chain_begin();
     const int n = a.nc;
     const int x = blockIdx.x * 32 + threadIdx.x;
     const int y = blockIdx.y * 8 + threadIdx.y;
@@ -263,7 +264,8 @@ __global__ void __launch_bounds__(256) k_mask(MaskArgs a) {
 
 cudaError_t launch_mask(rtsdf_ctx* c, float d_vox) {
     const int n = c->nc;
-    cudaError_t e = cudaMemsetAsync(c->d_masked_count, 0, sizeof(uint32_t), c->stream);
+    // the masked count and the tracer's ray counter (adjacent words)
+    cudaError_t e = cudaMemsetAsync(c->d_frame_words, 0, FRAME_WORDS * sizeof(uint64_t), c->stream);
     if (e != cudaSuccess) return e;
     MaskArgs a;
     a.seeds = c->seeds[c->cur];
@@ -315,7 +317,7 @@ cudaError_t launch_mask(rtsdf_ctx* c, float d_vox) {
         RTSDF_LAUNCH(c, k_bin_fill, gb, 128, 0, b);
     }
     dim3 block(32, 8, 1), grid((n + 31) / 32, (n + 7) / 8, n);
-    RTSDF_LAUNCH(c, k_mask, grid, block, 0, a);
+    launch_chain(c, k_mask, grid, block, 0, a);
     c->reset_pending = false;
     return cudaGetLastError();
 }

@@ -67,6 +67,7 @@ template <bool COUNT, bool TEX>
 __global__ void __launch_bounds__(TRACE_THREADS, TRACE_MIN_BLOCKS) k_trace(TraceArgs a) {
     __shared__ BlockTrace s_trace;
     __shared__ TraceArgs s_args;   // for the parts that are called
+    chain_wait();
     if (threadIdx.x == 0) s_args = a;
     __syncthreads();
     SceneUnits src{s_args, (unsigned long long)(*a.count) * 8u * (unsigned long long)a.rays};
@@ -77,6 +78,7 @@ __global__ void __launch_bounds__(TRACE_THREADS, TRACE_MIN_BLOCKS) k_trace(Trace
 // Eq. 1 per traced texel slot (see finalize_slot): a grid-stride loop over
 // the frame's slots (8 per masked voxel, a count known only on the device).
 __global__ void __launch_bounds__(256) k_trace_finalize(TraceArgs a) {
+    chain_begin();
     const uint64_t n = (uint64_t)(*a.count) * 8u;
     const uint64_t stride = gridDim.x * (uint64_t)blockDim.x;
     for (uint64_t s = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; s < n; s += stride) finalize_slot(a, s);
@@ -122,8 +124,7 @@ cudaError_t launch_trace(rtsdf_ctx* c, int rays, int frame) {
     a.leaf_min = c->tune.leaf_min;
     a.nc_mag = (uint32_t)((0x100000000ull + (unsigned long long)c->nc - 1) / (unsigned long long)c->nc);
     a.nearest = c->sign_mode == RTSDF_SIGN_NEAREST;
-    cudaError_t e = cudaMemsetAsync(c->d_next_ray, 0, sizeof(unsigned long long), c->stream);
-    if (e != cudaSuccess) return e;
+    // (the mask stage has cleared the ray counter)
     {
         int sms = 0, per_sm = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
@@ -136,11 +137,11 @@ cudaError_t launch_trace(rtsdf_ctx* c, int rays, int frame) {
     }
     // the texture path when the node texture exists (plain loads otherwise)
     if (a.wtex) {
-        if (c->counting) RTSDF_LAUNCH(c, (k_trace<true, true>), c->trace_grid, TRACE_THREADS, 0, a);
-        else RTSDF_LAUNCH(c, (k_trace<false, true>), c->trace_grid, TRACE_THREADS, 0, a);
+        if (c->counting) launch_chain(c, k_trace<true, true>, c->trace_grid, TRACE_THREADS, 0, a);
+        else launch_chain(c, k_trace<false, true>, c->trace_grid, TRACE_THREADS, 0, a);
     } else {
-        if (c->counting) RTSDF_LAUNCH(c, (k_trace<true, false>), c->trace_grid, TRACE_THREADS, 0, a);
-        else RTSDF_LAUNCH(c, (k_trace<false, false>), c->trace_grid, TRACE_THREADS, 0, a);
+        if (c->counting) launch_chain(c, k_trace<true, false>, c->trace_grid, TRACE_THREADS, 0, a);
+        else launch_chain(c, k_trace<false, false>, c->trace_grid, TRACE_THREADS, 0, a);
     }
     // the slot count is on the device: enough blocks to fill every SM
     // (8 x 256 threads each), capped by the largest possible slot count
@@ -149,7 +150,7 @@ cudaError_t launch_trace(rtsdf_ctx* c, int rays, int frame) {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
         const uint64_t most = (8 * (uint64_t)c->nc3 + 255) / 256;
         const uint64_t want = (uint64_t)(sms > 0 ? sms : 132) * 8u;
-        RTSDF_LAUNCH(c, k_trace_finalize, (unsigned)(most < want ? most : want), 256, 0, a);
+        launch_chain(c, k_trace_finalize, (unsigned)(most < want ? most : want), 256, 0, a);
     }
     return cudaGetLastError();
 }

@@ -25,6 +25,7 @@ using namespace dev;
 
 __global__ void k_quantise(const float* __restrict__ verts, int64_t nv, float bx, float by, float bz,
                            float scale, int n, int32_t* __restrict__ q, uint32_t* err) {
+    chain_begin();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= nv * 3) return;
     const int a = (int)(i % 3);
@@ -50,11 +51,22 @@ __global__ void k_validate_tris(int32_t* __restrict__ tris, int64_t nt, int64_t 
     }
 }
 
+// Seed grid to "no seed" and the list of large triangles to empty.
+__global__ void __launch_bounds__(256) k_vox_clear(uint32_t* __restrict__ seeds, size_t n3, uint32_t* big_count) {
+    chain_begin();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *big_count = 0u;
+    const size_t stride = (size_t)gridDim.x * blockDim.x, i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    const uint4 none = make_uint4(SEED_EMPTY, SEED_EMPTY, SEED_EMPTY, SEED_EMPTY);
+    for (size_t i = i0; i < n3 / 4; i += stride) reinterpret_cast<uint4*>(seeds)[i] = none;
+    if (i0 < n3 % 4) seeds[n3 - 1 - i0] = SEED_EMPTY;
+}
+
 __global__ void __launch_bounds__(128) k_voxelize_small(const int32_t* __restrict__ q,
                                                        const int32_t* __restrict__ tris, int64_t nt,
                                                        int n, uint32_t* __restrict__ seeds,
                                                        int32_t* __restrict__ big_list,
                                                        uint32_t* __restrict__ big_count) {
+    chain_begin();
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= nt) return;
     TriAxes s;
@@ -80,6 +92,7 @@ __global__ void __launch_bounds__(256) k_voxelize_big(const int32_t* __restrict_
                                                      const int32_t* __restrict__ big_list,
                                                      const uint32_t* __restrict__ big_count, int n,
                                                      uint32_t* __restrict__ seeds) {
+    chain_begin();
     const uint32_t nb = *big_count;
     for (uint32_t b = blockIdx.x; b < nb; b += gridDim.x) {
         TriAxes s;
@@ -101,7 +114,7 @@ cudaError_t launch_quantise(rtsdf_ctx* c) {
     if (c->nv == 0) return cudaSuccess;
     const float scale = (float)(c->nc * QSUB) / c->cfg.extent;
     int64_t m = c->nv * 3;
-    RTSDF_LAUNCH(c, k_quantise, (unsigned)((m + 255) / 256), 256, 0, c->verts, c->nv, c->cfg.bmin[0],
+    launch_chain(c, k_quantise, (unsigned)((m + 255) / 256), 256, 0, c->verts, c->nv, c->cfg.bmin[0],
                  c->cfg.bmin[1], c->cfg.bmin[2], scale, c->nc, c->qverts, c->d_err);
     return cudaGetLastError();
 }
@@ -114,18 +127,17 @@ cudaError_t launch_validate_tris(rtsdf_ctx* c) {
 }
 
 cudaError_t launch_voxelize(rtsdf_ctx* c) {
-    cudaError_t e = cudaMemsetAsync(c->seeds[0], 0xFF, c->nc3 * sizeof(uint32_t), c->stream);
-    if (e != cudaSuccess) return e;
     c->cur = 0;
-    if (c->nt == 0) return cudaSuccess;
-    e = cudaMemsetAsync(c->d_big_count, 0, sizeof(uint32_t), c->stream);
-    if (e != cudaSuccess) return e;
-    RTSDF_LAUNCH(c, k_voxelize_small, (unsigned)((c->nt + 127) / 128), 128, 0, c->qverts, c->tris, c->nt,
-                 c->nc, c->seeds[0], c->big_list, c->d_big_count);
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    RTSDF_LAUNCH(c, k_voxelize_big, (unsigned)(sms > 0 ? sms * 4 : 512), 256, 0, c->qverts, c->tris,
-                 c->big_list, c->d_big_count, c->nc, c->seeds[0]);
+    const size_t fill = (c->nc3 / 4 + 255) / 256, most = (size_t)(sms > 0 ? sms : 132) * 8;
+    launch_chain(c, k_vox_clear, (unsigned)(fill < 1 ? 1 : (fill < most ? fill : most)), 256, 0, c->seeds[0], c->nc3,
+                 c->d_big_count);
+    if (c->nt == 0) return cudaGetLastError();
+    launch_chain(c, k_voxelize_small, (unsigned)((c->nt + 127) / 128), 128, 0, c->qverts, c->tris, c->nt, c->nc,
+                 c->seeds[0], c->big_list, c->d_big_count);
+    launch_chain(c, k_voxelize_big, (unsigned)(sms > 0 ? sms * 4 : 512), 256, 0, c->qverts, c->tris, c->big_list,
+                 c->d_big_count, c->nc, c->seeds[0]);
     return cudaGetLastError();
 }
 
