@@ -53,7 +53,7 @@ void launch_pass(rtsdf_ctx* c, const uint32_t* in, uint32_t* out, int n, int k, 
 
 // z-blocked pass (dev::jfa_zblock_column): blocks of 32 x 4 threads in
 // (x, y), blockIdx.z = g k + rz.
-template <bool FINAL, int T>
+template <bool FINAL, int T, bool AHEAD>
 __global__ void __launch_bounds__(128, 4) k_jfa_zblock(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
                                                       int n, int k, float* __restrict__ coarse, float hc,
                                                       float beta_h) {
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(128, 4) k_jfa_zblock(const uint32_t* __restric
     const int y = blockIdx.y * 4 + threadIdx.y;
     const int rz = (int)(blockIdx.z % (unsigned)k), g = (int)(blockIdx.z / (unsigned)k);
     if (x >= n || y >= n) return;
-    dev::jfa_zblock_column<FINAL, T>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
+    dev::jfa_zblock_column<FINAL, T, AHEAD>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
 }
 
 // Columns below which shorter ones are taken: a thread floods its column
@@ -70,14 +70,19 @@ __global__ void __launch_bounds__(128, 4) k_jfa_zblock(const uint32_t* __restric
 // (38.0 with 50,000 columns, but 75^3 66.9 instead of 64.9); from 96^3 on, more
 // columns cost more than they hide (98 instead of 88 us at 96^3 with 400,000).
 constexpr int64_t JFA_COLUMNS = 100000;
+// Columns of 16 where there are enough of them: 256^3 1237 -> 1208 us (128^3,
+// with fewer: 139 -> 144).
+constexpr int64_t JFA_COLUMNS_16 = 400000;
+// Largest grid whose slices are read ahead (see jfa_zblock_column).
+constexpr int JFA_AHEAD_N = 64;
 
-template <int T>
+template <int T, bool AHEAD>
 void launch_zblock(rtsdf_ctx* c, const uint32_t* in, uint32_t* out, int n, int k, bool final, float beta_h) {
     const int lat = (n + k - 1) / k;          // z-lattice members of the fullest residue class
     const int groups = (lat + T - 1) / T;
     dim3 block(32, 4, 1), grid((n + 31) / 32, (n + 3) / 4, (unsigned)(groups * k));
-    if (final) launch_chain(c, k_jfa_zblock<true, T>, grid, block, 0, in, out, n, k, c->coarse, c->hc, beta_h);
-    else launch_chain(c, k_jfa_zblock<false, T>, grid, block, 0, in, out, n, k, c->coarse, c->hc, beta_h);
+    if (final) launch_chain(c, k_jfa_zblock<true, T, AHEAD>, grid, block, 0, in, out, n, k, c->coarse, c->hc, beta_h);
+    else launch_chain(c, k_jfa_zblock<false, T, AHEAD>, grid, block, 0, in, out, n, k, c->coarse, c->hc, beta_h);
 }
 
 // Coarse SDF without a pass (N = 1: no jump steps).
@@ -107,15 +112,22 @@ cudaError_t launch_jfa(rtsdf_ctx* c) {
             case 2: launch_pass<128, 2>(c, in, out, n, k, k == 1, beta_h); break;
             case 3: launch_pass<32, 4>(c, in, out, n, k, k == 1, beta_h); break;
             case 4: {
-                // columns of up to 8 voxels, shorter where the lattice is or
+                // columns of up to 16 voxels, shorter where the lattice is or
                 // where the columns would be too few to fill the GPU
                 const int lat = (n + k - 1) / k;
                 const int64_t cols = (int64_t)n * n * k;
-                int t = 8;
+                int t = cols * ((lat + 15) / 16) >= JFA_COLUMNS_16 ? 16 : 8;
                 while (t > 2 && (t / 2 >= lat || cols * ((lat + t - 1) / t) < JFA_COLUMNS)) t /= 2;
-                if (t == 2) launch_zblock<2>(c, in, out, n, k, k == 1, beta_h);
-                else if (t == 4) launch_zblock<4>(c, in, out, n, k, k == 1, beta_h);
-                else launch_zblock<8>(c, in, out, n, k, k == 1, beta_h);
+                const bool last = k == 1;
+                if (n <= JFA_AHEAD_N) {
+                    if (t == 2) launch_zblock<2, true>(c, in, out, n, k, last, beta_h);
+                    else launch_zblock<4, true>(c, in, out, n, k, last, beta_h);
+                } else {
+                    if (t == 2) launch_zblock<2, false>(c, in, out, n, k, last, beta_h);
+                    else if (t == 4) launch_zblock<4, false>(c, in, out, n, k, last, beta_h);
+                    else if (t == 8) launch_zblock<8, false>(c, in, out, n, k, last, beta_h);
+                    else launch_zblock<16, false>(c, in, out, n, k, last, beta_h);
+                }
                 break;
             }
             default: launch_pass<32, 8>(c, in, out, n, k, k == 1, beta_h); break;

@@ -76,12 +76,12 @@ __device__ __forceinline__ void jfa_voxel(const uint32_t* __restrict__ in, uint3
 // each) are read once and shared by the column's voxels.
 //
 // Per candidate seed s = (sx, sy, sz, 0) of a slice, once:
-//   A = (sx - x)^2 + (sy - y)^2 + sz^2            vabsdiff4 + dp4a, whose
-//       accumulator adds s's top byte (as 0x7F000000): a seedless candidate
-//       (all ones) lands above every real key
+//   A = s.s - 2 (x sx + y sy)                     dp4a, whose accumulator
+//       adds s's top byte (as 0x7F000000: a seedless candidate, all ones, lands
+//       above every real key), and dp2a.lo (16-bit -2 x, -2 y times bytes 0, 1)
 // Per voxel z_t and candidate, one instruction:
-//   key = A - 2 z_t sz = D2 - z_t^2               dp2a.hi (16-bit -2 z_t times byte 2)
-// Keys of one voxel share the z_t^2 offset, so their order is D2's; the
+//   key = A - 2 z_t sz = D2 - v.v                 dp2a.hi (16-bit -2 z_t times byte 2)
+// Keys of one voxel share the v.v offset, so their order is D2's; the
 // arg-min is the smallest key (three-input signed minima), then the smallest
 // seed among the candidates at that key (one clamped add-min and one
 // multiply-add per candidate, then unsigned minima) -- the lexicographic
@@ -89,19 +89,30 @@ __device__ __forceinline__ void jfa_voxel(const uint32_t* __restrict__ in, uint3
 // coordinate on that axis (a duplicate of another candidate); a z-slice
 // outside the grid holds no seed.  Slices roll through registers: voxel t
 // needs slices t .. t + 2 only.
+// AHEAD hides a slice's load latency where few warps do (32^3: 12.0 -> 9.4 us,
+// 61^3: 28.4 -> 25.8); with the registers it takes, large grids are slower with
+// it (200^3: 629 -> 683 us).  Tried: keys as whole numbers in fp32, three
+// multiply-adds at the full rate for the two dot products and the clamped add
+// (256^3: 1533 instead of 1237 us: 128 registers).
 __device__ __forceinline__ int dp2a_hi_s_u(uint32_t a, uint32_t b, int c) {
     int d;
     asm("dp2a.hi.s32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
     return d;
 }
 
+__device__ __forceinline__ int dp2a_lo_s_u(uint32_t a, uint32_t b, int c) {
+    int d;
+    asm("dp2a.lo.s32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+
 __device__ __forceinline__ int vimin3_s(int a, int b, int c) { return __vimin3_s32(a, b, c); }
 
-// the smallest key a seedless candidate can have: A >= 0x7F000000, minus
-// 2 z sz with z, sz <= 255
+// the smallest key a seedless candidate can have: 0x7F000000 + 4 255^2, minus
+// 2 255 (x + y + z) with x, y, z <= 255
 constexpr int SEEDLESS_KEY_MIN = 0x7F000000 - 2 * 255 * 255;
 
-template <bool FINAL, int T>
+template <bool FINAL, int T, bool AHEAD>
 __device__ __forceinline__ void jfa_zblock_column(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
                                                   int n, int k, int x, int y, int rz, int g,
                                                   float* __restrict__ coarse, float hc, float beta_h) {
@@ -113,10 +124,15 @@ __device__ __forceinline__ void jfa_zblock_column(const uint32_t* __restrict__ i
         xs[i] = (uint32_t)((x + o >= 0 && x + o < n) ? x + o : x);
         ys[i] = (uint32_t)((y + o >= 0 && y + o < n) ? y + o : y) * (uint32_t)n;
     }
-    const uint32_t vxy = (uint32_t)x | ((uint32_t)y << 8);
+    const uint32_t wxy = ((uint32_t)(-2 * x) & 0xFFFFu) | ((uint32_t)(-2 * y) << 16);
+    const int vv = x * x + y * y;
     // slice j (0 .. T + 1) holds z-lattice index T g + j - 1
     uint32_t ss[T + 2][9];
     int aa[T + 2][9];
+    auto take = [&](int j, int c, uint32_t sv) {
+        ss[j][c] = sv;
+        aa[j][c] = dp2a_lo_s_u(wxy, sv, (int)__dp4a(sv, sv, sv & 0x7F000000u));
+    };
     auto load_slice = [&](int j) {
         const int z = rz + k * (T * g + j - 1);
         if (z >= 0 && z < n) {
@@ -124,12 +140,7 @@ __device__ __forceinline__ void jfa_zblock_column(const uint32_t* __restrict__ i
 #pragma unroll
             for (int iy = 0; iy < 3; iy++)
 #pragma unroll
-                for (int ix = 0; ix < 3; ix++) {
-                    const uint32_t sv = __ldg(in + zo + ys[iy] + xs[ix]);
-                    const uint32_t d = __vabsdiffu4(sv, vxy);
-                    ss[j][3 * iy + ix] = sv;
-                    aa[j][3 * iy + ix] = (int)__dp4a(d, d, sv & 0x7F000000u);
-                }
+                for (int ix = 0; ix < 3; ix++) take(j, 3 * iy + ix, __ldg(in + zo + ys[iy] + xs[ix]));
         } else {
 #pragma unroll
             for (int c = 0; c < 9; c++) {
@@ -138,13 +149,38 @@ __device__ __forceinline__ void jfa_zblock_column(const uint32_t* __restrict__ i
             }
         }
     };
-    load_slice(0);
-    load_slice(1);
+    // AHEAD: the seeds of a slice without a branch, read one step before use
+    uint32_t nx[9];
+    auto fetch = [&](int j) {
+        const int z = rz + k * (T * g + j - 1);
+        const bool in_grid = z >= 0 && z < n;
+        const uint32_t* p = in + (uint32_t)(in_grid ? z : 0) * n2;
+#pragma unroll
+        for (int iy = 0; iy < 3; iy++)
+#pragma unroll
+            for (int ix = 0; ix < 3; ix++) nx[3 * iy + ix] = in_grid ? __ldg(p + (ys[iy] + xs[ix])) : SEED_EMPTY;
+    };
+    auto take_slice = [&](int j) {
+#pragma unroll
+        for (int c = 0; c < 9; c++) take(j, c, nx[c]);
+    };
+    if (AHEAD) {
+        fetch(0);
+        take_slice(0);
+        fetch(1);
+        take_slice(1);
+        fetch(2);
+    } else {
+        load_slice(0);
+        load_slice(1);
+    }
 #pragma unroll
     for (int t = 0; t < T; t++) {
-        load_slice(t + 2);
+        if (AHEAD) take_slice(t + 2);
+        else load_slice(t + 2);
         const int z = rz + k * (T * g + t);
         if (z >= n) break;
+        if (AHEAD && t + 1 < T) fetch(t + 3);
         // 16-bit -2 z in the low half, 0 in the high half (byte 3 is 0 or, for
         // a seedless candidate, already pushed out of range through A)
         const uint32_t wz = (uint32_t)(-2 * z) & 0xFFFFu;
@@ -175,7 +211,7 @@ __device__ __forceinline__ void jfa_zblock_column(const uint32_t* __restrict__ i
         const uint32_t best = kmin >= SEEDLESS_KEY_MIN ? SEED_EMPTY : vmin;
         const uint32_t idx = (uint32_t)x + ys[1] + (uint32_t)z * n2;
         out[idx] = best;
-        if (FINAL) coarse[idx] = dev::coarse_value(best, (uint32_t)(kmin + z * z), hc, beta_h);
+        if (FINAL) coarse[idx] = dev::coarse_value(best, (uint32_t)(kmin + vv + z * z), hc, beta_h);
     }
 }
 
