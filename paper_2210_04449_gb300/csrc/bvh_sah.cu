@@ -14,10 +14,10 @@
 // Three tiers by range size m (blk: 256, or 1024 for large meshes):
 //  * m > blk: level-synchronous over chunks of SAH_CH positions, the levels'
 //    sizes kept on the device so that no level waits for the host.
-//    k_sah_bin bins a chunk in shared memory and merges into the range's
-//    bins with global atomics (and keeps the chunk's histogram);
-//    k_sah_split (a warp per range) picks the split and every chunk's output
-//    offset; k_sah_partition scatters stably into the other order buffer.
+//    k_sah_split bins a chunk in shared memory and merges into the range's
+//    bins with global atomics (and keeps the chunk's histogram); the block
+//    that finishes a range picks the split and every chunk's output offset;
+//    k_sah_partition scatters stably into the other order buffer.
 //  * 32 < m <= blk: one block per range (k_sah_block), boxes in shared
 //    memory, the same binned split down to ranges of 32;
 //  * 2 <= m <= 32: one warp per range, the exact heuristic over every split
@@ -55,9 +55,9 @@ static_assert(SAH_ITEMS * SAH_THREADS == SAH_CH, "one chunk per block pass");
 // another, so a small mesh, whose few ranges leave most SMs idle, is split
 // further by the levels (each of which costs three launches).  Whole build
 // with 256 against 1024: 2.2k triangles 403 / 505 us, 104k 908 / 1270 us, 1M
-// 2587 / 2389 us (300k: 1103 / 1166 us).
+// 2587 / 2389 us (300k: 1170 / 1119 us).
 constexpr int SAH_BLK_SMALL = 256;
-constexpr int64_t SAH_SMALL_MESH = 400000;
+constexpr int64_t SAH_SMALL_MESH = 200000;
 __host__ __device__ constexpr int blk_of(int64_t n) { return n <= SAH_SMALL_MESH ? SAH_BLK_SMALL : SAH_CH; }
 
 // Device-side counters of a build: block ranges listed, a capacity guard that
@@ -124,69 +124,75 @@ struct Choice {
     int axis, split, nl;   // axis -1: no axis separates the range
 };
 
-// Lane l reads bin l of each axis; the split after bin l puts bins 0..l left.
-// Ties go to the smaller bin, then the smaller axis.  All 32 lanes call.
-__device__ Choice warp_choose(const uint32_t* bins, int lane) {
-    Choice best{CUDART_INF_F, -1, -1, 0};
-    for (int a = 0; a < 3; a++) {
-        const uint32_t* p = bins + (a * NB + lane) * BW;
-        const uint32_t cnt = p[0];
-        float plo[3], phi[3], slo[3], shi[3];
+// Lane l reads bin l of axis a; the split after bin l puts bins 0..l left.
+// Ties go to the smaller bin.  All 32 lanes call.
+__device__ Choice axis_choose(const uint32_t* bins, int a, int lane) {
+    const uint32_t* p = bins + (a * NB + lane) * BW;
+    const uint32_t cnt = p[0];
+    float plo[3], phi[3], slo[3], shi[3];
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        plo[k] = slo[k] = cnt ? o2f(p[1 + k]) : CUDART_INF_F;
+        phi[k] = shi[k] = cnt ? o2f(p[4 + k]) : -CUDART_INF_F;
+    }
+    uint32_t pc = cnt, sc = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t up = __shfl_up_sync(FULL, pc, o), dn = __shfl_down_sync(FULL, sc, o);
 #pragma unroll
         for (int k = 0; k < 3; k++) {
-            plo[k] = slo[k] = cnt ? o2f(p[1 + k]) : CUDART_INF_F;
-            phi[k] = shi[k] = cnt ? o2f(p[4 + k]) : -CUDART_INF_F;
-        }
-        uint32_t pc = cnt, sc = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t up = __shfl_up_sync(FULL, pc, o), dn = __shfl_down_sync(FULL, sc, o);
-#pragma unroll
-            for (int k = 0; k < 3; k++) {
-                const float ul = __shfl_up_sync(FULL, plo[k], o), uh = __shfl_up_sync(FULL, phi[k], o);
-                const float dl = __shfl_down_sync(FULL, slo[k], o), dh = __shfl_down_sync(FULL, shi[k], o);
-                if (lane >= o) {
-                    plo[k] = fminf(plo[k], ul);
-                    phi[k] = fmaxf(phi[k], uh);
-                }
-                if (lane + o < 32) {
-                    slo[k] = fminf(slo[k], dl);
-                    shi[k] = fmaxf(shi[k], dh);
-                }
+            const float ul = __shfl_up_sync(FULL, plo[k], o), uh = __shfl_up_sync(FULL, phi[k], o);
+            const float dl = __shfl_down_sync(FULL, slo[k], o), dh = __shfl_down_sync(FULL, shi[k], o);
+            if (lane >= o) {
+                plo[k] = fminf(plo[k], ul);
+                phi[k] = fmaxf(phi[k], uh);
             }
-            if (lane >= o) pc += up;
-            if (lane + o < 32) sc += dn;
-        }
-        // right side of the split after bin `lane`: the suffix from lane + 1
-        const uint32_t rc = __shfl_down_sync(FULL, sc, 1);
-        float rlo[3], rhi[3];
-#pragma unroll
-        for (int k = 0; k < 3; k++) {
-            rlo[k] = __shfl_down_sync(FULL, slo[k], 1);
-            rhi[k] = __shfl_down_sync(FULL, shi[k], 1);
-        }
-        float cost = CUDART_INF_F;
-        if (lane < NB - 1 && pc > 0 && rc > 0)
-            cost = half_area3(plo, phi) * (float)pc + half_area3(rlo, rhi) * (float)rc;
-        float bc = cost;
-        int bl = lane;
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) {
-            const float c2 = __shfl_xor_sync(FULL, bc, o);
-            const int l2 = __shfl_xor_sync(FULL, bl, o);
-            if (c2 < bc || (c2 == bc && l2 < bl)) {
-                bc = c2;
-                bl = l2;
+            if (lane + o < 32) {
+                slo[k] = fminf(slo[k], dl);
+                shi[k] = fmaxf(shi[k], dh);
             }
         }
-        const uint32_t nl = __shfl_sync(FULL, pc, bl);
-        if (bc < best.cost) {
-            best.cost = bc;
-            best.axis = a;
-            best.split = bl + 1;
-            best.nl = (int)nl;
+        if (lane >= o) pc += up;
+        if (lane + o < 32) sc += dn;
+    }
+    // right side of the split after bin `lane`: the suffix from lane + 1
+    const uint32_t rc = __shfl_down_sync(FULL, sc, 1);
+    float rlo[3], rhi[3];
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        rlo[k] = __shfl_down_sync(FULL, slo[k], 1);
+        rhi[k] = __shfl_down_sync(FULL, shi[k], 1);
+    }
+    float cost = CUDART_INF_F;
+    if (lane < NB - 1 && pc > 0 && rc > 0)
+        cost = half_area3(plo, phi) * (float)pc + half_area3(rlo, rhi) * (float)rc;
+    float bc = cost;
+    int bl = lane;
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+        const float c2 = __shfl_xor_sync(FULL, bc, o);
+        const int l2 = __shfl_xor_sync(FULL, bl, o);
+        if (c2 < bc || (c2 == bc && l2 < bl)) {
+            bc = c2;
+            bl = l2;
         }
     }
+    const uint32_t nl = __shfl_sync(FULL, pc, bl);
+    return bc < CUDART_INF_F ? Choice{bc, a, bl + 1, (int)nl} : Choice{CUDART_INF_F, -1, -1, 0};
+}
+
+// The cheapest of the three axes' splits (ties: the smaller axis); three warps
+// of the block find them side by side.  Every thread of the block calls.
+__device__ __forceinline__ Choice block_choose(const uint32_t* bins, Choice* s_axis) {
+    const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
+    if (warp < 3) {
+        const Choice c = axis_choose(bins, warp, lane);
+        if (lane == 0) s_axis[warp] = c;
+    }
+    __syncthreads();
+    Choice best = s_axis[0];
+    if (s_axis[1].cost < best.cost) best = s_axis[1];
+    if (s_axis[2].cost < best.cost) best = s_axis[2];
     return best;
 }
 
@@ -389,18 +395,25 @@ __global__ void k_sah_top_single(const int32_t* child_of, BNode* nodes, int32_t*
 
 // ------------------------------------------------------------- big ranges
 
-__global__ void __launch_bounds__(SAH_THREADS) k_sah_bin(const int4* __restrict__ chunks,
-                                                         const SahTask* __restrict__ tasks,
-                                                         const int32_t* __restrict__ ord0,
-                                                         const int32_t* __restrict__ ord1,
-                                                         const float4* __restrict__ pbox, uint32_t* bins,
-                                                         uint32_t* __restrict__ hist,
-                                                         const int32_t* counters, int lev) {
+// One block per chunk bins it; the block that finishes a range's last chunk
+// then splits the range: split choice, node links, chunk output offsets, and
+// the children (leaf, block range or next-level big range).
+__global__ void __launch_bounds__(SAH_THREADS) k_sah_split(const int4* chunks, SahTask* tasks,
+                                                           const int32_t* __restrict__ ord0,
+                                                           const int32_t* __restrict__ ord1,
+                                                           const float4* __restrict__ pbox, uint32_t* bins,
+                                                           uint32_t* hist, int32_t* __restrict__ left_off, Links L,
+                                                           SahTask* next, int4* next_chunks, uint32_t* next_bins,
+                                                           SahRange* blist, int32_t* counters, int lev,
+                                                           int32_t cap_task, int32_t cap_chunk, int32_t cap_blist,
+                                                           int blk) {
     __shared__ uint32_t sb[SAH_BIN_WORDS];
+    __shared__ Choice s_axis[3];
+    __shared__ int s_last;
     chain_begin();
     if ((int)blockIdx.x >= counters[lev + 1] || counters[CT_BAD]) return;
-    const int4 ch = chunks[blockIdx.x];        // (task, start, length)
-    const SahTask& T = tasks[ch.x];
+    const int4 chunk = chunks[blockIdx.x];     // (task, start, length)
+    SahTask& T = tasks[chunk.x];
     for (int i = threadIdx.x; i < SAH_BIN_WORDS; i += SAH_THREADS) sb[i] = bin_init(i);
     float clo[3], chi[3];
 #pragma unroll
@@ -411,8 +424,8 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_bin(const int4* __restrict_
     const BinMap m = bin_map(clo, chi);
     const int32_t* ord = T.buf ? ord1 : ord0;
     __syncthreads();
-    for (int i = threadIdx.x; i < ch.z; i += SAH_THREADS) {
-        const int32_t t = ord[ch.y + i];
+    for (int i = threadIdx.x; i < chunk.z; i += SAH_THREADS) {
+        const int32_t t = ord[chunk.y + i];
         const float4 lo = pbox[2 * (int64_t)t], hi = pbox[2 * (int64_t)t + 1];
         const float l[3] = {lo.x, lo.y, lo.z}, h[3] = {hi.x, hi.y, hi.z};
 #pragma unroll
@@ -427,35 +440,30 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_bin(const int4* __restrict_
         }
     }
     __syncthreads();
-    uint32_t* gb = bins + (size_t)ch.x * SAH_BIN_WORDS;
+    uint32_t* gb = bins + (size_t)chunk.x * SAH_BIN_WORDS;
     for (int i = threadIdx.x; i < SAH_BIN_WORDS; i += SAH_THREADS) {
         const int w = i % BW;
         const uint32_t cnt = sb[i - w];
-        if (w == 0) hist[(size_t)blockIdx.x * 3 * NB + i / BW] = cnt;
+        if (w == 0) __stcg(hist + (size_t)blockIdx.x * 3 * NB + i / BW, cnt);
         if (cnt == 0) continue;
         if (w == 0) atomicAdd(gb + i, cnt);
         else if (w < 4) atomicMin(gb + i, sb[i]);
         else atomicMax(gb + i, sb[i]);
     }
-}
-
-// One warp per big range: split choice, node links, chunk output offsets,
-// and the children (leaf, block range or next-level big range).
-__global__ void __launch_bounds__(SAH_THREADS) k_sah_split(SahTask* tasks, int lev, const uint32_t* bins,
-                                                           const uint32_t* __restrict__ hist,
-                                                           const int4* __restrict__ chunks,
-                                                           int32_t* __restrict__ left_off, Links L, SahTask* next,
-                                                           int4* next_chunks, uint32_t* next_bins, SahRange* blist,
-                                                           int32_t* counters, int32_t cap_task, int32_t cap_chunk,
-                                                           int32_t cap_blist, int blk) {
-    chain_begin();
-    const int w = (int)((blockIdx.x * (unsigned)SAH_THREADS + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (w >= counters[lev] || counters[CT_BAD]) return;   // warp-uniform
-    SahTask& T = tasks[w];
-    const int b = T.b, e = T.e, m = e - b;
-    const Choice ch = warp_choose(bins + (size_t)w * SAH_BIN_WORDS, lane);
-    const int nl = ch.axis < 0 ? m / 2 : ch.nl;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&T.pad[0], 1) == T.nchunk - 1;
+    __syncthreads();
+    if (!s_last) return;
+    // every chunk of the range is binned: its bins and histograms come from L2
+    __threadfence();
+    for (int i = threadIdx.x; i < SAH_BIN_WORDS; i += SAH_THREADS) sb[i] = __ldcg(gb + i);
+    __syncthreads();
+    const Choice ch = block_choose(sb, s_axis);
+    if (threadIdx.x >= 32) return;
+    const int lane = (int)threadIdx.x;
+    const int b = T.b, e = T.e, msz = e - b;
+    const int nl = ch.axis < 0 ? msz / 2 : ch.nl;
     // left items before each chunk (chunks of a range are in position order)
     int carry = 0;
     for (int k0 = 0; k0 < T.nchunk; k0 += 32) {
@@ -467,7 +475,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_split(SahTask* tasks, int l
                 lc = min(max(nl - (cr.y - b), 0), cr.z);
             } else {
                 const uint32_t* h = hist + (size_t)(T.chunk0 + k) * 3 * NB + ch.axis * NB;
-                for (int j = 0; j < ch.split; j++) lc += (int)h[j];
+                for (int j = 0; j < ch.split; j++) lc += (int)__ldcg(h + j);
             }
         }
         int inc = lc;
@@ -622,7 +630,7 @@ struct BlockSmem {
     SahRange wlist[WLIST_CAP];
     float red[SAH_WARPS][6];
     int scan[SAH_WARPS];
-    Choice choice;
+    Choice axis[3];
     int top, nw, bad, take;
 };
 
@@ -830,14 +838,8 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_block(const SahRange* __res
             }
         }
         __syncthreads();
-        if (warp == 0) {
-            Choice c = warp_choose(S.bins, lane);
-            if (c.axis < 0) c.nl = mm / 2;
-            if (lane == 0) S.choice = c;
-        }
-        __syncthreads();
-        const Choice c = S.choice;
-        const int nl = c.nl;
+        const Choice c = block_choose(S.bins, S.axis);
+        const int nl = c.axis < 0 ? mm / 2 : c.nl;
         // stable partition of positions [lb, le)
         const int i0 = tid * SAH_ITEMS;
         bool left[SAH_ITEMS];
@@ -976,13 +978,10 @@ cudaError_t run_levels(rtsdf_ctx* c, SahArena& A, const Links& L, int32_t* order
         int64_t tasks = ntask;
         for (int l = 0; l < levels; l++) {
             const int lev = CT_LEVELS + 2 * l;
-            const unsigned gt = (unsigned)((tasks + SAH_WARPS - 1) / SAH_WARPS);
             const unsigned gc = (unsigned)std::min<int64_t>(n / SAH_CH + tasks + 1, A.cap_chunk);
-            launch_chain(c, k_sah_bin, gc, SAH_THREADS, 0, A.chunks[cur], A.tasks[cur], A.ord0, A.ord1, A.pbox,
-                         A.bins[cur], A.hist, A.counters, lev);
-            launch_chain(c, k_sah_split, gt, SAH_THREADS, 0, A.tasks[cur], lev, A.bins[cur], A.hist, A.chunks[cur],
-                         A.loff, L, A.tasks[cur ^ 1], A.chunks[cur ^ 1], A.bins[cur ^ 1], A.blist, A.counters,
-                         A.cap_task, A.cap_chunk, A.cap_blist, blk);
+            launch_chain(c, k_sah_split, gc, SAH_THREADS, 0, A.chunks[cur], A.tasks[cur], A.ord0, A.ord1, A.pbox,
+                         A.bins[cur], A.hist, A.loff, L, A.tasks[cur ^ 1], A.chunks[cur ^ 1], A.bins[cur ^ 1],
+                         A.blist, A.counters, lev, A.cap_task, A.cap_chunk, A.cap_blist, blk);
             launch_chain(c, k_sah_partition, gc, SAH_THREADS, 0, A.chunks[cur], A.tasks[cur], A.loff, A.ord0, A.ord1,
                          A.pbox, order, A.tasks[cur ^ 1], A.counters, lev);
             tasks = std::min<int64_t>(2 * tasks, A.cap_task);
