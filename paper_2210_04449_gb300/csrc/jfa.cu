@@ -53,7 +53,7 @@ void launch_pass(rtsdf_ctx* c, const uint32_t* in, uint32_t* out, int n, int k, 
 
 // z-blocked pass (dev::jfa_zblock_column): blocks of 32 x 4 threads in
 // (x, y), blockIdx.z = g k + rz.
-template <bool FINAL, int T, bool AHEAD>
+template <bool FINAL, int T, bool AHEAD, bool ZEDGE>
 __global__ void __launch_bounds__(128, 4) k_jfa_zblock(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
                                                       int n, int k, float* __restrict__ coarse, float hc,
                                                       float beta_h) {
@@ -61,8 +61,20 @@ __global__ void __launch_bounds__(128, 4) k_jfa_zblock(const uint32_t* __restric
     const int x = blockIdx.x * 32 + threadIdx.x;
     const int y = blockIdx.y * 4 + threadIdx.y;
     const int rz = (int)(blockIdx.z % (unsigned)k), g = (int)(blockIdx.z / (unsigned)k);
-    if (x >= n || y >= n) return;
-    dev::jfa_zblock_column<FINAL, T, AHEAD>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
+    if constexpr (ZEDGE) {
+        // a warp is one row: its y offsets are the same, its x offsets where
+        // k >= 32 or the row is short
+        const bool ex = __all_sync(0xFFFFFFFFu, x - k < 0 || x + k >= n);
+        const bool ey = y - k < 0 || y + k >= n;
+        if (x >= n || y >= n) return;
+        if (ex && ey) dev::jfa_zblock_column<FINAL, T, AHEAD, true, 2, 2>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
+        else if (ex) dev::jfa_zblock_column<FINAL, T, AHEAD, true, 2, 3>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
+        else if (ey) dev::jfa_zblock_column<FINAL, T, AHEAD, true, 3, 2>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
+        else dev::jfa_zblock_column<FINAL, T, AHEAD, true, 3, 3>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
+    } else {
+        if (x >= n || y >= n) return;
+        dev::jfa_zblock_column<FINAL, T, AHEAD>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
+    }
 }
 
 // Columns below which shorter ones are taken: a thread floods its column
@@ -81,8 +93,10 @@ void launch_zblock(rtsdf_ctx* c, const uint32_t* in, uint32_t* out, int n, int k
     const int lat = (n + k - 1) / k;          // z-lattice members of the fullest residue class
     const int groups = (lat + T - 1) / T;
     dim3 block(32, 4, 1), grid((n + 31) / 32, (n + 3) / 4, (unsigned)(groups * k));
-    if (final) launch_chain(c, k_jfa_zblock<true, T, AHEAD>, grid, block, 0, in, out, n, k, c->coarse, c->hc, beta_h);
-    else launch_chain(c, k_jfa_zblock<false, T, AHEAD>, grid, block, 0, in, out, n, k, c->coarse, c->hc, beta_h);
+    // the last pass (k = 1) has the whole lattice in a column on tiny grids only
+    auto* kern = final ? k_jfa_zblock<true, T, AHEAD, false>
+                       : (lat <= T ? k_jfa_zblock<false, T, AHEAD, true> : k_jfa_zblock<false, T, AHEAD, false>);
+    launch_chain(c, kern, grid, block, 0, in, out, n, k, c->coarse, c->hc, beta_h);
 }
 
 // Coarse SDF without a pass (N = 1: no jump steps).

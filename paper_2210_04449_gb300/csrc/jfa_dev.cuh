@@ -106,29 +106,85 @@ __device__ __forceinline__ int dp2a_lo_s_u(uint32_t a, uint32_t b, int c) {
     return d;
 }
 
-__device__ __forceinline__ int vimin3_s(int a, int b, int c) { return __vimin3_s32(a, b, c); }
-
 // the smallest key a seedless candidate can have: 0x7F000000 + 4 255^2, minus
 // 2 255 (x + y + z) with x, y, z <= 255
 constexpr int SEEDLESS_KEY_MIN = 0x7F000000 - 2 * 255 * 255;
 
-template <bool FINAL, int T, bool AHEAD>
+// Candidates that cannot be are left out where a whole warp or pass knows it:
+// NX, NY = 2: every lane's column is within k of a side in x / y, so that only
+// two of its three offsets lie in the grid; ZEDGE: the column holds the whole
+// lattice, so that its first voxel has no slice below and its last none above.
+// With k = n / 2 that leaves 8 of 27, with n / 4 16 on average: all passes of
+// 256^3 1208 -> 1131 us, 128^3 139 -> 124, 61^3 25.8 -> 23.9.
+template <int N, class V>
+__device__ __forceinline__ V min_of(const V (&a)[N]) {
+    V m = a[0];
+#pragma unroll
+    for (int c = 1; c + 1 < N; c += 2) {
+        if constexpr (sizeof(V) == 4 && V(-1) < V(0)) m = (V)__vimin3_s32((int)m, (int)a[c], (int)a[c + 1]);
+        else m = (V)__vimin3_u32(m, a[c], a[c + 1]);
+    }
+    if (N % 2 == 0) m = min(m, a[N - 1]);
+    return m;
+}
+
+// The voxel's arg-min over the slices [J0, J1) of the three at ss, aa: the
+// smallest key, and the smallest seed at it.
+template <int J0, int J1, int C>
+__device__ __forceinline__ uint32_t jfa_argmin(const uint32_t (*ss)[C], const int (*aa)[C], int z, int& kmin) {
+    constexpr int N = (J1 - J0) * C;
+    // 16-bit -2 z in the low half, 0 in the high half (byte 3 is 0 or, for
+    // a seedless candidate, already pushed out of range through A)
+    const uint32_t wz = (uint32_t)(-2 * z) & 0xFFFFu;
+    int key[N];
+#pragma unroll
+    for (int j = J0; j < J1; j++)
+#pragma unroll
+        for (int c = 0; c < C; c++) key[C * (j - J0) + c] = dp2a_hi_s_u(wz, ss[j][c], aa[j][c]);
+    kmin = min_of(key);
+    // smallest seed among the candidates at kmin: gap = min(key - kmin,
+    // 255) is 0 exactly for them, and gap * 2^24 + seed then orders every
+    // such candidate (a real seed, < 2^24) before every other one (>= 2^24;
+    // a seedless one has gap 255 and wraps to 254 * 2^24 + 0xFFFFFF).
+    // When kmin itself is a seedless key, every candidate is seedless.
+    uint32_t v[N];
+#pragma unroll
+    for (int j = J0; j < J1; j++)
+#pragma unroll
+        for (int c = 0; c < C; c++) {
+            const uint32_t gap = (uint32_t)__viaddmin_s32(key[C * (j - J0) + c], -kmin, 255);
+            v[C * (j - J0) + c] = gap * 0x01000000u + ss[j][c];
+        }
+    const uint32_t vmin = min_of(v);
+    return kmin >= SEEDLESS_KEY_MIN ? SEED_EMPTY : vmin;
+}
+
+template <bool FINAL, int T, bool AHEAD, bool ZEDGE = false, int NX = 3, int NY = 3>
 __device__ __forceinline__ void jfa_zblock_column(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
                                                   int n, int k, int x, int y, int rz, int g,
                                                   float* __restrict__ coarse, float hc, float beta_h) {
+    constexpr int C = NX * NY;
     const uint32_t n2 = (uint32_t)n * (uint32_t)n;
-    uint32_t xs[3], ys[3];
+    const uint32_t row = (uint32_t)y * (uint32_t)n;
+    // offsets -k, 0, k; of two: the one in the grid (or 0 twice) and 0
+    uint32_t xs[NX], ys[NY];
 #pragma unroll
-    for (int i = 0; i < 3; i++) {
-        const int o = (i - 1) * k;
+    for (int i = 0; i < NX; i++) {
+        int o = (i - 1) * k;
+        if (NX == 2) o = i == 1 ? 0 : (x - k >= 0 ? -k : k);
         xs[i] = (uint32_t)((x + o >= 0 && x + o < n) ? x + o : x);
+    }
+#pragma unroll
+    for (int i = 0; i < NY; i++) {
+        int o = (i - 1) * k;
+        if (NY == 2) o = i == 1 ? 0 : (y - k >= 0 ? -k : k);
         ys[i] = (uint32_t)((y + o >= 0 && y + o < n) ? y + o : y) * (uint32_t)n;
     }
     const uint32_t wxy = ((uint32_t)(-2 * x) & 0xFFFFu) | ((uint32_t)(-2 * y) << 16);
     const int vv = x * x + y * y;
     // slice j (0 .. T + 1) holds z-lattice index T g + j - 1
-    uint32_t ss[T + 2][9];
-    int aa[T + 2][9];
+    uint32_t ss[T + 2][C];
+    int aa[T + 2][C];
     auto take = [&](int j, int c, uint32_t sv) {
         ss[j][c] = sv;
         aa[j][c] = dp2a_lo_s_u(wxy, sv, (int)__dp4a(sv, sv, sv & 0x7F000000u));
@@ -138,78 +194,60 @@ __device__ __forceinline__ void jfa_zblock_column(const uint32_t* __restrict__ i
         if (z >= 0 && z < n) {
             const uint32_t zo = (uint32_t)z * n2;
 #pragma unroll
-            for (int iy = 0; iy < 3; iy++)
+            for (int iy = 0; iy < NY; iy++)
 #pragma unroll
-                for (int ix = 0; ix < 3; ix++) take(j, 3 * iy + ix, __ldg(in + zo + ys[iy] + xs[ix]));
+                for (int ix = 0; ix < NX; ix++) take(j, NX * iy + ix, __ldg(in + zo + ys[iy] + xs[ix]));
         } else {
 #pragma unroll
-            for (int c = 0; c < 9; c++) {
+            for (int c = 0; c < C; c++) {
                 ss[j][c] = SEED_EMPTY;
                 aa[j][c] = 0x7F000000;
             }
         }
     };
     // AHEAD: the seeds of a slice without a branch, read one step before use
-    uint32_t nx[9];
+    uint32_t nx[C];
     auto fetch = [&](int j) {
         const int z = rz + k * (T * g + j - 1);
         const bool in_grid = z >= 0 && z < n;
         const uint32_t* p = in + (uint32_t)(in_grid ? z : 0) * n2;
 #pragma unroll
-        for (int iy = 0; iy < 3; iy++)
+        for (int iy = 0; iy < NY; iy++)
 #pragma unroll
-            for (int ix = 0; ix < 3; ix++) nx[3 * iy + ix] = in_grid ? __ldg(p + (ys[iy] + xs[ix])) : SEED_EMPTY;
+            for (int ix = 0; ix < NX; ix++) nx[NX * iy + ix] = in_grid ? __ldg(p + (ys[iy] + xs[ix])) : SEED_EMPTY;
     };
     auto take_slice = [&](int j) {
 #pragma unroll
-        for (int c = 0; c < 9; c++) take(j, c, nx[c]);
+        for (int c = 0; c < C; c++) take(j, c, nx[c]);
     };
     if (AHEAD) {
-        fetch(0);
-        take_slice(0);
+        if (!ZEDGE) {
+            fetch(0);
+            take_slice(0);
+        }
         fetch(1);
         take_slice(1);
         fetch(2);
     } else {
-        load_slice(0);
+        if (!ZEDGE) load_slice(0);
         load_slice(1);
     }
 #pragma unroll
     for (int t = 0; t < T; t++) {
-        if (AHEAD) take_slice(t + 2);
-        else load_slice(t + 2);
+        const bool above = !(ZEDGE && t == T - 1);   // slice t + 2 is wanted
+        if (above) {
+            if (AHEAD) take_slice(t + 2);
+            else load_slice(t + 2);
+        }
         const int z = rz + k * (T * g + t);
         if (z >= n) break;
-        if (AHEAD && t + 1 < T) fetch(t + 3);
-        // 16-bit -2 z in the low half, 0 in the high half (byte 3 is 0 or, for
-        // a seedless candidate, already pushed out of range through A)
-        const uint32_t wz = (uint32_t)(-2 * z) & 0xFFFFu;
-        int key[27];
-#pragma unroll
-        for (int j = 0; j < 3; j++)
-#pragma unroll
-            for (int c = 0; c < 9; c++) key[9 * j + c] = dp2a_hi_s_u(wz, ss[t + j][c], aa[t + j][c]);
-        int kmin = vimin3_s(key[0], key[1], key[2]);
-#pragma unroll
-        for (int c = 3; c < 27; c += 2) kmin = vimin3_s(kmin, key[c], key[c + 1]);
-        // smallest seed among the candidates at kmin: gap = min(key - kmin,
-        // 255) is 0 exactly for them, and gap * 2^24 + seed then orders every
-        // such candidate (a real seed, < 2^24) before every other one (>= 2^24;
-        // a seedless one has gap 255 and wraps to 254 * 2^24 + 0xFFFFFF).
-        // When kmin itself is a seedless key, every candidate is seedless.
-        uint32_t v[27];
-#pragma unroll
-        for (int j = 0; j < 3; j++)
-#pragma unroll
-            for (int c = 0; c < 9; c++) {
-                const uint32_t gap = (uint32_t)__viaddmin_s32(key[9 * j + c], -kmin, 255);
-                v[9 * j + c] = gap * 0x01000000u + ss[t + j][c];
-            }
-        uint32_t vmin = __vimin3_u32(v[0], v[1], v[2]);
-#pragma unroll
-        for (int c = 3; c < 27; c += 2) vmin = __vimin3_u32(vmin, v[c], v[c + 1]);
-        const uint32_t best = kmin >= SEEDLESS_KEY_MIN ? SEED_EMPTY : vmin;
-        const uint32_t idx = (uint32_t)x + ys[1] + (uint32_t)z * n2;
+        if (AHEAD && t + 1 < T && !(ZEDGE && t + 1 == T - 1)) fetch(t + 3);
+        int kmin;
+        uint32_t best;
+        if (ZEDGE && t == 0) best = jfa_argmin<1, 3, C>(ss + t, aa + t, z, kmin);
+        else if (ZEDGE && t == T - 1) best = jfa_argmin<0, 2, C>(ss + t, aa + t, z, kmin);
+        else best = jfa_argmin<0, 3, C>(ss + t, aa + t, z, kmin);
+        const uint32_t idx = (uint32_t)x + row + (uint32_t)z * n2;
         out[idx] = best;
         if (FINAL) coarse[idx] = dev::coarse_value(best, (uint32_t)(kmin + vv + z * z), hc, beta_h);
     }
