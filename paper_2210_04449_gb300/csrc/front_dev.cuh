@@ -29,8 +29,7 @@
 // instead of 8 cost 7 %, so latency binds (72 % of the issue slots used),
 // and what a front may cost in registers and shared memory is bounded by
 // that.  A fifth of the time goes into making rays and testing the front.
-// Tried: two boxes at a time with packed fp32 (the same time, more
-// registers), rays made in a called function (5 % slower: registers saved
+// Tried: rays made in a called function (5 % slower: registers saved
 // around the call), one stack entry a step instead of a loop (the same), runs
 // of neighbouring units for the warps of an SM (L1 hits 27 instead of 11 %,
 // the same time), fronts of 32 (3 % faster on the 1M frame, 14 % slower in
@@ -55,9 +54,13 @@ constexpr int FRONT_STACK = 8;       // stack entries in shared memory below a f
 // One warp's shared state.
 struct WarpTrace {
     // the front of the unit whose rays are being made
-    // (while it is opened: lo xyz, hi x | hi yz; then: centre xyz, half extent x | y z)
-    float4 box0[FRONT_MAX];
-    float2 box1[FRONT_MAX];
+    union {
+        struct {                     // while it is opened, by entry:
+            float4 box0[FRONT_MAX];  // lo xyz, hi x
+            float2 box1[FRONT_MAX];  // hi yz
+        };
+        float4 pair[FRONT_MAX / 2][3];   // then, by two entries: centre x x y y | z z, half extent x x | y y z z
+    };
     // two units' entries (rays of the previous unit may still be under way):
     // (node or ~leaf, distance from the unit as float bits)
     int2 ent[2][FRONT_MAX];
@@ -113,6 +116,25 @@ struct FrontStack : Stack<FRONT_STACK> {
         return true;
     }
 };
+
+// Packed fp32 (sm_100 and later): two fused multiply-adds, each rounded as
+// the scalar one.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pair2(float a) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
+    return r;
+}
+__device__ __forceinline__ float2 split2(f32x2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
 
 __device__ __forceinline__ void texel_coords(const TraceArgs& a, uint32_t slot, uint32_t& jx, uint32_t& jy,
                                              uint32_t& jz) {
@@ -288,8 +310,12 @@ __device__ __forceinline__ int build_front(const WNode* __restrict__ wide, int r
                 h[k] = fmaxf(hi[k] - c[k], c[k] - lo[k]) * (1.f + 0x1p-20f);
             }
         }
-        w.box0[e] = make_float4(c[0], c[1], c[2], h[0]);
-        w.box1[e] = make_float2(h[1], h[2]);
+        float* p = &w.pair[e >> 1][0].x + (e & 1);
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            p[2 * k] = c[k];
+            p[6 + 2 * k] = h[k];
+        }
         ent[e] = make_int2(id[s], (int)(key[s] & ~63u));
     }
     __syncwarp();
@@ -313,20 +339,32 @@ __device__ __forceinline__ int make_rays(const TraceArgs& a, WarpTrace& w, int b
     const float3 d = sphere_dir(a.key0, a.key1, jx + nf * (jy + nf * jz), a.frame, ray);
     const float3 id = make_float3(safe_inv(d.x), safe_inv(d.y), safe_inv(d.z));
     const float3 oid = make_float3(o.x * id.x, o.y * id.y, o.z * id.z);
-    const float3 ad = make_float3(fabsf(id.x), fabsf(id.y), fabsf(id.z));
+    // two boxes at a time with packed fp32: the slab of an axis is centre +-
+    // half extent, times the reciprocal direction.  Four boxes a turn: with
+    // eight, their loads push the traversal's registers out (1M frame 358 and
+    // 377 ms; one box at a time 358, but 6 % slower where most of the time goes
+    // into making rays)
+    const f32x2 ix = pair2(id.x), iy = pair2(id.y), iz = pair2(id.z);
+    const f32x2 ox = pair2(-oid.x), oy = pair2(-oid.y), oz = pair2(-oid.z);
+    const f32x2 ax = pair2(fabsf(id.x)), ay = pair2(fabsf(id.y)), az = pair2(fabsf(id.z));
+    const f32x2 bx = pair2(-fabsf(id.x)), by = pair2(-fabsf(id.y)), bz = pair2(-fabsf(id.z));
     uint32_t m[2] = {0u, 0u};
 #pragma unroll
     for (int s = 0; s < 2; s++) {
         for (int b = 32 * s; b < min(n, 32 * s + 32); b += 8) {
             uint32_t part = 0u;
-#pragma unroll
-            for (int k = 0; k < 8; k++) {
-                const float4 p = w.box0[b + k];
-                const float2 q = w.box1[b + k];
-                const float cx = fmaf(p.x, id.x, -oid.x), cy = fmaf(p.y, id.y, -oid.y), cz = fmaf(p.z, id.z, -oid.z);
-                const float t0 = fmax3(fmaf(-p.w, ad.x, cx), fmaf(-q.x, ad.y, cy), fmaxf(fmaf(-q.y, ad.z, cz), 0.f));
-                const float t1 = fmin3(fmaf(p.w, ad.x, cx), fmaf(q.x, ad.y, cy), fmaf(q.y, ad.z, cz));
-                if (t0 <= t1) part |= 1u << k;
+#pragma unroll 2
+            for (int k = 0; k < 4; k++) {
+                const f32x2* p = reinterpret_cast<const f32x2*>(w.pair[(b >> 1) + k]);
+                const ulonglong2 p0 = *reinterpret_cast<const ulonglong2*>(p);
+                const ulonglong2 p1 = *reinterpret_cast<const ulonglong2*>(p + 2);
+                const ulonglong2 p2 = *reinterpret_cast<const ulonglong2*>(p + 4);
+                const f32x2 cx = fma2(p0.x, ix, ox), cy = fma2(p0.y, iy, oy), cz = fma2(p1.x, iz, oz);
+                const float2 lx = split2(fma2(p1.y, bx, cx)), hx = split2(fma2(p1.y, ax, cx));
+                const float2 ly = split2(fma2(p2.x, by, cy)), hy = split2(fma2(p2.x, ay, cy));
+                const float2 lz = split2(fma2(p2.y, bz, cz)), hz = split2(fma2(p2.y, az, cz));
+                if (fmax3(lx.x, ly.x, fmaxf(lz.x, 0.f)) <= fmin3(hx.x, hy.x, hz.x)) part |= 1u << (2 * k);
+                if (fmax3(lx.y, ly.y, fmaxf(lz.y, 0.f)) <= fmin3(hx.y, hy.y, hz.y)) part |= 2u << (2 * k);
             }
             m[s] |= part << (b & 31);
         }
