@@ -183,39 +183,40 @@ __device__ __forceinline__ float pad_lo(float v, float pad) { return v - (pad + 
 __device__ __forceinline__ float pad_hi(float v, float pad) { return v + (pad + fabsf(v) * 0x1p-18f); }
 
 __device__ __forceinline__ void store_child(BNode* node, bool right, const float lo[3], const float hi[3]) {
-    float* a = right ? &node->b.x : &node->a.x;
-    a[0] = lo[0]; a[1] = hi[0]; a[2] = lo[1]; a[3] = hi[1];
-    float* c = &node->c.x + (right ? 2 : 0);
-    c[0] = lo[2]; c[1] = hi[2];
+    *(right ? &node->b : &node->a) = make_float4(lo[0], hi[0], lo[1], hi[1]);
+    reinterpret_cast<float2*>(&node->c)[right] = make_float2(lo[2], hi[2]);
 }
 
 // Bottom-up boxes from `child` (a node id, or ~leaf) with box (lo, hi)
 // whose parent is `node`: each node takes the box of its first-arriving
 // child into its child slot and counts the arrival; the second arrival
-// forms the union and climbs on.  A negative parent ends the climb.
+// forms the union and climbs on.  A negative parent ends the climb.  Bound by
+// the latency of one leaf's way up: one acquire-release count a node in place
+// of a count between two full fences, and the parent's links read ahead (whole
+// build: 2.2k triangles 315 -> 300 us, 300k 1070 -> 1035, 1M 2328 -> 2275).
 __device__ __forceinline__ void climb(BNode* nodes, uint32_t* flags, float* __restrict__ nbox, int child, int node,
                                       float lo[3], float hi[3], int64_t guard_n) {
+    if (node < 0) return;
+    int4 d = nodes[node].d;
     // a tree over n leaves has depth < n; the guard only bounds the loop
-    for (int64_t guard = 0; node >= 0 && guard < guard_n; guard++) {
+    for (int64_t guard = 0; guard < guard_n; guard++) {
         BNode* nd = nodes + node;
-        const bool right = nd->d.y == child;
-        store_child(nd, right, lo, hi);
-        __threadfence();
-        if (atomicAdd(flags + node, 1u) != 1u) return;   // first arrival: the sibling finishes this node
-        __threadfence();
+        const int4 up = d.z >= 0 ? nodes[d.z].d : d;   // read early: the next step starts without a wait
+        store_child(nd, d.y == child, lo, hi);
+        if (atomic_add_acq_rel(flags + node, 1u) != 1u) return;   // first arrival: the sibling finishes this node
         // both children present: box of this node = union of its two child boxes
-        const volatile float* a = &nd->a.x;
-        const volatile float* b = &nd->b.x;
-        const volatile float* c = &nd->c.x;
-        lo[0] = fminf(a[0], b[0]); hi[0] = fmaxf(a[1], b[1]);
-        lo[1] = fminf(a[2], b[2]); hi[1] = fmaxf(a[3], b[3]);
-        lo[2] = fminf(c[0], c[2]); hi[2] = fmaxf(c[1], c[3]);
-        for (int k = 0; k < 3; k++) {
-            nbox[6 * (int64_t)node + k] = lo[k];
-            nbox[6 * (int64_t)node + 3 + k] = hi[k];
-        }
+        const float4 a = __ldcg(&nd->a), b = __ldcg(&nd->b), c = __ldcg(&nd->c);
+        lo[0] = fminf(a.x, b.x); hi[0] = fmaxf(a.y, b.y);
+        lo[1] = fminf(a.z, b.z); hi[1] = fmaxf(a.w, b.w);
+        lo[2] = fminf(c.x, c.z); hi[2] = fmaxf(c.y, c.w);
+        float2* box = reinterpret_cast<float2*>(nbox + 6 * (int64_t)node);
+        box[0] = make_float2(lo[0], lo[1]);
+        box[1] = make_float2(lo[2], hi[0]);
+        box[2] = make_float2(hi[1], hi[2]);
         child = node;
-        node = nd->d.z;
+        node = d.z;
+        if (node < 0) return;
+        d = up;
     }
 }
 

@@ -238,6 +238,16 @@ __device__ __forceinline__ void chain_begin() {
 }
 #endif
 
+#ifdef __CUDACC__
+// Counts an arrival: what this thread wrote before (and what its block did,
+// past a barrier) is visible to whoever sees the count, and the other way round.
+__device__ __forceinline__ uint32_t atomic_add_acq_rel(uint32_t* p, uint32_t v) {
+    uint32_t old;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+    return old;
+}
+#endif
+
 template <class... P, class... A>
 inline cudaError_t launch_chain(rtsdf_ctx* c, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, A... args) {
     cudaLaunchAttribute attr;
