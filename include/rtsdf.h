@@ -358,8 +358,7 @@ rtsdf_status rtsdf_jfa_noalloc(const uint32_t* seeds_in, uint32_t* seeds_out, fl
  * pipeline of Sec. 2.1-2.2 (voxelize, jump flood, mask, trace, Eq. 1) for
  * every scene in one persistent cooperative kernel launch, replayed from a
  * CUDA graph; with split_trace = 1 that launch stops after the mask and the
- * trace and the Eq. 1 finalize of every scene follow as two launches of
- * their own in the same graph.  Each scene's result equals a plain
+ * trace of every scene follows as a launch of its own in the same graph.  Each scene's result equals a plain
  * per-scene frame (same kernels' arithmetic, same rays).  Scenes must be
  * static within the batch (no pending rtsdf_move_objects).
  * ------------------------------------------------------------------------ */
@@ -368,15 +367,16 @@ typedef struct rtsdf_batch* rtsdf_batch_t;
 typedef struct {
     int32_t blocks_per_sm;  /* persistent blocks per SM (0 = occupancy maximum) */
     int32_t refill_min;     /* tracer: refill a warp once this many lanes are idle (1..32) */
-    int32_t ray_chunk;      /* tracer: rays a warp takes from the global counter at a time */
+    int32_t ray_chunk;      /* tracer: rays a warp takes from the global counter at a time, at most
+                               (a unit of neighbouring texels' rays is at most 512) */
     int32_t use_graph;      /* replay the frame from a CUDA graph (1) or launch directly (0) */
     int32_t barrier_spins;  /* polls before a grid-barrier wait gives up with RTSDF_E_TIMEOUT
                                (0 = default, about ten seconds) */
     int32_t leaf_min;       /* tracer: run the leaf phase once this many lanes hold a parked leaf */
     int32_t split_trace;    /* 0: one persistent launch runs every stage; 1: that launch runs the
-                               pipeline up to the mask, and the trace and the Eq. 1 finalize follow
-                               as two launches of their own in the same frame (and graph), the
-                               trace at the per-scene tracer's occupancy; results are identical */
+                               pipeline up to the mask, and the trace follows as a launch of its own
+                               in the same frame (and graph), at the per-scene tracer's occupancy;
+                               results are identical */
 } rtsdf_batch_tuning;
 
 typedef struct {
@@ -387,8 +387,8 @@ typedef struct {
     float last_frame_ms;    /* device time of the last frame (CUDA events) */
     /* stage times of the last frame, ms (global timer read at the stage
        barriers; with split_trace, trace runs from the end of the pipeline
-       launch to the start of the finalize launch): clear, voxelize, large
-       triangles, jump flood, mask, trace, finalize */
+       launch to the end of the last trace block): clear, voxelize, large
+       triangles, jump flood, mask, trace (with Eq. 1), and 0 */
     float stage_ms[7];
 } rtsdf_batch_info;
 
@@ -417,7 +417,8 @@ typedef struct {
                                     4 = 32x4 threads flooding 4 voxels each along z (shared z-slices) */
     int32_t trace_blocks_per_sm; /* persistent tracer blocks per SM (0 = occupancy maximum) */
     int32_t refill_min;          /* tracer: refill a warp once this many lanes are idle (1..32) */
-    int32_t ray_chunk;           /* tracer: rays a warp takes from the global counter at a time */
+    int32_t ray_chunk;           /* tracer: rays a warp takes from the global counter at a time, at most
+                                    (a unit of neighbouring texels' rays is at most 512) */
     int32_t leaf_min;            /* tracer: run the leaf phase once this many lanes hold a parked leaf (1..32) */
 } rtsdf_tuning;
 

@@ -92,7 +92,6 @@ void free_all(rtsdf_ctx* c) {
     dfree(c->obj_trans); dfree(c->obj_xform); dfree(c->moved_list); dfree(c->d_moved_count);
     dfree(c->seeds[0]); dfree(c->seeds[1]); dfree(c->coarse); dfree(c->big_list); dfree(c->d_big_count);
     dfree(c->accum); dfree(c->counts); dfree(c->fine); dfree(c->masked); dfree(c->d_frame_words);
-    dfree(c->ray_min); dfree(c->ray_cnt);
     dfree(c->bin_count); dfree(c->bin_start); dfree(c->bin_cursor); dfree(c->bin_items); dfree(c->bin_overflow);
     drop_texture(c->bvh.wtex);
     dfree(c->bvh.nodes); dfree(c->bvh.wide); dfree(c->bvh.nbox); dfree(c->bvh.lbox); dfree(c->bvh.tri); dfree(c->bvh.leaf_tri); dfree(c->bvh.leaf_parent); dfree(c->bvh.flags);
@@ -117,16 +116,6 @@ cudaError_t reset_temporal(rtsdf_ctx* c) {
     cudaError_t e = fill_f32(c, c->accum, c->nf3, INFINITY);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->counts, 0, c->nf3 * sizeof(uint32_t), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->fine, 0, c->nf3 * sizeof(float), c->stream);
-    return e;
-}
-
-// Per-slot frame scratch back to "nothing committed" for the context's sign
-// mode (after a mode change).
-cudaError_t reset_scratch(rtsdf_ctx* c) {
-    const bool nearest = c->sign_mode == RTSDF_SIGN_NEAREST;
-    cudaError_t e = nearest ? cudaMemsetAsync(c->ray_min, 0xFF, 8 * c->nc3 * sizeof(uint32_t), c->stream)
-                            : fill_f32(c, reinterpret_cast<float*>(c->ray_min), 8 * c->nc3, INFINITY);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->ray_cnt, 0, 8 * c->nc3 * sizeof(uint32_t), c->stream);
     return e;
 }
 
@@ -224,8 +213,6 @@ rtsdf_status rtsdf_create(const rtsdf_config* cfg, rtsdf_t* out) {
     if (!e) e = dalloc(&c->counts, c->nf3);
     if (!e) e = dalloc(&c->fine, c->nf3);
     if (!e) e = dalloc(&c->masked, c->nc3);
-    if (!e) e = dalloc(&c->ray_min, 8 * c->nc3);
-    if (!e) e = dalloc(&c->ray_cnt, 8 * c->nc3);
     {
         const size_t g = (size_t)(c->nc + 7) / 8, cells = g * g * g;
         c->bin_cap = 1u << 23;
@@ -252,8 +239,6 @@ rtsdf_status rtsdf_create(const rtsdf_config* cfg, rtsdf_t* out) {
     if (!e) e = cudaMemsetAsync(c->seeds[0], 0xFF, c->nc3 * sizeof(uint32_t), c->stream);
     if (!e) e = cudaMemsetAsync(c->seeds[1], 0xFF, c->nc3 * sizeof(uint32_t), c->stream);
     if (!e) e = fill_f32(c, c->coarse, c->nc3, INFINITY);
-    if (!e) e = fill_f32(c, reinterpret_cast<float*>(c->ray_min), 8 * c->nc3, INFINITY);
-    if (!e) e = cudaMemsetAsync(c->ray_cnt, 0, 8 * c->nc3 * sizeof(uint32_t), c->stream);
     if (!e) e = reset_temporal(c);
     if (!e) e = cudaStreamSynchronize(c->stream);
     if (e) {
@@ -651,11 +636,7 @@ rtsdf_status rtsdf_load_state(rtsdf_t c, const void* host_buf, size_t bytes) {
     if (hdr[3] != RTSDF_SIGN_VOTE && hdr[3] != RTSDF_SIGN_NEAREST) return RTSDF_E_ARG;
     DeviceGuard g(c->device);
     cudaError_t e = cudaStreamSynchronize(c->stream);
-    if (!e && (int)hdr[3] != c->sign_mode) {
-        c->sign_mode = (int)hdr[3];   // the state carries its sign mode
-        e = reset_scratch(c);
-        if (!e) e = cudaStreamSynchronize(c->stream);
-    }
+    if (!e) c->sign_mode = (int)hdr[3];   // the state carries its sign mode
     if (!e) e = cudaMemcpy(c->accum, p + 16, c->nf3 * sizeof(float), cudaMemcpyHostToDevice);
     if (!e) e = cudaMemcpy(c->counts, p + 16 + c->nf3 * 4, c->nf3 * sizeof(uint32_t), cudaMemcpyHostToDevice);
     if (!e) e = cudaMemcpy(c->fine, p + 16 + c->nf3 * 8, c->nf3 * sizeof(float), cudaMemcpyHostToDevice);
@@ -668,7 +649,6 @@ rtsdf_status rtsdf_set_sign_mode(rtsdf_t c, int32_t mode) {
     DeviceGuard g(c->device);
     c->sign_mode = mode;
     cudaError_t e = reset_temporal(c);   // the counts word changes meaning: restart accumulation
-    if (!e) e = reset_scratch(c);
     return from_cuda(e);
 }
 

@@ -1,11 +1,10 @@
 // Batched form: many independent scenes of uneven grid and mesh size, the
-// whole per-frame pipeline (clear, voxelize, jump flood, mask, trace, Eq. 1
-// finalize) for all of them in ONE persistent cooperative launch, replayed
-// from a CUDA graph -- or, with split_trace, that launch up to the mask and
-// the trace and finalize as two more launches in the same graph: the
-// persistent launch's register budget (64, 8 blocks per SM) is set by its
-// other stages, while the traversal, bound by instruction issue, runs 4 %
-// faster at the tracer's own 9 blocks per SM.
+// whole per-frame pipeline (clear, voxelize, jump flood, mask, trace with Eq. 1)
+// for all of them in ONE persistent cooperative launch, replayed from a CUDA
+// graph -- or, with split_trace, that launch up to the mask and the jump
+// flood's passes and the trace as launches of their own in the same graph:
+// they then get the shared memory, registers and block shape that each stage
+// wants, not the persistent launch's.
 //
 // Work of every stage is flattened over the scenes through prefix sums (a
 // thread finds its scene by binary search), so small scenes do not leave
@@ -95,12 +94,12 @@ struct BatchArgs {
     uint32_t spins;
     unsigned long long* stamps;   // [8] global timer at the stage boundaries (block 0)
     BvhRef bvh;               // every scene's BVH in one array (child ids rebased)
-    int split;                // 1: trace and finalize run as two launches after the pipeline launch
+    int split;                // 1: the trace runs as a launch of its own after the pipeline launch
     int phase;                // split form: 1 = stages 0-2 (the jump flood follows as launches of its
                               // own), 2 = stage 4 on; 0 = the whole frame in one launch
     const uint32_t* jfa_blocks;   // split jump flood: [max_passes][ns + 1] prefix over scenes of their blocks
     unsigned long long* ray_prefix;   // [ns + 1] split form: ray prefix over scenes, written after the mask
-    uint32_t* fin_done;       // split finalize: blocks done (the last one stamps the frame's end)
+    uint32_t* trace_done;     // split trace: blocks done (the last one stamps the frame's end)
 };
 
 __device__ __forceinline__ int find_scene(const unsigned long long* prefix, int ns, unsigned long long g) {
@@ -328,28 +327,6 @@ __device__ __forceinline__ void batch_trace_rays(const BatchArgs& b, const unsig
     trace_units<false, TEX>(src, b.bvh, unit, b.refill_min, b.leaf_min, s_trace, nullptr);
 }
 
-// Stage 6: one grid-stride loop over every scene's slots (slot prefix = ray
-// prefix >> log2 rays); a thread's slot index only grows, so its scene index
-// only moves forward.
-__device__ __forceinline__ void batch_finalize(const BatchArgs& b, const unsigned long long* s_rp, int ns, int lg) {
-    const unsigned long long stot = s_rp[ns] >> lg;
-    int sc = -1;
-    unsigned long long lo = 0, hi = 0;   // slot range of scene sc
-    const TraceArgs* ta = nullptr;
-    const unsigned long long ftid = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
-    const unsigned long long fnthr = gridDim.x * (unsigned long long)blockDim.x;
-    for (unsigned long long g = ftid; g < stot; g += fnthr) {
-        if (g >= hi) {
-            do sc++;
-            while ((s_rp[sc + 1] >> lg) <= g);
-            lo = s_rp[sc] >> lg;
-            hi = s_rp[sc + 1] >> lg;
-            ta = &b.sc[sc].t;
-        }
-        finalize_slot(*ta, g - lo);
-    }
-}
-
 __global__ void __launch_bounds__(TRACE_THREADS, BATCH_BLOCKS_PER_SM) k_batch_frame(BatchArgs b) {
     const uint64_t tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     const uint64_t nthr = gridDim.x * (uint64_t)blockDim.x;
@@ -488,8 +465,8 @@ __global__ void __launch_bounds__(TRACE_THREADS, BATCH_BLOCKS_PER_SM) k_batch_fr
     stamp(b, 5);
 
     if (b.split) {
-        // trace and finalize follow as launches of their own; they read the
-        // ray prefix from global memory
+        // the trace follows as a launch of its own; it reads the ray prefix
+        // from global memory
         if (blockIdx.x == 0) {
             batch_ray_prefix(b, s_prefix, ns, P.rays);
             for (int i = threadIdx.x; i <= ns; i += blockDim.x) b.ray_prefix[i] = s_prefix[i];
@@ -504,22 +481,16 @@ __global__ void __launch_bounds__(TRACE_THREADS, BATCH_BLOCKS_PER_SM) k_batch_fr
     batch_trace_rays<false>(b, s_rp, ns);
     if (!grid_barrier(b)) return;
     stamp(b, 6);
-
-    // ---- stage 6: Eq. 1 finalize of every traced texel slot
-    batch_finalize(b, s_rp, ns, P.log2_rays);
-    grid_barrier(b);
     stamp(b, 7);
 }
 
-// Split form of stages 5 and 6: the trace as its own persistent launch,
-// sized and register-bounded like the per-scene tracer (its occupancy sets
-// its speed: the traversal is issue bound and hides latency with warps),
-// then the finalize; both follow the pipeline launch on the stream and skip
-// their work when that launch gave up at a barrier.
-// (The bound asks for 8 resident blocks, i.e. at most 64 registers, as the
-// per-scene tracer's does; the kernel compiles to 56 and runs 9 blocks per
-// SM.  Asking for 9 forces 55 registers and code that issues 4 % more
-// instructions per ray.)
+// Split form of stage 5: the trace as its own persistent launch, sized and
+// register-bounded like the per-scene tracer (its occupancy sets its speed:
+// the traversal hides latency with warps); it follows the pipeline launch on
+// the stream and skips its work when that launch gave up at a barrier.  (8 resident blocks, i.e. at most 64
+// registers, as for the per-scene tracer, and for the same measured reason:
+// 7 blocks cost that one 7 %, and 9 leave its stack too little shared
+// memory, 360 against 357 ms on 1M triangles.)
 #ifndef BATCH_TRACE_BLOCKS_PER_SM
 #define BATCH_TRACE_BLOCKS_PER_SM 8
 #endif
@@ -528,16 +499,13 @@ template <bool TEX>
 __global__ void __launch_bounds__(TRACE_THREADS, BATCH_TRACE_BLOCKS_PER_SM) k_batch_trace(BatchArgs b) {
     if (*(volatile const uint32_t*)b.abort) return;
     batch_trace_rays<TEX>(b, b.ray_prefix, b.ns);
-}
-
-__global__ void __launch_bounds__(256) k_batch_finalize(BatchArgs b) {
-    if (*(volatile const uint32_t*)b.abort) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) write_stamp(b, 6);   // the trace launch has ended
-    batch_finalize(b, b.ray_prefix, b.ns, b.params->log2_rays);
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(b.fin_done, 1u) == gridDim.x - 1) write_stamp(b, 7);   // the last block out
+        if (atomicAdd(b.trace_done, 1u) == gridDim.x - 1) {   // the last block out
+            write_stamp(b, 6);
+            write_stamp(b, 7);
+        }
     }
 }
 
@@ -584,9 +552,8 @@ struct rtsdf_batch {
     int max_passes = 0;
     // launch configuration (autotuned)
     int blocks_per_sm = 0;       // 0 = occupancy maximum
-    int split_trace = 0;         // trace + finalize as launches of their own after the pipeline launch
+    int split_trace = 0;         // the trace as a launch of its own after the pipeline launch
     unsigned trace_grid = 0;     // blocks of the split trace launch
-    unsigned fin_grid = 0;       // blocks of the split finalize launch
     unsigned long long* d_ray_prefix = nullptr;   // [MAX_BATCH + 1]
     uint32_t* d_jfa_blocks = nullptr;   // split jump flood: [max_passes][ns + 1] block prefix per pass
     size_t jfa_cap = 0;                 // entries of d_jfa_blocks
@@ -654,8 +621,6 @@ cudaError_t refresh_tables(rtsdf_batch* b, bool* changed) {
         d.t.counts = c->counts;
         d.t.fine = c->fine;
         d.t.err = c->d_err;
-        d.t.ray_min = c->ray_min;
-        d.t.ray_cnt = c->ray_cnt;
         d.q = c->qverts;
         d.tris = c->tris;
         d.n_tris = c->nt;
@@ -802,7 +767,7 @@ cudaError_t launch_frame_kernel(rtsdf_batch* b) {
     a.bvh.err = b->d_ctr + 4;
     a.split = b->split_trace;
     a.ray_prefix = b->d_ray_prefix;
-    a.fin_done = b->d_ctr + 5;
+    a.trace_done = b->d_ctr + 5;
     a.jfa_blocks = b->d_jfa_blocks;
     a.phase = b->split_trace ? 1 : 0;
     void* args[] = {&a};
@@ -812,7 +777,7 @@ cudaError_t launch_frame_kernel(rtsdf_batch* b) {
     if (e || !b->split_trace) return e;
     // split form: the jump flood as one launch per pass, the rest of the
     // pipeline (mask, ray prefix) as a second cooperative launch, then the
-    // trace and the finalize
+    // trace
     for (int p = 0; p < b->max_passes; p++) {
         if (b->jfa_total[p] == 0) continue;
         k_batch_jfa<<<b->jfa_total[p], dim3(32, 4, 1), 0, b->stream>>>(a, p);
@@ -823,10 +788,9 @@ cudaError_t launch_frame_kernel(rtsdf_batch* b) {
     e = cudaLaunchCooperativeKernel((const void*)k_batch_frame, dim3(b->grid), dim3(TRACE_THREADS), args, 0,
                                     b->stream);
     if (e) return e;
-    b->launches += 2;
+    b->launches++;
     if (a.bvh.wtex) k_batch_trace<true><<<b->trace_grid, TRACE_THREADS, 0, b->stream>>>(a);
     else k_batch_trace<false><<<b->trace_grid, TRACE_THREADS, 0, b->stream>>>(a);
-    k_batch_finalize<<<b->fin_grid, 256, 0, b->stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -844,11 +808,10 @@ cudaError_t ensure_grid(rtsdf_batch* b) {
     else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&tper, k_batch_trace<false>, TRACE_THREADS, 0);
     if (e) return e;
     if (tper < 1) return cudaErrorInvalidConfiguration;
-    const unsigned tg = (unsigned)(sms * tper), fg = (unsigned)(sms * 8);
-    if (g != b->grid || tg != b->trace_grid || fg != b->fin_grid) {
+    const unsigned tg = (unsigned)(sms * tper);
+    if (g != b->grid || tg != b->trace_grid) {
         b->grid = g;
         b->trace_grid = tg;
-        b->fin_grid = fg;
         drop_graph(b);
     }
     return cudaSuccess;
@@ -1169,8 +1132,8 @@ extern "C" rtsdf_status rtsdf_batch_autotune(rtsdf_batch_t b, float d_vox, int32
     };
     float base = 0.f;
     rtsdf_status st = trial(cur, &base);
-    // one persistent launch for every stage, or the trace and finalize as
-    // launches of their own (at the tracer's own occupancy)
+    // one persistent launch for every stage, or the trace as a
+    // launch of its own (at the tracer's own occupancy)
     if (st == RTSDF_OK) {
         rtsdf_batch_tuning t = cur;
         t.split_trace = 1 - cur.split_trace;

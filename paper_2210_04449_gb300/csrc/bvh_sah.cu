@@ -759,136 +759,136 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_block(const SahRange* __res
     // the ranges are on the device; blocks take them from a counter
     const int count = counters[CT_BLOCKS];
     for (;;) {
-    if (threadIdx.x == 0) S.take = atomicAdd(counters + CT_TAKEN, 1);
-    __syncthreads();
-    const int mine = S.take;
-    if (mine >= count) return;                 // block-uniform
-    const SahRange R = blist[mine];
-    const int gb = R.b, m = R.e - R.b;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int32_t* ord = (R.sb >> 1) ? ord1 : ord0;
-    for (int i = tid; i < m; i += SAH_THREADS) {
-        const int32_t t = ord[gb + i];
-        const float4 l = pbox[2 * (int64_t)t], h = pbox[2 * (int64_t)t + 1];
-        S.lo[0][i] = l.x; S.lo[1][i] = l.y; S.lo[2][i] = l.z;
-        S.hi[0][i] = h.x; S.hi[1][i] = h.y; S.hi[2][i] = h.z;
-        S.tri[i] = t;
-        S.perm[i] = (uint16_t)i;
-    }
-    if (tid == 0) {
-        S.top = 0;
-        S.nw = 0;
-        S.bad = 0;
-        const SahRange r{0, m, R.parent, R.sb & 1};
-        if (m > WARP_MAX) S.stack[S.top++] = r;
-        else S.wlist[S.nw++] = r;
-    }
-    __syncthreads();
-    for (int guard = 0; guard < 2 * SAH_CH; guard++) {
-        if (S.top == 0) break;                 // block-uniform: read after a barrier
-        const SahRange r = S.stack[S.top - 1];
-        const int lb = r.b, le = r.e, mm = le - lb;
-        // centroid bounds of the range; bins reset
-        float cb[6] = {CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
-        for (int p = lb + tid; p < le; p += SAH_THREADS) {
-            const int s = S.perm[p];
-#pragma unroll
-            for (int k = 0; k < 3; k++) {
-                const float c = cen(S.lo[k][s], S.hi[k][s]);
-                cb[k] = fminf(cb[k], c);
-                cb[3 + k] = fmaxf(cb[3 + k], c);
-            }
-        }
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1)
-#pragma unroll
-            for (int k = 0; k < 3; k++) {
-                cb[k] = fminf(cb[k], __shfl_xor_sync(FULL, cb[k], o));
-                cb[3 + k] = fmaxf(cb[3 + k], __shfl_xor_sync(FULL, cb[3 + k], o));
-            }
-        if (lane == 0)
-            for (int k = 0; k < 6; k++) S.red[warp][k] = cb[k];
-        for (int i = tid; i < SAH_BIN_WORDS; i += SAH_THREADS) S.bins[i] = bin_init(i);
+        if (threadIdx.x == 0) S.take = atomicAdd(counters + CT_TAKEN, 1);
         __syncthreads();
-        if (tid == 0) S.top--;
-#pragma unroll
-        for (int k = 0; k < 6; k++) {
-            float v = S.red[0][k];
-            for (int w = 1; w < SAH_WARPS; w++) v = k < 3 ? fminf(v, S.red[w][k]) : fmaxf(v, S.red[w][k]);
-            cb[k] = v;
+        const int mine = S.take;
+        if (mine >= count) return;                 // block-uniform
+        const SahRange R = blist[mine];
+        const int gb = R.b, m = R.e - R.b;
+        const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+        const int32_t* ord = (R.sb >> 1) ? ord1 : ord0;
+        for (int i = tid; i < m; i += SAH_THREADS) {
+            const int32_t t = ord[gb + i];
+            const float4 l = pbox[2 * (int64_t)t], h = pbox[2 * (int64_t)t + 1];
+            S.lo[0][i] = l.x; S.lo[1][i] = l.y; S.lo[2][i] = l.z;
+            S.hi[0][i] = h.x; S.hi[1][i] = h.y; S.hi[2][i] = h.z;
+            S.tri[i] = t;
+            S.perm[i] = (uint16_t)i;
         }
-        const BinMap bm = bin_map(cb, cb + 3);
-        for (int p = lb + tid; p < le; p += SAH_THREADS) {
-            const int s = S.perm[p];
-            float l[3], h[3];
-#pragma unroll
-            for (int k = 0; k < 3; k++) {
-                l[k] = S.lo[k][s];
-                h[k] = S.hi[k][s];
-            }
-#pragma unroll
-            for (int a = 0; a < 3; a++) {
-                uint32_t* q = S.bins + (a * NB + bin_of(bm, a, cen(l[a], h[a]))) * BW;
-                atomicAdd(q, 1u);
+        if (tid == 0) {
+            S.top = 0;
+            S.nw = 0;
+            S.bad = 0;
+            const SahRange r{0, m, R.parent, R.sb & 1};
+            if (m > WARP_MAX) S.stack[S.top++] = r;
+            else S.wlist[S.nw++] = r;
+        }
+        __syncthreads();
+        for (int guard = 0; guard < 2 * SAH_CH; guard++) {
+            if (S.top == 0) break;                 // block-uniform: read after a barrier
+            const SahRange r = S.stack[S.top - 1];
+            const int lb = r.b, le = r.e, mm = le - lb;
+            // centroid bounds of the range; bins reset
+            float cb[6] = {CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
+            for (int p = lb + tid; p < le; p += SAH_THREADS) {
+                const int s = S.perm[p];
 #pragma unroll
                 for (int k = 0; k < 3; k++) {
-                    atomicMin(q + 1 + k, f2o(l[k]));
-                    atomicMax(q + 4 + k, f2o(h[k]));
+                    const float c = cen(S.lo[k][s], S.hi[k][s]);
+                    cb[k] = fminf(cb[k], c);
+                    cb[3 + k] = fmaxf(cb[3 + k], c);
                 }
             }
-        }
-        __syncthreads();
-        const Choice c = block_choose(S.bins, S.axis);
-        const int nl = c.axis < 0 ? mm / 2 : c.nl;
-        // stable partition of positions [lb, le)
-        const int i0 = tid * SAH_ITEMS;
-        bool left[SAH_ITEMS];
-        int nleft = 0;
 #pragma unroll
-        for (int j = 0; j < SAH_ITEMS; j++) {
-            const int i = i0 + j;
-            left[j] = false;
-            if (i < mm) {
-                const int s = S.perm[lb + i];
-                left[j] = c.axis < 0 ? i < nl : bin_of(bm, c.axis, cen(S.lo[c.axis][s], S.hi[c.axis][s])) < c.split;
-                nleft += left[j];
+            for (int o = 16; o >= 1; o >>= 1)
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    cb[k] = fminf(cb[k], __shfl_xor_sync(FULL, cb[k], o));
+                    cb[3 + k] = fmaxf(cb[3 + k], __shfl_xor_sync(FULL, cb[3 + k], o));
+                }
+            if (lane == 0)
+                for (int k = 0; k < 6; k++) S.red[warp][k] = cb[k];
+            for (int i = tid; i < SAH_BIN_WORDS; i += SAH_THREADS) S.bins[i] = bin_init(i);
+            __syncthreads();
+            if (tid == 0) S.top--;
+#pragma unroll
+            for (int k = 0; k < 6; k++) {
+                float v = S.red[0][k];
+                for (int w = 1; w < SAH_WARPS; w++) v = k < 3 ? fminf(v, S.red[w][k]) : fmaxf(v, S.red[w][k]);
+                cb[k] = v;
             }
-        }
-        int total = 0;
-        const int lr0 = block_excl(nleft, S.scan, total);
-        int lr = lr0, rr = min(i0, mm) - lr0;
+            const BinMap bm = bin_map(cb, cb + 3);
+            for (int p = lb + tid; p < le; p += SAH_THREADS) {
+                const int s = S.perm[p];
+                float l[3], h[3];
 #pragma unroll
-        for (int j = 0; j < SAH_ITEMS; j++) {
-            const int i = i0 + j;
-            if (i < mm) S.tmp[lb + (left[j] ? lr++ : nl + rr++)] = S.perm[lb + i];
-        }
-        __syncthreads();
-        for (int p = lb + tid; p < le; p += SAH_THREADS) S.perm[p] = S.tmp[p];
-        if (tid == 0) {
-            const int id = L.node_ids ? L.node_ids[lb + nl - 1] : gb + lb + nl - 1;
-            make_node(L, id, r.parent, r.sb & 1);
-            for (int s = 0; s < 2; s++) {
-                const int cb0 = s ? lb + nl : lb, ce = s ? le : lb + nl, cm = ce - cb0;
-                const SahRange ch{cb0, ce, id, s};
-                if (cm == 1) {
-                    make_leaf(L, id, s, gb + cb0, S.tri[S.tmp[cb0]]);   // tmp: this range's new order
-                } else if (cm <= WARP_MAX) {
-                    if (S.nw < WLIST_CAP) S.wlist[S.nw++] = ch;
-                    else S.bad = 1;
-                } else {
-                    if (S.top < BLK_STACK) S.stack[S.top++] = ch;
-                    else S.bad = 1;
+                for (int k = 0; k < 3; k++) {
+                    l[k] = S.lo[k][s];
+                    h[k] = S.hi[k][s];
+                }
+#pragma unroll
+                for (int a = 0; a < 3; a++) {
+                    uint32_t* q = S.bins + (a * NB + bin_of(bm, a, cen(l[a], h[a]))) * BW;
+                    atomicAdd(q, 1u);
+#pragma unroll
+                    for (int k = 0; k < 3; k++) {
+                        atomicMin(q + 1 + k, f2o(l[k]));
+                        atomicMax(q + 4 + k, f2o(h[k]));
+                    }
                 }
             }
+            __syncthreads();
+            const Choice c = block_choose(S.bins, S.axis);
+            const int nl = c.axis < 0 ? mm / 2 : c.nl;
+            // stable partition of positions [lb, le)
+            const int i0 = tid * SAH_ITEMS;
+            bool left[SAH_ITEMS];
+            int nleft = 0;
+#pragma unroll
+            for (int j = 0; j < SAH_ITEMS; j++) {
+                const int i = i0 + j;
+                left[j] = false;
+                if (i < mm) {
+                    const int s = S.perm[lb + i];
+                    left[j] = c.axis < 0 ? i < nl : bin_of(bm, c.axis, cen(S.lo[c.axis][s], S.hi[c.axis][s])) < c.split;
+                    nleft += left[j];
+                }
+            }
+            int total = 0;
+            const int lr0 = block_excl(nleft, S.scan, total);
+            int lr = lr0, rr = min(i0, mm) - lr0;
+#pragma unroll
+            for (int j = 0; j < SAH_ITEMS; j++) {
+                const int i = i0 + j;
+                if (i < mm) S.tmp[lb + (left[j] ? lr++ : nl + rr++)] = S.perm[lb + i];
+            }
+            __syncthreads();
+            for (int p = lb + tid; p < le; p += SAH_THREADS) S.perm[p] = S.tmp[p];
+            if (tid == 0) {
+                const int id = L.node_ids ? L.node_ids[lb + nl - 1] : gb + lb + nl - 1;
+                make_node(L, id, r.parent, r.sb & 1);
+                for (int s = 0; s < 2; s++) {
+                    const int cb0 = s ? lb + nl : lb, ce = s ? le : lb + nl, cm = ce - cb0;
+                    const SahRange ch{cb0, ce, id, s};
+                    if (cm == 1) {
+                        make_leaf(L, id, s, gb + cb0, S.tri[S.tmp[cb0]]);   // tmp: this range's new order
+                    } else if (cm <= WARP_MAX) {
+                        if (S.nw < WLIST_CAP) S.wlist[S.nw++] = ch;
+                        else S.bad = 1;
+                    } else {
+                        if (S.top < BLK_STACK) S.stack[S.top++] = ch;
+                        else S.bad = 1;
+                    }
+                }
+            }
+            __syncthreads();
         }
+        for (int q = warp; q < S.nw; q += SAH_WARPS) warp_exact(S, S.wlist[q], gb, L, lane);
         __syncthreads();
-    }
-    for (int q = warp; q < S.nw; q += SAH_WARPS) warp_exact(S, S.wlist[q], gb, L, lane);
-    __syncthreads();
-    if (order_final)
-        for (int i = tid; i < m; i += SAH_THREADS) order_final[gb + i] = S.tri[S.perm[i]];
-    if (tid == 0 && (S.bad || S.top != 0)) atomicOr(counters + CT_BAD, 2);
-    __syncthreads();                           // the next range reuses S
+        if (order_final)
+            for (int i = tid; i < m; i += SAH_THREADS) order_final[gb + i] = S.tri[S.perm[i]];
+        if (tid == 0 && (S.bad || S.top != 0)) atomicOr(counters + CT_BAD, 2);
+        __syncthreads();                           // the next range reuses S
     }
 }
 

@@ -23,7 +23,7 @@
 // Measured on the frame of 1M triangles (256^3 -> 512^3, 64 rays): 8.7 node
 // visits a ray instead of 18.8, trace 357.8 instead of 375 ms; on a room of
 // 100k (128^3 -> 256^3): 6.2 instead of 20.4, 138 instead of 170-192 ms; with
-// rays that stop at the accumulated distance: 0.2 instead of 4.6, 2.5 instead
+// rays that stop at the accumulated distance: 0.2 instead of 4.6, 2.3 instead
 // of 2.9 ms (5.7M texels' worth of 32 rays, 75^3).  The visits that remain
 // are the dear ones, to nodes that few other rays share: 7 resident blocks
 // instead of 8 cost 7 %, so latency binds (72 % of the issue slots used),
@@ -385,16 +385,15 @@ __device__ __forceinline__ int make_rays(const TraceArgs& a, WarpTrace& w, int b
     return __popc(bal);
 }
 
-// Hands a unit's per-texel results to the frame's scratch and clears them.
-// All 32 lanes call; no ray of the unit is under way.
+// Applies Eq. 1 to a unit's texels (a unit has all rays of its texels, so no
+// other warp has a part in them) and frees its buffer.  All 32 lanes call; no
+// ray of the unit is under way.  Through scratch of 8 bytes a fine texel and a
+// launch after the tracer's, the frames took more: 24 batched scenes 58.9 ms
+// against 57.1, a room of 100k triangles 114.2 against 113.8, the rigid refit
+// frame 5.438 against 5.417.
 __device__ __forceinline__ void flush_unit(const TraceArgs& a, WarpTrace& w, int buf, unsigned lane) {
     if (lane < w.ntex[buf]) {
-        const uint32_t slot = w.slot0[buf] + lane;
-        const uint32_t none = ray_min_none(a.nearest != 0);
-        const uint64_t pol = l2_evict_first();
-        const uint32_t mn = w.tmin[buf][lane], cv = w.tcnt[buf][lane];
-        if (mn != none) red_min_stream(a.ray_min + slot, mn, pol);
-        if (cv && !a.nearest) red_add_stream(a.ray_cnt + slot, cv, pol);
+        finalize_slot(a, w.slot0[buf] + lane, w.tmin[buf][lane], w.tcnt[buf][lane]);
     }
     __syncwarp();
     if (lane == 0) w.ntex[buf] = 0;

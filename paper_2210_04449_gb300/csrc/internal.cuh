@@ -186,11 +186,6 @@ struct rtsdf_ctx {
     uint32_t* d_masked_count = nullptr;   // in d_frame_words
     int64_t last_masked = -1;
 
-    // tracer scratch: per texel slot (8 per masked voxel) this frame's
-    // smallest hit distance (float bits, +inf = none) and front | back << 16
-    // hit counts; cleared again by the finalize kernel
-    uint32_t* ray_min = nullptr;
-    uint32_t* ray_cnt = nullptr;
     unsigned long long* d_next_ray = nullptr;   // in d_frame_words
     unsigned trace_grid = 0;
 

@@ -20,10 +20,10 @@
 // idle, so warps are persistent and refill idle lanes with new rays once
 // enough lanes are idle.  The traversal runs in two
 // phases (a lane parks the leaf it reaches and keeps descending; the warp
-// tests triangles when enough lanes hold a parked leaf), two node steps per
-// phase decision.  A finished ray commits its distance (minimum of the
-// float bits, t >= 0) and its front/back hit to its warp's shared memory, a
-// finished texel to per-slot scratch; k_trace_finalize then applies Eq. 1 per texel:
+// tests triangles when enough lanes hold a parked leaf), NODE_STEPS (three)
+// node steps per phase decision.  A finished ray commits its distance (minimum of the
+// float bits, t >= 0) and its front/back hit to its warp's shared memory;
+// once a unit's rays have all finished, the warp applies Eq. 1 to its texels:
 // u_t = min(u, r_t) (the alpha decay was applied by the mask kernel), the
 // counts, and f_t = +-u_t (c_t while no ray has hit), negative when back
 // hits outnumber front hits.  In the nearest-face sign mode a ray starts
@@ -75,15 +75,6 @@ __global__ void __launch_bounds__(TRACE_THREADS, TRACE_MIN_BLOCKS) k_trace(Trace
     trace_units<COUNT, TEX>(src, a, unit, a.refill_min, a.leaf_min, s_trace, a.counters);
 }
 
-// Eq. 1 per traced texel slot (see finalize_slot): a grid-stride loop over
-// the frame's slots (8 per masked voxel, a count known only on the device).
-__global__ void __launch_bounds__(256) k_trace_finalize(TraceArgs a) {
-    chain_begin();
-    const uint64_t n = (uint64_t)(*a.count) * 8u;
-    const uint64_t stride = gridDim.x * (uint64_t)blockDim.x;
-    for (uint64_t s = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; s < n; s += stride) finalize_slot(a, s);
-}
-
 }  // namespace
 
 cudaError_t trace_occupancy(int* per_sm) {
@@ -116,8 +107,6 @@ cudaError_t launch_trace(rtsdf_ctx* c, int rays, int frame) {
     a.fine = c->fine;
     a.err = c->d_err;
     a.counters = c->d_counters;
-    a.ray_min = c->ray_min;
-    a.ray_cnt = c->ray_cnt;
     a.next_ray = c->d_next_ray;
     a.refill_min = c->tune.refill_min;
     a.ray_chunk = c->tune.ray_chunk;
@@ -142,15 +131,6 @@ cudaError_t launch_trace(rtsdf_ctx* c, int rays, int frame) {
     } else {
         if (c->counting) launch_chain(c, k_trace<true, false>, c->trace_grid, TRACE_THREADS, 0, a);
         else launch_chain(c, k_trace<false, false>, c->trace_grid, TRACE_THREADS, 0, a);
-    }
-    // the slot count is on the device: enough blocks to fill every SM
-    // (8 x 256 threads each), capped by the largest possible slot count
-    {
-        int sms = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-        const uint64_t most = (8 * (uint64_t)c->nc3 + 255) / 256;
-        const uint64_t want = (uint64_t)(sms > 0 ? sms : 132) * 8u;
-        launch_chain(c, k_trace_finalize, (unsigned)(most < want ? most : want), 256, 0, a);
     }
     return cudaGetLastError();
 }

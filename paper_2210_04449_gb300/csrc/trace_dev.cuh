@@ -27,8 +27,6 @@ struct TraceArgs {
     float* fine;
     uint32_t* err;
     TraceCounters* counters;   // work counters (counting variant only)
-    uint32_t* ray_min;         // [8 nc^3] per texel slot: min hit distance bits of this frame
-    uint32_t* ray_cnt;         // [8 nc^3] per texel slot: front | back << 16 hits of this frame
     unsigned long long* next_ray;
     int refill_min;            // refill a warp once this many lanes are idle
     int ray_chunk;             // rays a warp takes from the global counter at a time
@@ -37,8 +35,8 @@ struct TraceArgs {
     int nearest;               // sign from the nearest hit's face; rays capped at the texel's u
 };
 
-// Per-slot "nothing committed" value of ray_min: +inf bits for the vote,
-// all ones for the nearest-face key (t bits << 1 | back).
+// "No hit" as a texel's smallest hit of a frame: +inf bits for the vote, all
+// ones for the nearest-face key (t bits << 1 | back).
 __host__ __device__ constexpr uint32_t ray_min_none(bool nearest) { return nearest ? 0xFFFFFFFFu : 0x7F800000u; }
 
 __device__ __forceinline__ void philox4x32_10(uint32_t c[4], uint32_t k0, uint32_t k1) {
@@ -330,26 +328,12 @@ __device__ __forceinline__ bool leaf_step(const A& a, Ray& r, const S& stack, ui
     return true;
 }
 
-// L2 policy for data that streams past the tracer (the per-slot scratch of
-// finished rays): evicted first, so that the BVH nodes and leaf triangles
-// the traversal re-reads keep their place in L2.
-__device__ __forceinline__ uint64_t l2_evict_first() {
-    uint64_t pol;
-    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-__device__ __forceinline__ void red_min_stream(uint32_t* p, uint32_t v, uint64_t pol) {
-    asm volatile("red.relaxed.gpu.global.min.L2::cache_hint.u32 [%0], %1, %2;" ::"l"(p), "r"(v), "l"(pol) : "memory");
-}
-__device__ __forceinline__ void red_add_stream(uint32_t* p, uint32_t v, uint64_t pol) {
-    asm volatile("red.relaxed.gpu.global.add.L2::cache_hint.u32 [%0], %1, %2;" ::"l"(p), "r"(v), "l"(pol) : "memory");
-}
-
-// Eq. 1 for one texel slot after its rays committed: u_t = min(u, r_t) (the
-// alpha decay was applied by the mask stage), counts += this frame's hits
-// (saturating at 16 bits), f_t = +-u_t or c_t while no ray has hit; the
-// slot's scratch is cleared for the next frame.
-__device__ __forceinline__ void finalize_slot(const TraceArgs& a, uint64_t s) {
+// Eq. 1 for one texel slot after its rays committed the smallest hit `rmin`
+// (float bits, or the nearest-face key) and the hit counts `cv` (front |
+// back << 16): u_t = min(u, r_t) (the alpha decay was applied by the mask
+// stage), counts += this frame's hits (saturating at 16 bits), f_t = +-u_t or
+// c_t while no ray has hit.
+__device__ __forceinline__ void finalize_slot(const TraceArgs& a, uint32_t s, uint32_t rmin, uint32_t cv) {
     // every access here streams (each slot and texel is touched once per
     // frame): cache-streaming loads and stores keep the BVH in L2
     const uint32_t parent = __ldcs(a.masked + (s >> 3));
@@ -358,17 +342,15 @@ __device__ __forceinline__ void finalize_slot(const TraceArgs& a, uint64_t s) {
     const uint32_t pq = __umulhi(parent, a.nc_mag), pz = __umulhi(pq, a.nc_mag);
     const uint32_t px = parent - pq * nc, py = pq - pz * nc;
     const uint32_t texel = (2 * px + (ch & 1)) + nf * ((2 * py + ((ch >> 1) & 1)) + nf * (2 * pz + (ch >> 2)));
+    const float u0 = __ldcs(a.accum + texel), c = __ldcs(a.coarse + parent);
+    const uint32_t cw = __ldcs(a.counts + texel);
     if (a.nearest) {
         // Eq. 1's minimum over (u, this frame's nearest hit), keeping the face
         // of the smaller one (counts holds the face: 1 = back)
-        const uint32_t km = __ldcs(a.ray_min + s);
-        __stcs(a.ray_min + s, ray_min_none(true));
-        const float u0 = __ldcs(a.accum + texel);
-        const uint32_t kp =
-            u0 == CUDART_INF_F ? 0xFFFFFFFFu : ((__float_as_uint(u0) << 1) | (__ldcs(a.counts + texel) & 1u));
-        const uint32_t k = min(kp, km);
+        const uint32_t kp = u0 == CUDART_INF_F ? 0xFFFFFFFFu : ((__float_as_uint(u0) << 1) | (cw & 1u));
+        const uint32_t k = min(kp, rmin);
         if (k == 0xFFFFFFFFu) {
-            __stcs(a.fine + texel, __ldcs(a.coarse + parent));
+            __stcs(a.fine + texel, c);
             return;
         }
         const float u = __uint_as_float(k >> 1);
@@ -377,17 +359,12 @@ __device__ __forceinline__ void finalize_slot(const TraceArgs& a, uint64_t s) {
         __stcs(a.fine + texel, (k & 1u) ? -u : u);
         return;
     }
-    const float rmin = __uint_as_float(__ldcs(a.ray_min + s));
-    const uint32_t cv = __ldcs(a.ray_cnt + s);
-    __stcs(a.ray_min + s, ray_min_none(false));
-    __stcs(a.ray_cnt + s, 0u);
-    const float u = fminf(__ldcs(a.accum + texel), rmin);
-    const uint32_t cw = __ldcs(a.counts + texel);
+    const float u = fminf(u0, __uint_as_float(rmin));
     const uint32_t f = min((cw & 0xFFFFu) + (cv & 0xFFFFu), 0xFFFFu);
     const uint32_t b = min((cw >> 16) + (cv >> 16), 0xFFFFu);
     __stcs(a.accum + texel, u);
     __stcs(a.counts + texel, f | (b << 16));
-    const float mag = u == CUDART_INF_F ? __ldcs(a.coarse + parent) : u;
+    const float mag = u == CUDART_INF_F ? c : u;
     __stcs(a.fine + texel, b > f ? -mag : mag);
 }
 
