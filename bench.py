@@ -63,7 +63,7 @@ TRAFFIC = {
     # 174.75 MB written
     "4585f2179a4ae7de": 10.76e9 + 174.75e6,
 }
-TRAFFIC_SOURCES = ("trace.cu", "trace_dev.cuh", "bvh.cu", "bvh_sah.cu")
+TRAFFIC_SOURCES = ("trace.cu", "trace_dev.cuh", "front_dev.cuh", "bvh.cu", "bvh_sah.cu")
 
 
 def _src_hash(*names):

@@ -238,7 +238,7 @@ __device__ __forceinline__ bool node_step(const A& a, Ray& r, S& stack, uint32_t
     // L1's load/store data pipe spends one wavefront per lane and sector, not
     // per 16 bytes, and that pipe binds the traversal.  The texture pipe has
     // its own: with TEX, the child ids (the node's fourth sector) are fetched
-    // as an int4 texel through it, 3.7 % faster on the 1M-triangle frame.
+    // as an int4 texel through it.
     const WNode* w = a.wide + node;
     const float4* row = &w->lox;
     float4 lx, hx, ly, hy, lz, hz;
