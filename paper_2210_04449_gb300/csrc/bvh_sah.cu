@@ -19,7 +19,8 @@
 //    that finishes a range picks the split and every chunk's output offset;
 //    k_sah_partition scatters stably into the other order buffer.
 //  * 32 < m <= blk: one block per range (k_sah_block), boxes in shared
-//    memory, the same binned split down to ranges of 32;
+//    memory, the same binned split down to ranges of 32: by the whole block
+//    above MID_MAX positions, by a warp per range below;
 //  * 2 <= m <= 32: one warp per range, the exact heuristic over every split
 //    of the centroids sorted along each axis (bitonic sort in registers).
 // Float min/max merges go through an order-preserving map to uint32, so
@@ -46,6 +47,13 @@ constexpr int SAH_ITEMS = SAH_CH / SAH_THREADS;
 constexpr int SAH_WARPS = SAH_THREADS / 32;
 constexpr int WARP_MAX = 32;                  // largest range of the exact warp build
 constexpr int BLK_STACK = 48;                 // disjoint ranges > 32 in 1024: at most 31
+// Largest range of the block tier that one warp bins and splits, so that the
+// ranges of a level are split side by side and without block barriers (which
+// bound the tier: 4.5 of its stalls per issue).  Whole build with 256 against
+// the whole block for every range: 2.2k triangles 300 -> 287 us, 104k 642 ->
+// 625, 300k 1034 -> 966, 1M 2277 -> 2076 (with 128: 2110, 1024: 2087).
+constexpr int MID_MAX = 256;
+constexpr int MID_CAP = 32;                   // disjoint ranges > 32 in 1024: at most 31
 constexpr int WLIST_CAP = SAH_CH / 2;         // disjoint ranges >= 2 in 1024
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
@@ -53,9 +61,10 @@ static_assert(SAH_ITEMS * SAH_THREADS == SAH_CH, "one chunk per block pass");
 
 // Largest range of the block tier.  A block splits its range one node after
 // another, so a small mesh, whose few ranges leave most SMs idle, is split
-// further by the levels (each of which costs three launches).  Whole build
-// with 256 against 1024: 2.2k triangles 403 / 505 us, 104k 908 / 1270 us, 1M
-// 2587 / 2389 us (300k: 1170 / 1119 us).
+// further by the levels (each of which costs two launches).  Whole build
+// with 256 against 1024: 2.2k triangles 287 / 357 us, 104k 625 / 685 us (512:
+// 288 / 612); 1M 2587 / 2389 and 300k 1170 / 1119 us when the block tier split
+// node by node.
 constexpr int SAH_BLK_SMALL = 256;
 constexpr int64_t SAH_SMALL_MESH = 200000;
 __host__ __device__ constexpr int blk_of(int64_t n) { return n <= SAH_SMALL_MESH ? SAH_BLK_SMALL : SAH_CH; }
@@ -625,13 +634,14 @@ struct BlockSmem {
     float lo[3][SAH_CH], hi[3][SAH_CH];   // by slot (load order)
     int32_t tri[SAH_CH];                  // triangle of each slot
     uint16_t perm[SAH_CH], tmp[SAH_CH];   // slot at each position
-    uint32_t bins[SAH_BIN_WORDS];
+    uint32_t bins[SAH_WARPS][SAH_BIN_WORDS];   // of each warp's range; [0] also the block's
     SahRange stack[BLK_STACK];
+    SahRange mid[2][MID_CAP];
     SahRange wlist[WLIST_CAP];
     float red[SAH_WARPS][6];
     int scan[SAH_WARPS];
     Choice axis[3];
-    int top, nw, bad, take;
+    int top, nw, bad, take, nmid[2];
 };
 
 // Exact heuristic for a range of <= 32 positions, one warp, one item per lane:
@@ -747,6 +757,100 @@ __device__ void warp_exact(BlockSmem& S, SahRange r0, int gb, const Links& L, in
     if (lane < m) S.perm[lb + lane] = (uint16_t)slot;
 }
 
+// Hands a new range to its tier: a leaf, the exact warp build, the next round
+// of the warps' binned splits (list `to`), or the block's stack.  One thread;
+// others may add ranges at the same time, but not to the stack.
+__device__ __forceinline__ void add_range(BlockSmem& S, const SahRange& r, int gb, const Links& L, int to) {
+    const int m = r.e - r.b;
+    if (m == 1) {
+        make_leaf(L, r.parent, r.sb, gb + r.b, S.tri[S.tmp[r.b]]);   // tmp: the parent's new order
+        return;
+    }
+    SahRange* list = m <= WARP_MAX ? S.wlist : (m <= MID_MAX ? S.mid[to] : S.stack);
+    int* n = m <= WARP_MAX ? &S.nw : (m <= MID_MAX ? &S.nmid[to] : &S.top);
+    const int at = atomicAdd(n, 1);
+    if (at < (m <= WARP_MAX ? WLIST_CAP : (m <= MID_MAX ? MID_CAP : BLK_STACK))) list[at] = r;
+    else S.bad = 1;
+}
+
+// One binned split of a range of at most MID_MAX positions by one warp, as the
+// block splits larger ones (the same bins, choice and stable order); the
+// children go to list `to`.  All 32 lanes call.
+__device__ __forceinline__ void warp_split(BlockSmem& S, const SahRange& r, uint32_t* bins, int gb, const Links& L,
+                                           int lane, int to) {
+    const int lb = r.b, le = r.e, mm = le - lb;
+    float cb[6] = {CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
+    for (int p = lb + lane; p < le; p += 32) {
+        const int s = S.perm[p];
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const float c = cen(S.lo[k][s], S.hi[k][s]);
+            cb[k] = fminf(cb[k], c);
+            cb[3 + k] = fmaxf(cb[3 + k], c);
+        }
+    }
+    for (int i = lane; i < SAH_BIN_WORDS; i += 32) bins[i] = bin_init(i);
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            cb[k] = fminf(cb[k], __shfl_xor_sync(FULL, cb[k], o));
+            cb[3 + k] = fmaxf(cb[3 + k], __shfl_xor_sync(FULL, cb[3 + k], o));
+        }
+    const BinMap bm = bin_map(cb, cb + 3);
+    __syncwarp();
+    for (int p = lb + lane; p < le; p += 32) {
+        const int s = S.perm[p];
+        float l[3], h[3];
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            l[k] = S.lo[k][s];
+            h[k] = S.hi[k][s];
+        }
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            uint32_t* q = bins + (a * NB + bin_of(bm, a, cen(l[a], h[a]))) * BW;
+            atomicAdd(q, 1u);
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                atomicMin(q + 1 + k, f2o(l[k]));
+                atomicMax(q + 4 + k, f2o(h[k]));
+            }
+        }
+    }
+    __syncwarp();
+    Choice c = axis_choose(bins, 0, lane);
+#pragma unroll 1
+    for (int a = 1; a < 3; a++) {
+        const Choice d = axis_choose(bins, a, lane);
+        if (d.cost < c.cost) c = d;
+    }
+    const int nl = c.axis < 0 ? mm / 2 : c.nl;
+    const unsigned lt = (1u << lane) - 1u;
+    int lr = 0, rr = nl;   // stable partition of positions [lb, le)
+    for (int i0 = 0; i0 < mm; i0 += 32) {
+        const int i = i0 + lane;
+        bool left = false;
+        int s = 0;
+        if (i < mm) {
+            s = S.perm[lb + i];
+            left = c.axis < 0 ? i < nl : bin_of(bm, c.axis, cen(S.lo[c.axis][s], S.hi[c.axis][s])) < c.split;
+        }
+        const unsigned in = __ballot_sync(FULL, i < mm), ml = __ballot_sync(FULL, left), mr = in & ~ml;
+        if (i < mm) S.tmp[lb + (left ? lr + __popc(ml & lt) : rr + __popc(mr & lt))] = (uint16_t)s;
+        lr += __popc(ml);
+        rr += __popc(mr);
+    }
+    __syncwarp();
+    for (int p = lb + lane; p < le; p += 32) S.perm[p] = S.tmp[p];
+    if (lane < 2) {
+        const int id = L.node_ids ? L.node_ids[lb + nl - 1] : gb + lb + nl - 1;
+        if (lane == 0) make_node(L, id, r.parent, r.sb & 1);
+        add_range(S, lane ? SahRange{lb + nl, le, id, 1} : SahRange{lb, lb + nl, id, 0}, gb, L, to);
+    }
+    __syncwarp();   // the next range reuses the bins
+}
+
 __global__ void __launch_bounds__(SAH_THREADS) k_sah_block(const SahRange* __restrict__ blist,
                                                            const int32_t* __restrict__ ord0,
                                                            const int32_t* __restrict__ ord1,
@@ -779,9 +883,8 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_block(const SahRange* __res
             S.top = 0;
             S.nw = 0;
             S.bad = 0;
-            const SahRange r{0, m, R.parent, R.sb & 1};
-            if (m > WARP_MAX) S.stack[S.top++] = r;
-            else S.wlist[S.nw++] = r;
+            S.nmid[0] = S.nmid[1] = 0;
+            add_range(S, SahRange{0, m, R.parent, R.sb & 1}, gb, L, 0);   // (m >= 2)
         }
         __syncthreads();
         for (int guard = 0; guard < 2 * SAH_CH; guard++) {
@@ -808,7 +911,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_block(const SahRange* __res
                 }
             if (lane == 0)
                 for (int k = 0; k < 6; k++) S.red[warp][k] = cb[k];
-            for (int i = tid; i < SAH_BIN_WORDS; i += SAH_THREADS) S.bins[i] = bin_init(i);
+            for (int i = tid; i < SAH_BIN_WORDS; i += SAH_THREADS) S.bins[0][i] = bin_init(i);
             __syncthreads();
             if (tid == 0) S.top--;
 #pragma unroll
@@ -828,7 +931,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_block(const SahRange* __res
                 }
 #pragma unroll
                 for (int a = 0; a < 3; a++) {
-                    uint32_t* q = S.bins + (a * NB + bin_of(bm, a, cen(l[a], h[a]))) * BW;
+                    uint32_t* q = S.bins[0] + (a * NB + bin_of(bm, a, cen(l[a], h[a]))) * BW;
                     atomicAdd(q, 1u);
 #pragma unroll
                     for (int k = 0; k < 3; k++) {
@@ -838,7 +941,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_block(const SahRange* __res
                 }
             }
             __syncthreads();
-            const Choice c = block_choose(S.bins, S.axis);
+            const Choice c = block_choose(S.bins[0], S.axis);
             const int nl = c.axis < 0 ? mm / 2 : c.nl;
             // stable partition of positions [lb, le)
             const int i0 = tid * SAH_ITEMS;
@@ -867,27 +970,27 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_block(const SahRange* __res
             if (tid == 0) {
                 const int id = L.node_ids ? L.node_ids[lb + nl - 1] : gb + lb + nl - 1;
                 make_node(L, id, r.parent, r.sb & 1);
-                for (int s = 0; s < 2; s++) {
-                    const int cb0 = s ? lb + nl : lb, ce = s ? le : lb + nl, cm = ce - cb0;
-                    const SahRange ch{cb0, ce, id, s};
-                    if (cm == 1) {
-                        make_leaf(L, id, s, gb + cb0, S.tri[S.tmp[cb0]]);   // tmp: this range's new order
-                    } else if (cm <= WARP_MAX) {
-                        if (S.nw < WLIST_CAP) S.wlist[S.nw++] = ch;
-                        else S.bad = 1;
-                    } else {
-                        if (S.top < BLK_STACK) S.stack[S.top++] = ch;
-                        else S.bad = 1;
-                    }
-                }
+                add_range(S, SahRange{lb, lb + nl, id, 0}, gb, L, 0);
+                add_range(S, SahRange{lb + nl, le, id, 1}, gb, L, 0);
             }
             __syncthreads();
+        }
+        // ranges of up to MID_MAX: a warp each, all of a level at once
+        int from = 0;
+        for (int guard = 0; guard < MID_MAX; guard++) {   // (each level takes at least one off the largest)
+            const int nm = min(S.nmid[from], MID_CAP);
+            if (nm == 0) break;                    // block-uniform
+            for (int q = warp; q < nm; q += SAH_WARPS) warp_split(S, S.mid[from][q], S.bins[warp], gb, L, lane, from ^ 1);
+            __syncthreads();
+            if (tid == 0) S.nmid[from] = 0;
+            __syncthreads();
+            from ^= 1;
         }
         for (int q = warp; q < S.nw; q += SAH_WARPS) warp_exact(S, S.wlist[q], gb, L, lane);
         __syncthreads();
         if (order_final)
             for (int i = tid; i < m; i += SAH_THREADS) order_final[gb + i] = S.tri[S.perm[i]];
-        if (tid == 0 && (S.bad || S.top != 0)) atomicOr(counters + CT_BAD, 2);
+        if (tid == 0 && (S.bad || S.top != 0 || S.nmid[0] != 0 || S.nmid[1] != 0)) atomicOr(counters + CT_BAD, 2);
         __syncthreads();                           // the next range reuses S
     }
 }
