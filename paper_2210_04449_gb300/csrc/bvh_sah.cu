@@ -483,8 +483,14 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_split(const int4* chunks, S
             if (ch.axis < 0) {
                 lc = min(max(nl - (cr.y - b), 0), cr.z);
             } else {
-                const uint32_t* h = hist + (size_t)(T.chunk0 + k) * 3 * NB + ch.axis * NB;
-                for (int j = 0; j < ch.split; j++) lc += (int)__ldcg(h + j);
+                // (all bins, so that their loads are under way together)
+                const uint4* h = reinterpret_cast<const uint4*>(hist + (size_t)(T.chunk0 + k) * 3 * NB + ch.axis * NB);
+#pragma unroll
+                for (int j = 0; j < NB / 4; j++) {
+                    const uint4 v = __ldcg(h + j);
+                    lc += (4 * j < ch.split ? v.x : 0u) + (4 * j + 1 < ch.split ? v.y : 0u) +
+                          (4 * j + 2 < ch.split ? v.z : 0u) + (4 * j + 3 < ch.split ? v.w : 0u);
+                }
             }
         }
         int inc = lc;
@@ -606,16 +612,30 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_partition(const int4* __res
         const int pos = left[j] ? lo_base + lr++ : ro_base + rr++;
         dst[pos] = t[j];
         if ((left[j] ? nl : msz - nl) == 1) order_final[pos] = t[j];
-        if (need_cb && T.child[left[j] ? 0 : 1] >= 0) {
-            uint32_t* p = s_cb[left[j] ? 0 : 1];
+    }
+    if (!need_cb) return;                      // block-uniform
+    // the children's centroid bounds, over the warp first: all items of a
+    // chunk meet in six words a side
 #pragma unroll
-            for (int k = 0; k < 3; k++) {
-                atomicMin(p + k, f2o(c[j][k]));
-                atomicMax(p + 3 + k, f2o(c[j][k]));
+    for (int s = 0; s < 2; s++) {
+        if (T.child[s] < 0) continue;          // block-uniform
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+#pragma unroll
+            for (int j = 0; j < SAH_ITEMS; j++)
+                if (t[j] >= 0 && left[j] == (s == 0)) {
+                    lo = min(lo, f2o(c[j][k]));
+                    hi = max(hi, f2o(c[j][k]));
+                }
+            lo = __reduce_min_sync(FULL, lo);
+            hi = __reduce_max_sync(FULL, hi);
+            if ((threadIdx.x & 31) == 0) {
+                atomicMin(&s_cb[s][k], lo);
+                atomicMax(&s_cb[s][3 + k], hi);
             }
         }
     }
-    if (!need_cb) return;                      // block-uniform
     __syncthreads();
     if (threadIdx.x < 12) {
         const int s = threadIdx.x / 6, k = threadIdx.x % 6;
