@@ -12,7 +12,7 @@
 // tree: [nt - 1] nodes, [nt] leaves, any node may be the root.
 //
 // Three tiers by range size m (blk: 256, or 1024 for large meshes):
-//  * m > blk: level-synchronous over chunks of SAH_CH positions, the levels'
+//  * m > blk: level-synchronous over chunks of 256 or 1024 positions, the levels'
 //    sizes kept on the device so that no level waits for the host.
 //    k_sah_split bins a chunk in shared memory and merges into the range's
 //    bins with global atomics (and keeps the chunk's histogram); the block
@@ -68,6 +68,12 @@ static_assert(SAH_ITEMS * SAH_THREADS == SAH_CH, "one chunk per block pass");
 constexpr int SAH_BLK_SMALL = 256;
 constexpr int64_t SAH_SMALL_MESH = 200000;
 __host__ __device__ constexpr int blk_of(int64_t n) { return n <= SAH_SMALL_MESH ? SAH_BLK_SMALL : SAH_CH; }
+// Positions that a block bins and scatters at a level: 1024, or 256 where those
+// would be too few blocks (the bin atomics of a chunk bound its time).  Whole
+// build with 256 against 1024: 2.2k triangles 254 / 273 us, 12k 325 / 357, 104k
+// 521 / 557, 300k 814 / 848, 1M 2034 / 1820.
+constexpr int64_t SAH_SMALL_CHUNKS = 500000;
+__host__ __device__ constexpr int chunk_of(int64_t n) { return n <= SAH_SMALL_CHUNKS ? SAH_THREADS : SAH_CH; }
 
 // Device-side counters of a build: block ranges listed, a capacity guard that
 // fired, block ranges taken, then (tasks, chunks) of each level of a batch.
@@ -278,7 +284,7 @@ __global__ void k_sah_root(SahTask* t, int4* chunks, uint32_t* bins, SahRange* b
                            int32_t* counters) {
     chain_begin();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nch = (n + SAH_CH - 1) / SAH_CH;
+    const int size = chunk_of(n), nch = (n + size - 1) / size;
     if (i == 0) {
         SahTask r;
         r.b = 0; r.e = n; r.parent = -1; r.side = 0;
@@ -300,7 +306,7 @@ __global__ void k_sah_root(SahTask* t, int4* chunks, uint32_t* bins, SahRange* b
         counters[i] = v;
     }
     if (n > blk) {
-        if (i < nch) chunks[i] = make_int4(0, i * SAH_CH, min(SAH_CH, n - i * SAH_CH), 0);
+        if (i < nch) chunks[i] = make_int4(0, i * size, min(size, n - i * size), 0);
         if (i < SAH_BIN_WORDS) bins[i] = bin_init(i);
     }
 }
@@ -407,6 +413,7 @@ __global__ void k_sah_top_single(const int32_t* child_of, BNode* nodes, int32_t*
 // One block per chunk bins it; the block that finishes a range's last chunk
 // then splits the range: split choice, node links, chunk output offsets, and
 // the children (leaf, block range or next-level big range).
+template <int ITEMS>
 __global__ void __launch_bounds__(SAH_THREADS) k_sah_split(const int4* chunks, SahTask* tasks,
                                                            const int32_t* __restrict__ ord0,
                                                            const int32_t* __restrict__ ord1,
@@ -416,12 +423,13 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_split(const int4* chunks, S
                                                            SahRange* blist, int32_t* counters, int lev,
                                                            int32_t cap_task, int32_t cap_chunk, int32_t cap_blist,
                                                            int blk) {
+    constexpr int CH = ITEMS * SAH_THREADS;   // chunk size
     __shared__ uint32_t sb[SAH_BIN_WORDS];
     __shared__ Choice s_axis[3];
     __shared__ int s_last;
     chain_begin();
+    const int4 chunk = chunks[blockIdx.x];     // (task, start, length); read beside the counters, before they are known
     if ((int)blockIdx.x >= counters[lev + 1] || counters[CT_BAD]) return;
-    const int4 chunk = chunks[blockIdx.x];     // (task, start, length)
     SahTask& T = tasks[chunk.x];
     for (int i = threadIdx.x; i < SAH_BIN_WORDS; i += SAH_THREADS) sb[i] = bin_init(i);
     float clo[3], chi[3];
@@ -433,10 +441,24 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_split(const int4* chunks, S
     const BinMap m = bin_map(clo, chi);
     const int32_t* ord = T.buf ? ord1 : ord0;
     __syncthreads();
-    for (int i = threadIdx.x; i < chunk.z; i += SAH_THREADS) {
-        const int32_t t = ord[chunk.y + i];
-        const float4 lo = pbox[2 * (int64_t)t], hi = pbox[2 * (int64_t)t + 1];
-        const float l[3] = {lo.x, lo.y, lo.z}, h[3] = {hi.x, hi.y, hi.z};
+    // (all items' loads before the first of them is binned)
+    int32_t t[ITEMS];
+    float4 blo[ITEMS], bhi[ITEMS];
+#pragma unroll
+    for (int j = 0; j < ITEMS; j++) {
+        const int i = (int)threadIdx.x + j * SAH_THREADS;
+        t[j] = i < chunk.z ? ord[chunk.y + i] : -1;
+    }
+#pragma unroll
+    for (int j = 0; j < ITEMS; j++) {
+        const int64_t b = t[j] >= 0 ? 2 * (int64_t)t[j] : 0;
+        blo[j] = pbox[b];
+        bhi[j] = pbox[b + 1];
+    }
+#pragma unroll
+    for (int j = 0; j < ITEMS; j++) {
+        if (t[j] < 0) break;
+        const float l[3] = {blo[j].x, blo[j].y, blo[j].z}, h[3] = {bhi[j].x, bhi[j].y, bhi[j].z};
 #pragma unroll
         for (int a = 0; a < 3; a++) {
             uint32_t* p = sb + (a * NB + bin_of(m, a, cen(l[a], h[a]))) * BW;
@@ -503,46 +525,47 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_split(const int4* chunks, S
         carry += __shfl_sync(FULL, inc, 31);
     }
     const int id = b + nl - 1;
+    // lane s takes side s: a leaf, a block range or a place in the next level
     int child[2] = {-1, -1};
+    int q = 0, c0 = 0;
+    if (lane < 2) {
+        const int cb = lane ? b + nl : b, ce = lane ? e : b + nl, cm = ce - cb;
+        if (cm == 1) {
+            make_leaf(L, id, lane, cb, -1);
+        } else if (cm <= blk) {
+            q = atomicAdd(counters + CT_BLOCKS, 1);
+            if (q < cap_blist) blist[q] = SahRange{cb, ce, id, lane | ((T.buf ^ 1) << 1)};
+            else atomicOr(counters + CT_BAD, 1);
+        } else {
+            q = atomicAdd(counters + lev + 2, 1);
+            c0 = atomicAdd(counters + lev + 3, (cm + CH - 1) / CH);
+        }
+    }
+#pragma unroll
     for (int s = 0; s < 2; s++) {
         const int cb = s ? b + nl : b, ce = s ? e : b + nl, cm = ce - cb;
-        if (cm == 1) {
-            if (lane == 0) make_leaf(L, id, s, cb, -1);
-        } else if (cm <= blk) {
+        if (cm <= blk) continue;
+        const int nch = (cm + CH - 1) / CH;
+        const int qs = __shfl_sync(FULL, q, s), cs = __shfl_sync(FULL, c0, s);
+        if (qs < cap_task && cs + nch <= cap_chunk) {
+            child[s] = qs;
             if (lane == 0) {
-                const int q = atomicAdd(counters + CT_BLOCKS, 1);
-                if (q < cap_blist) blist[q] = SahRange{cb, ce, id, s | ((T.buf ^ 1) << 1)};
-                else atomicOr(counters + CT_BAD, 1);
-            }
-        } else {
-            const int nch = (cm + SAH_CH - 1) / SAH_CH;
-            int q = 0, c0 = 0;
-            if (lane == 0) {
-                q = atomicAdd(counters + lev + 2, 1);
-                c0 = atomicAdd(counters + lev + 3, nch);
-            }
-            q = __shfl_sync(FULL, q, 0);
-            c0 = __shfl_sync(FULL, c0, 0);
-            if (q < cap_task && c0 + nch <= cap_chunk) {
-                child[s] = q;
-                if (lane == 0) {
-                    SahTask r;
-                    r.b = cb; r.e = ce; r.parent = id; r.side = s;
-                    r.buf = T.buf ^ 1; r.chunk0 = c0; r.nchunk = nch; r.axis = -1;
-                    r.split = -1; r.nl = 0; r.child[0] = r.child[1] = -1;
-                    for (int k = 0; k < 3; k++) {
-                        r.cb[k] = 0xFFFFFFFFu;
-                        r.cb[3 + k] = 0u;
-                    }
-                    r.pad[0] = r.pad[1] = 0;
-                    next[q] = r;
+                SahTask r;
+                r.b = cb; r.e = ce; r.parent = id; r.side = s;
+                r.buf = T.buf ^ 1; r.chunk0 = cs; r.nchunk = nch; r.axis = -1;
+                r.split = -1; r.nl = 0; r.child[0] = r.child[1] = -1;
+                for (int k = 0; k < 3; k++) {
+                    r.cb[k] = 0xFFFFFFFFu;
+                    r.cb[3 + k] = 0u;
                 }
-                for (int k = lane; k < nch; k += 32)
-                    next_chunks[c0 + k] = make_int4(q, cb + k * SAH_CH, min(SAH_CH, ce - (cb + k * SAH_CH)), 0);
-                for (int i = lane; i < SAH_BIN_WORDS; i += 32) next_bins[(size_t)q * SAH_BIN_WORDS + i] = bin_init(i);
-            } else if (lane == 0) {
-                atomicOr(counters + CT_BAD, 1);
+                r.pad[0] = r.pad[1] = 0;
+                next[qs] = r;
             }
+            for (int k = lane; k < nch; k += 32)
+                next_chunks[cs + k] = make_int4(qs, cb + k * CH, min(CH, ce - (cb + k * CH)), 0);
+            for (int i = lane; i < SAH_BIN_WORDS; i += 32) next_bins[(size_t)qs * SAH_BIN_WORDS + i] = bin_init(i);
+        } else if (lane == 0) {
+            atomicOr(counters + CT_BAD, 1);
         }
     }
     if (lane == 0) {
@@ -557,6 +580,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_split(const int4* chunks, S
 
 // Stable scatter of a chunk to the other order buffer; leaves get their
 // final position; big children get their centroid bounds.
+template <int ITEMS>
 __global__ void __launch_bounds__(SAH_THREADS) k_sah_partition(const int4* __restrict__ chunks,
                                                                const SahTask* __restrict__ tasks,
                                                                const int32_t* __restrict__ left_off, int32_t* ord0,
@@ -566,8 +590,8 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_partition(const int4* __res
     __shared__ int s_warp[SAH_WARPS];
     __shared__ uint32_t s_cb[2][6];
     chain_begin();
+    const int4 ch = chunks[blockIdx.x];        // as in k_sah_split
     if ((int)blockIdx.x >= counters[lev + 1] || counters[CT_BAD]) return;
-    const int4 ch = chunks[blockIdx.x];
     const SahTask& T = tasks[ch.x];
     const int32_t* src = T.buf ? ord1 : ord0;
     int32_t* dst = T.buf ? ord0 : ord1;
@@ -580,13 +604,13 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_partition(const int4* __res
     }
     const BinMap m = bin_map(clo, chi);
     const int axis = T.axis, split = T.split, nl = T.nl, b = T.b, msz = T.e - T.b;
-    const int i0 = threadIdx.x * SAH_ITEMS;
-    int32_t t[SAH_ITEMS];
-    float c[SAH_ITEMS][3];
-    bool left[SAH_ITEMS];
+    const int i0 = threadIdx.x * ITEMS;
+    int32_t t[ITEMS];
+    float c[ITEMS][3];
+    bool left[ITEMS];
     int nleft = 0;
 #pragma unroll
-    for (int j = 0; j < SAH_ITEMS; j++) {
+    for (int j = 0; j < ITEMS; j++) {
         const int i = i0 + j;
         left[j] = false;
         t[j] = -1;
@@ -607,7 +631,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_partition(const int4* __res
     int lr = lrank0, rr = min(i0, ch.z) - lrank0;
     const bool need_cb = T.child[0] >= 0 || T.child[1] >= 0;
 #pragma unroll
-    for (int j = 0; j < SAH_ITEMS; j++) {
+    for (int j = 0; j < ITEMS; j++) {
         if (t[j] < 0) continue;
         const int pos = left[j] ? lo_base + lr++ : ro_base + rr++;
         dst[pos] = t[j];
@@ -623,7 +647,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_partition(const int4* __res
         for (int k = 0; k < 3; k++) {
             uint32_t lo = 0xFFFFFFFFu, hi = 0u;
 #pragma unroll
-            for (int j = 0; j < SAH_ITEMS; j++)
+            for (int j = 0; j < ITEMS; j++)
                 if (t[j] >= 0 && left[j] == (s == 0)) {
                     lo = min(lo, f2o(c[j][k]));
                     hi = max(hi, f2o(c[j][k]));
@@ -1019,7 +1043,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_block(const SahRange* __res
 
 size_t sah_scratch_bytes(int64_t n) {
     const int64_t cap_task = n / (blk_of(n) + 1) + 2;
-    const int64_t cap_chunk = n / SAH_CH + cap_task + 4;
+    const int64_t cap_chunk = n / chunk_of(n) + cap_task + 4;
     const int64_t cap_blist = n / 2 + 2;
     return sizeof(float4) * 2 * n + sizeof(int32_t) * 3 * n + sizeof(uint32_t) * 3 * NB * cap_chunk +
            sizeof(int32_t) * cap_chunk + sizeof(SahTask) * 2 * cap_task + sizeof(int4) * 2 * cap_chunk +
@@ -1042,7 +1066,7 @@ struct SahArena {
 
 cudaError_t carve(void* scratch, int32_t n, SahArena& A) {
     A.cap_task = n / (blk_of(n) + 1) + 2;
-    A.cap_chunk = n / SAH_CH + A.cap_task + 4;
+    A.cap_chunk = n / chunk_of(n) + A.cap_task + 4;
     A.cap_blist = n / 2 + 2;
     unsigned char* p = (unsigned char*)scratch;
     auto take = [&](size_t bytes) {
@@ -1095,17 +1119,20 @@ cudaError_t run_levels(rtsdf_ctx* c, SahArena& A, const Links& L, int32_t* order
         while (((int64_t)blk << levels) < largest) levels++;
         levels = std::min(levels + 6, LEVEL_BATCH);
     }
+    const bool one = chunk_of(n) == SAH_THREADS;   // items a thread: one or SAH_ITEMS
+    const auto split = one ? k_sah_split<1> : k_sah_split<SAH_ITEMS>;
+    const auto part = one ? k_sah_partition<1> : k_sah_partition<SAH_ITEMS>;
     const int64_t block_grid = std::min<int64_t>(std::max<int64_t>(n / 64, 1), 4 * (int64_t)(sms > 0 ? sms : 132));
     for (int batch = 0;; batch++) {
         if (batch >= 4096) return cudaErrorUnknown;   // sizes shrink every level; only a fault gets here
         int64_t tasks = ntask;
         for (int l = 0; l < levels; l++) {
             const int lev = CT_LEVELS + 2 * l;
-            const unsigned gc = (unsigned)std::min<int64_t>(n / SAH_CH + tasks + 1, A.cap_chunk);
-            launch_chain(c, k_sah_split, gc, SAH_THREADS, 0, A.chunks[cur], A.tasks[cur], A.ord0, A.ord1, A.pbox,
+            const unsigned gc = (unsigned)std::min<int64_t>(n / chunk_of(n) + tasks + 1, A.cap_chunk);
+            launch_chain(c, split, gc, SAH_THREADS, 0, A.chunks[cur], A.tasks[cur], A.ord0, A.ord1, A.pbox,
                          A.bins[cur], A.hist, A.loff, L, A.tasks[cur ^ 1], A.chunks[cur ^ 1], A.bins[cur ^ 1],
                          A.blist, A.counters, lev, A.cap_task, A.cap_chunk, A.cap_blist, blk);
-            launch_chain(c, k_sah_partition, gc, SAH_THREADS, 0, A.chunks[cur], A.tasks[cur], A.loff, A.ord0, A.ord1,
+            launch_chain(c, part, gc, SAH_THREADS, 0, A.chunks[cur], A.tasks[cur], A.loff, A.ord0, A.ord1,
                          A.pbox, order, A.tasks[cur ^ 1], A.counters, lev);
             tasks = std::min<int64_t>(2 * tasks, A.cap_task);
             cur ^= 1;
@@ -1139,7 +1166,7 @@ cudaError_t sah_topology(rtsdf_ctx* c, void* scratch, int32_t* order) {
     cudaError_t e = carve(scratch, n, A);
     if (!e) e = block_attr(c);
     if (e) return e;
-    const int nch0 = (n + SAH_CH - 1) / SAH_CH;
+    const int nch0 = (n + chunk_of(n) - 1) / chunk_of(n);
     const int init_threads = nch0 > SAH_BIN_WORDS ? nch0 : SAH_BIN_WORDS;
     launch_chain(c, k_sah_root, (unsigned)((init_threads + 255) / 256), 256, 0, A.tasks[0], A.chunks[0], A.bins[0],
                  A.blist, n, blk_of(n), A.counters);
@@ -1163,6 +1190,7 @@ cudaError_t sah_segments(rtsdf_ctx* c, void* scratch, int32_t* order, const int3
     std::vector<SahRange> blist;
     std::vector<int32_t> root0((size_t)nseg, 0);
     int32_t largest = 0;
+    const int size = chunk_of(n);
     for (int32_t k = 0; k < nseg; k++) {
         const int32_t b = bounds[k], en = bounds[k + 1], m = en - b;
         if (m == 1) {
@@ -1175,10 +1203,10 @@ cudaError_t sah_segments(rtsdf_ctx* c, void* scratch, int32_t* order, const int3
             memset(&t, 0, sizeof(t));
             t.b = b; t.e = en; t.parent = -2 - k; t.side = 0; t.buf = 0;
             t.chunk0 = (int32_t)chunks.size();
-            t.nchunk = (m + SAH_CH - 1) / SAH_CH;
+            t.nchunk = (m + size - 1) / size;
             t.axis = -1; t.split = -1; t.child[0] = t.child[1] = -1;
             for (int q = 0; q < t.nchunk; q++)
-                chunks.push_back(make_int4((int)tasks.size(), b + q * SAH_CH, std::min(SAH_CH, en - (b + q * SAH_CH)), 0));
+                chunks.push_back(make_int4((int)tasks.size(), b + q * size, std::min(size, en - (b + q * size)), 0));
             tasks.push_back(t);
         }
     }
