@@ -51,7 +51,9 @@ constexpr int BLK_STACK = 48;                 // disjoint ranges > 32 in 1024: a
 // ranges of a level are split side by side and without block barriers (which
 // bound the tier: 4.5 of its stalls per issue).  Whole build with 256 against
 // the whole block for every range: 2.2k triangles 300 -> 287 us, 104k 642 ->
-// 625, 300k 1034 -> 966, 1M 2277 -> 2076 (with 128: 2110, 1024: 2087).
+// 625, 300k 1034 -> 966, 1M 2277 -> 2076 (with 128: 2110, 1024: 2087).  Warps
+// that take ranges from a list as they come, without rounds, were slower: 520 us
+// at 2.2k triangles.
 constexpr int MID_MAX = 256;
 constexpr int MID_CAP = 32;                   // disjoint ranges > 32 in 1024: at most 31
 constexpr int WLIST_CAP = SAH_CH / 2;         // disjoint ranges >= 2 in 1024
@@ -693,8 +695,10 @@ struct BlockSmem {
 // minima), so that a range takes as many steps as its subtree is deep, not as
 // many as it has nodes (a step is a long chain of shuffles, and a block's
 // warps are too few to hide it; node by node, the block tier of 1M triangles
-// took 1.7 ms, and that of 2.2k 0.5 ms).  Positions are local to the block's range
-// (global position = gb + local).
+// took 1.7 ms, and that of 2.2k 0.5 ms).  The three axes' chains run side by
+// side, and small segments take shorter sorts and scans (whole build: 2.2k
+// triangles 251 -> 236 us, 104k 517 -> 499, 300k 803 -> 760, 1M 1817 -> 1757).
+// Positions are local to the block's range (global position = gb + local).
 __device__ void warp_exact(BlockSmem& S, SahRange r0, int gb, const Links& L, int lane) {
     const int lb = r0.b, m = r0.e - r0.b;
     int slot = lane < m ? (int)S.perm[lb + lane] : 0;
@@ -712,22 +716,55 @@ __device__ void warp_exact(BlockSmem& S, SahRange r0, int gb, const Links& L, in
         const int end = sb + sm - 1;                     // last lane of the segment
         float bestc = CUDART_INF_F;
         int bestj = sb, bestidx = lane;
-        if (__any_sync(FULL, sm >= 3)) {
+        const int most = __reduce_max_sync(FULL, sm);   // items of the largest segment
+        if (most >= 3) {
+            // each axis's order: by (segment, centroid, lane); a pair keeps its
+            // order.  Small segments by exchanges between neighbours (as many
+            // steps as the largest has items), else a bitonic sort
+            int order[3];
+            uint32_t key[3];
+#pragma unroll
             for (int a = 0; a < 3; a++) {
-                // sort by (segment, centroid, lane); a pair keeps its order
-                const uint32_t key = sm >= 3 ? f2o(cen(a == 0 ? lo[0] : (a == 1 ? lo[1] : lo[2]),
-                                                       a == 0 ? hi[0] : (a == 1 ? hi[1] : hi[2]))) : 0u;
-                unsigned long long v = ((unsigned long long)sb << 37) | ((unsigned long long)key << 5) |
-                                       (unsigned long long)lane;
+                key[a] = sm >= 3 ? f2o(cen(lo[a], hi[a])) : 0u;
+                order[a] = lane;
+            }
+            if (most <= 8) {
+                for (int step = 0; step < most; step++) {
+                    const bool first = (((lane - sb) ^ step) & 1) == 0;   // of its pair
+                    const int other = (first ? lane + 1 : lane - 1) & 31;
+                    const bool pair = first ? lane < end : lane > sb && sm > 0;
+#pragma unroll
+                    for (int a = 0; a < 3; a++) {
+                        const uint32_t ok = __shfl_sync(FULL, key[a], other);
+                        const int oi = __shfl_sync(FULL, order[a], other);
+                        if (pair && (first ? ok < key[a] : ok > key[a])) {
+                            key[a] = ok;
+                            order[a] = oi;
+                        }
+                    }
+                }
+            } else {
+                unsigned long long v[3];
+#pragma unroll
+                for (int a = 0; a < 3; a++)
+                    v[a] = ((unsigned long long)sb << 37) | ((unsigned long long)key[a] << 5) | (unsigned long long)lane;
 #pragma unroll
                 for (int k = 2; k <= 32; k <<= 1)
 #pragma unroll
                     for (int j = k >> 1; j > 0; j >>= 1) {
-                        const unsigned long long o = __shfl_xor_sync(FULL, v, j);
                         const bool keep_min = ((lane & j) == 0) == ((lane & k) == 0);
-                        v = keep_min == (o < v) ? o : v;
+#pragma unroll
+                        for (int a = 0; a < 3; a++) {
+                            const unsigned long long o = __shfl_xor_sync(FULL, v[a], j);
+                            v[a] = keep_min == (o < v[a]) ? o : v[a];
+                        }
                     }
-                const int idx = (int)(v & 31ull);
+#pragma unroll
+                for (int a = 0; a < 3; a++) order[a] = (int)(v[a] & 31ull);
+            }
+#pragma unroll
+            for (int a = 0; a < 3; a++) {
+                const int idx = order[a];
                 float plo[3], phi[3], slo[3], shi[3];
 #pragma unroll
                 for (int k = 0; k < 3; k++) {
@@ -735,7 +772,8 @@ __device__ void warp_exact(BlockSmem& S, SahRange r0, int gb, const Links& L, in
                     phi[k] = shi[k] = __shfl_sync(FULL, hi[k], idx);
                 }
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1)
+                for (int o = 1; o < 32; o <<= 1) {
+                    if (o >= most) break;
 #pragma unroll
                     for (int k = 0; k < 3; k++) {
                         const float ul = __shfl_up_sync(FULL, plo[k], o), uh = __shfl_up_sync(FULL, phi[k], o);
@@ -749,6 +787,7 @@ __device__ void warp_exact(BlockSmem& S, SahRange r0, int gb, const Links& L, in
                             shi[k] = fmaxf(shi[k], dh);
                         }
                     }
+                }
                 float rlo[3], rhi[3];
 #pragma unroll
                 for (int k = 0; k < 3; k++) {
@@ -763,6 +802,7 @@ __device__ void warp_exact(BlockSmem& S, SahRange r0, int gb, const Links& L, in
                 int bl = lane;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
+                    if (o >= most) break;
                     const float c2 = __shfl_up_sync(FULL, bc, o);
                     const int l2 = __shfl_up_sync(FULL, bl, o);
                     const int d1 = abs(2 * (bl - sb) + 2 - sm), d2 = abs(2 * (l2 - sb) + 2 - sm);
