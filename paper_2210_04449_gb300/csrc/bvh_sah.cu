@@ -50,10 +50,9 @@ constexpr int BLK_STACK = 48;                 // disjoint ranges > 32 in 1024: a
 // Largest range of the block tier that one warp bins and splits, so that the
 // ranges of a level are split side by side and without block barriers (which
 // bound the tier: 4.5 of its stalls per issue).  Whole build with 256 against
-// the whole block for every range: 2.2k triangles 300 -> 287 us, 104k 642 ->
-// 625, 300k 1034 -> 966, 1M 2277 -> 2076 (with 128: 2110, 1024: 2087).  Warps
-// that take ranges from a list as they come, without rounds, were slower: 520 us
-// at 2.2k triangles.
+// the whole block for every range: 2.2k triangles 240 / 249 us, 104k 502 / 517,
+// 300k 757 / 836, 1M 1752 / 1949 (with 128 and 1024: between).  Warps that take
+// ranges from a list as they come, without rounds, were slower: 520 us at 2.2k.
 constexpr int MID_MAX = 256;
 constexpr int MID_CAP = 32;                   // disjoint ranges > 32 in 1024: at most 31
 constexpr int WLIST_CAP = SAH_CH / 2;         // disjoint ranges >= 2 in 1024
@@ -63,17 +62,16 @@ static_assert(SAH_ITEMS * SAH_THREADS == SAH_CH, "one chunk per block pass");
 
 // Largest range of the block tier.  A block splits its range one node after
 // another, so a small mesh, whose few ranges leave most SMs idle, is split
-// further by the levels (each of which costs two launches).  Whole build
-// with 256 against 1024: 2.2k triangles 287 / 357 us, 104k 625 / 685 us (512:
-// 288 / 612); 1M 2587 / 2389 and 300k 1170 / 1119 us when the block tier split
-// node by node.
+// further by the levels (each of which costs two launches).  Whole build with
+// 256 against 1024: 2.2k triangles 240 / 295 us, 104k 502 / 556 (512: 247 and
+// 490); 300k 825 / 755, 1M 1940 / 1752.
 constexpr int SAH_BLK_SMALL = 256;
 constexpr int64_t SAH_SMALL_MESH = 200000;
 __host__ __device__ constexpr int blk_of(int64_t n) { return n <= SAH_SMALL_MESH ? SAH_BLK_SMALL : SAH_CH; }
 // Positions that a block bins and scatters at a level: 1024, or 256 where those
 // would be too few blocks (the bin atomics of a chunk bound its time).  Whole
-// build with 256 against 1024: 2.2k triangles 254 / 273 us, 12k 325 / 357, 104k
-// 521 / 557, 300k 814 / 848, 1M 2034 / 1820.
+// build with 256 against 1024: 2.2k triangles 240 / 262 us, 12k 315 / 346, 104k
+// 502 / 533, 300k 757 / 800, 1M 1960 / 1752.
 constexpr int64_t SAH_SMALL_CHUNKS = 500000;
 __host__ __device__ constexpr int chunk_of(int64_t n) { return n <= SAH_SMALL_CHUNKS ? SAH_THREADS : SAH_CH; }
 
