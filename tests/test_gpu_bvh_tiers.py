@@ -41,3 +41,32 @@ def test_tiers(name, n):
     pipe = oracle.FinePipeline(np.zeros(3, np.float32), 1.0, nc, 0.5, 2.0, 1.0, 2, accel="bvh")
     pipe.frame(v, t, 0, R)
     assert np.array_equal(rt.grids()["accum"].cpu().numpy().astype(np.float64), pipe.u)
+
+
+@pytest.mark.parametrize("n", [200000, 200001, 500000, 500001])
+def test_large_meshes(n):
+    # either side of the mesh sizes at which the build's block tier and its
+    # chunks change: the SAH and the two-level tree (an object of most of the
+    # triangles, one of 300, one of 2) trace the same grids as the Morton tree
+    from paper_2210_04449_gb300 import RTSDF
+    rng = np.random.default_rng(n)
+    c = rng.uniform(0.1, 0.9, (n, 1, 3))
+    v = (c + rng.uniform(-0.004, 0.004, (n, 3, 3))).reshape(-1, 3).astype(np.float32)
+    t = np.arange(3 * n, dtype=np.int32).reshape(-1, 3)
+    obj = np.zeros(3 * n, np.int32)
+    obj[:900], obj[-6:] = 1, 2
+    got = {}
+    for builder in ("lbvh", "sah", "two_level"):
+        rt = RTSDF(10, seed=2)
+        rt.upload_mesh(v, t)
+        rt.set_objects(obj, 3)
+        rt.set_bvh_builder(builder)
+        rt.build_bvh()
+        rt.update(2.0, 4, 0)
+        rt.sync()
+        got[builder] = {k: rt.grids()[k].cpu().numpy() for k in ("accum", "counts", "fine")}
+        rt.close()
+    assert got["lbvh"]["counts"].any()
+    for builder in ("sah", "two_level"):
+        for k, ref in got["lbvh"].items():
+            assert np.array_equal(got[builder][k], ref), (builder, k)
