@@ -543,6 +543,7 @@ struct rtsdf_batch {
     cudaTextureObject_t wtex_all = 0;  // d_wide_all as int4 texels (0: plain loads)
     float4* d_tri_all = nullptr;     // all scenes' leaf triangles
     int64_t wide_cap = 0, tri_cap = 0, total_nt = 0;
+    std::vector<uint64_t> tree_gen;  // Bvh::gen of each scene's tree in these copies (empty: none)
     uint32_t* d_ctr = nullptr;   // big_count, bar_count, bar_gen, abort, err
     unsigned long long* d_stamps = nullptr;
     unsigned long long* d_next_ray = nullptr;
@@ -592,8 +593,67 @@ void drop_graph(rtsdf_batch* b) {
     b->graph_ok = false;
 }
 
-// Rebuild the descriptor table from the scene contexts; returns true when it
-// changed (pointers move when a mesh is uploaded or a BVH rebuilt).
+// Copy the scenes' trees (all, or those built or refitted since their last
+// copy) into the concatenated arrays, on the batch's stream.  Sets *moved when
+// the arrays had to grow, so that a captured frame holds old pointers.
+cudaError_t copy_trees(rtsdf_batch* b, const std::vector<SceneDesc>& desc, bool all, bool* moved) {
+    const int ns = (int)b->scenes.size();
+    int64_t wo = 0, to = 0;
+    for (const rtsdf_ctx* c : b->scenes) {
+        wo += c->bvh.n_wide;
+        to += c->bvh.nt;
+    }
+    cudaError_t e;
+    std::vector<uint64_t> gen;
+    gen.swap(b->tree_gen);   // no copy counts as good until all are made
+    if (wo > b->wide_cap || to > b->tri_cap) {
+        if ((e = cudaStreamSynchronize(b->stream))) return e;   // nothing under way reads the old arrays
+        all = true;
+        *moved = true;
+        if (wo > b->wide_cap) {
+            drop_texture(b->wtex_all);
+            if (b->d_wide_all) cudaFree(b->d_wide_all);
+            b->d_wide_all = nullptr;
+            b->wide_cap = 0;
+            if ((e = cudaMalloc(&b->d_wide_all, sizeof(WNode) * wo))) return e;
+            b->wide_cap = wo;
+            b->wtex_all = make_int4_texture(b->d_wide_all, (sizeof(WNode) / 16) * (size_t)wo, b->device);
+        }
+        if (to > b->tri_cap) {
+            if (b->d_tri_all) cudaFree(b->d_tri_all);
+            b->d_tri_all = nullptr;
+            b->tri_cap = 0;
+            if ((e = cudaMalloc(&b->d_tri_all, sizeof(float4) * TRI_F4 * to))) return e;
+            b->tri_cap = to;
+        }
+    }
+    b->total_nt = to;
+    all = all || gen.size() != (size_t)ns;
+    gen.resize((size_t)ns, 0);
+    for (int s = 0; s < ns; s++) {
+        const Bvh& bv = b->scenes[s]->bvh;
+        if (!all && gen[s] == bv.gen) continue;
+        gen[s] = bv.gen;
+        if (bv.n_wide > 0) {
+            k_rebase_nodes<<<(unsigned)((bv.n_wide + 255) / 256), 256, 0, b->stream>>>(bv.wide, b->d_wide_all,
+                                                                                     bv.n_wide, desc[s].wide_off,
+                                                                                     desc[s].tri_off);
+            b->launches++;
+        }
+        if (bv.nt > 0 &&
+            (e = cudaMemcpyAsync(b->d_tri_all + TRI_F4 * (int64_t)desc[s].tri_off, bv.tri, sizeof(float4) * TRI_F4 * bv.nt,
+                                 cudaMemcpyDeviceToDevice, b->stream)))
+            return e;
+    }
+    if ((e = cudaGetLastError())) return e;
+    b->tree_gen.swap(gen);
+    return cudaSuccess;
+}
+
+// Rebuild the descriptor table from the scene contexts, and the copies of
+// their trees; *changed: the table differs or an array moved (pointers move
+// when a mesh is uploaded or a BVH rebuilt).  A build or refit that keeps all
+// pointers and counts leaves the table as it was and is seen by Bvh::gen.
 cudaError_t refresh_tables(rtsdf_batch* b, bool* changed) {
     const int ns = (int)b->scenes.size();
     std::vector<SceneDesc> desc((size_t)ns);
@@ -653,7 +713,11 @@ cudaError_t refresh_tables(rtsdf_batch* b, bool* changed) {
     }
     *changed = desc.size() != b->h_desc.size() ||
                memcmp(desc.data(), b->h_desc.data(), sizeof(SceneDesc) * desc.size()) != 0 || maxp != b->max_passes;
-    if (!*changed && b->d_desc) return cudaSuccess;
+    if (!*changed && b->d_desc) {
+        bool stale = b->tree_gen.size() != (size_t)ns;
+        for (int s = 0; s < ns && !stale; s++) stale = b->tree_gen[s] != b->scenes[s]->bvh.gen;
+        return stale ? copy_trees(b, desc, false, changed) : cudaSuccess;
+    }
     cudaError_t e = cudaStreamSynchronize(b->stream);
     if (e) return e;
     if (!b->d_desc) {
@@ -667,35 +731,7 @@ cudaError_t refresh_tables(rtsdf_batch* b, bool* changed) {
         if ((e = cudaMalloc(&b->d_big, sizeof(int2) * (at > 0 ? at : 1)))) return e;
         b->big_cap = (int64_t)at;
     }
-    // concatenated BVH of all scenes
-    if (wo > b->wide_cap) {
-        drop_texture(b->wtex_all);   // the stream is idle (synchronised above)
-        if (b->d_wide_all) cudaFree(b->d_wide_all);
-        b->d_wide_all = nullptr;
-        if ((e = cudaMalloc(&b->d_wide_all, sizeof(WNode) * (wo > 0 ? wo : 1)))) return e;
-        b->wide_cap = wo;
-        b->wtex_all = make_int4_texture(b->d_wide_all, (sizeof(WNode) / 16) * (size_t)(wo > 0 ? wo : 1), b->device);
-    }
-    if (to > b->tri_cap) {
-        if (b->d_tri_all) cudaFree(b->d_tri_all);
-        b->d_tri_all = nullptr;
-        if ((e = cudaMalloc(&b->d_tri_all, sizeof(float4) * TRI_F4 * (to > 0 ? to : 1)))) return e;
-        b->tri_cap = to;
-    }
-    b->total_nt = to;
-    for (int s = 0; s < ns; s++) {
-        const Bvh& bv = b->scenes[s]->bvh;
-        if (bv.n_wide > 0) {
-            k_rebase_nodes<<<(unsigned)((bv.n_wide + 255) / 256), 256, 0, b->stream>>>(bv.wide, b->d_wide_all,
-                                                                                     bv.n_wide, desc[s].wide_off,
-                                                                                     desc[s].tri_off);
-            b->launches++;
-        }
-        if (bv.nt > 0 &&
-            (e = cudaMemcpyAsync(b->d_tri_all + TRI_F4 * (int64_t)desc[s].tri_off, bv.tri, sizeof(float4) * TRI_F4 * bv.nt,
-                                 cudaMemcpyDeviceToDevice, b->stream)))
-            return e;
-    }
+    if ((e = copy_trees(b, desc, true, changed))) return e;
     if ((e = cudaGetLastError())) return e;
     if ((e = cudaStreamSynchronize(b->stream))) return e;
     if ((e = cudaMemcpy(b->d_desc, desc.data(), sizeof(SceneDesc) * ns, cudaMemcpyHostToDevice))) return e;

@@ -731,6 +731,7 @@ static cudaError_t build_top(rtsdf_ctx* c) {
 cudaError_t launch_bvh_build(rtsdf_ctx* c) {
     Bvh& b = c->bvh;
     const int64_t n = c->nt;
+    b.gen++;
     b.nt = n;
     b.built = false;
     b.n_wide = 0;
@@ -817,6 +818,7 @@ cudaError_t launch_bvh_build(rtsdf_ctx* c) {
 cudaError_t launch_bvh_refit(rtsdf_ctx* c) {
     Bvh& b = c->bvh;
     const int64_t n = b.nt;
+    b.gen++;
     if (n == 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(b.flags, 0, sizeof(uint32_t) * n, c->stream);
     if (e != cudaSuccess) return e;

@@ -73,6 +73,7 @@ struct Bvh {
     uint32_t* flags = nullptr;     // [nt] bottom-up visit counters
     int32_t* root = nullptr;       // [1] binary root node (device)
     int64_t cap_nt = 0;            // capacity of the per-triangle arrays above
+    uint64_t gen = 0;              // builds and refits so far: a copy of the tree made at another count is stale
     // build scratch, kept across builds: Morton keys / order x 2, radix
     // histograms, and the SAH builder's arena
     uint32_t *mk0 = nullptr, *mk1 = nullptr, *hist = nullptr;

@@ -213,3 +213,56 @@ def test_batch_matches_oracle():
         assert bad.mean() <= 1e-4, (i, int(bad.sum()))
         assert np.isfinite(pipe.u).mean() > 0.5
     b.close()
+
+
+def _shifted(mesh, by):
+    return S.Mesh((mesh.verts + np.asarray(by, np.float32)).astype(np.float32), mesh.tris)
+
+
+@pytest.mark.parametrize("use_graph,split", [(1, 0), (0, 0), (1, 1)])
+@pytest.mark.parametrize("single", [True, False])
+def test_batch_follows_rebuilt_and_refitted_trees(use_graph, split, single):
+    # a rebuild after an upload of the same size, and a refit, keep every
+    # pointer and count of a scene: the batch's copy of the tree must follow
+    # them all the same (a batch of one scene has no later scene's offset that
+    # could tell either)
+    from paper_2210_04449_gb300 import RTSDF
+    items = _workload()[1:2] if single else _workload()[1:4]
+    d, R = 2.0, 8
+    b = _make_batch(items)
+    b.set_tuning(use_graph=use_graph, split_trace=split)
+    plain = []
+    for cfg, mesh in items:
+        rt = RTSDF(**cfg)
+        rt.upload_mesh(mesh.verts, mesh.tris)
+        rt.build_bvh()
+        plain.append(rt)
+
+    def frame_and_compare(f, step):
+        b.frame(d, R, f)
+        b.sync()
+        for i, (sc, rt) in enumerate(zip(b.scenes, plain)):
+            rt.update(d, R, f)
+            rt.sync()
+            got, want = _grids(sc), _grids(rt)
+            for k in ("seeds", "coarse", "accum", "counts", "fine", "masked"):
+                assert np.array_equal(got[k], want[k]), (step, i, k)
+
+    frame_and_compare(0, "first")
+    last = len(items) - 1
+    cfg, mesh = items[last]
+    moved = _shifted(mesh, (0.03, -0.02, 0.04))
+    for rt in (b.scenes[last], plain[last]):
+        rt.upload_mesh(moved.verts, moved.tris)
+        rt.build_bvh()
+    frame_and_compare(1, "same-size upload")
+    for scene in (0, last):
+        for rt in (b.scenes[scene], plain[scene]):
+            rt.set_reset(False)
+            rt.set_objects(np.zeros(items[scene][1].verts.shape[0], np.int32), 1)
+            rt.move_objects(np.array([[-0.05, 0.03, 0.01]], np.float32))
+            rt.build_bvh(refit=True)
+    frame_and_compare(2, "refit")
+    for rt in plain:
+        rt.close()
+    b.close()
