@@ -265,8 +265,8 @@ __global__ void __launch_bounds__(128, 4) k_batch_jfa(BatchArgs b, int p) {
     const uint32_t* in = d.seeds[p & 1];
     uint32_t* out = d.seeds[(p + 1) & 1];
     float* coarse = const_cast<float*>(d.t.coarse);
-    if (p == L - 1) dev::jfa_zblock_column<true, 8, false>(in, out, n, k, x, y, rz, g, coarse, d.hc, d.beta_h);
-    else dev::jfa_zblock_column<false, 8, false>(in, out, n, k, x, y, rz, g, coarse, d.hc, d.beta_h);
+    if (p == L - 1) dev::jfa_zblock_column<true, 8, false, true>(in, out, n, k, x, y, rz, g, coarse, d.hc, d.beta_h);
+    else dev::jfa_zblock_column<false, 8, false, true>(in, out, n, k, x, y, rz, g, coarse, d.hc, d.beta_h);
 }
 
 // Ray prefix over scenes (8 texel slots per masked voxel, `rays` rays

@@ -296,7 +296,7 @@ __global__ void k_top_up(const int32_t* __restrict__ child, int32_t n, const int
     climb(nodes, flags, nbox, c, c >= 0 ? nodes[c].d.z : leaf_parent[~c], lo, hi, nt);
 }
 
-__global__ void k_depth(const int32_t* __restrict__ leaf_parent, const BNode* __restrict__ nodes, int64_t n,
+__global__ void k_depth(const int32_t* __restrict__ leaf_parent, const BNode* nodes, int64_t n,
                         int32_t* depth) {
     chain_begin();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -433,7 +433,7 @@ namespace {
 constexpr int COL_BATCH = 30;   // levels enqueued without a look from the host
 constexpr int COL_WORDS = 2 * (COL_BATCH + 1) + 1;   // the levels, then the binary tree's depth
 
-__device__ __forceinline__ float half_area(const float* __restrict__ nbox, int node) {
+__device__ __forceinline__ float half_area(const float* nbox, int node) {
     const float* p = nbox + 6 * (int64_t)node;
     const float dx = p[3] - p[0], dy = p[4] - p[1], dz = p[5] - p[2];
     return dx * dy + dy * dz + dz * dx;
@@ -483,7 +483,7 @@ __global__ void k_batch_boxes(const int32_t* lev, int levels, int64_t cap, WNode
 // -> 304 us, 104k 710 -> 655, 1M 2415 -> 2320.  Also sets the levels to their
 // start: the root alone.
 __global__ void __launch_bounds__(128) k_collapse_kids(const int32_t* root, int32_t* from, int32_t* lev, int64_t nodes,
-                                                       BNode* bn, const float* __restrict__ nbox) {
+                                                       BNode* bn, const float* nbox) {
     chain_begin();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (blockIdx.x == 0) {
@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(128) k_collapse_kids(const int32_t* root, int3
 // are in `from`.  Writes lev[2 l + 2] (the next level's first slot) and counts
 // its nodes in lev[2 l + 3].
 __global__ void __launch_bounds__(128) k_collapse_level(int32_t* lev, int l, int64_t cap,
-                                                        const BNode* __restrict__ bn, int32_t* from,
+                                                        const BNode* bn, int32_t* from,
                                                         WNode* __restrict__ wide) {
     chain_begin();
     const int32_t first = lev[2 * l];

@@ -415,9 +415,8 @@ __global__ void k_sah_top_single(const int32_t* child_of, BNode* nodes, int32_t*
 // the children (leaf, block range or next-level big range).
 template <int ITEMS>
 __global__ void __launch_bounds__(SAH_THREADS) k_sah_split(const int4* chunks, SahTask* tasks,
-                                                           const int32_t* __restrict__ ord0,
-                                                           const int32_t* __restrict__ ord1,
-                                                           const float4* __restrict__ pbox, uint32_t* bins,
+                                                           const int32_t* ord0, const int32_t* ord1,
+                                                           const float4* pbox, uint32_t* bins,
                                                            uint32_t* hist, int32_t* __restrict__ left_off, Links L,
                                                            SahTask* next, int4* next_chunks, uint32_t* next_bins,
                                                            SahRange* blist, int32_t* counters, int lev,
@@ -440,8 +439,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_split(const int4* chunks, S
     }
     const BinMap m = bin_map(clo, chi);
     const int32_t* ord = T.buf ? ord1 : ord0;
-    __syncthreads();
-    // (all items' loads before the first of them is binned)
+    // (all items' loads before the barrier and before the first of them is binned)
     int32_t t[ITEMS];
     float4 blo[ITEMS], bhi[ITEMS];
 #pragma unroll
@@ -455,6 +453,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_split(const int4* chunks, S
         blo[j] = pbox[b];
         bhi[j] = pbox[b + 1];
     }
+    __syncthreads();
 #pragma unroll
     for (int j = 0; j < ITEMS; j++) {
         if (t[j] < 0) break;
@@ -582,9 +581,9 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_split(const int4* chunks, S
 // final position; big children get their centroid bounds.
 template <int ITEMS>
 __global__ void __launch_bounds__(SAH_THREADS) k_sah_partition(const int4* __restrict__ chunks,
-                                                               const SahTask* __restrict__ tasks,
-                                                               const int32_t* __restrict__ left_off, int32_t* ord0,
-                                                               int32_t* ord1, const float4* __restrict__ pbox,
+                                                               const SahTask* tasks, const int32_t* left_off,
+                                                               int32_t* ord0, int32_t* ord1,
+                                                               const float4* __restrict__ pbox,
                                                                int32_t* __restrict__ order_final, SahTask* next,
                                                                const int32_t* counters, int lev) {
     __shared__ int s_warp[SAH_WARPS];
@@ -604,6 +603,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_partition(const int4* __res
     }
     const BinMap m = bin_map(clo, chi);
     const int axis = T.axis, split = T.split, nl = T.nl, b = T.b, msz = T.e - T.b;
+    const int child[2] = {T.child[0], T.child[1]};
     const int i0 = threadIdx.x * ITEMS;
     int32_t t[ITEMS];
     float c[ITEMS][3];
@@ -629,7 +629,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_partition(const int4* __res
     const int lo_base = b + left_off[blockIdx.x];
     const int ro_base = b + nl + (ch.y - b - left_off[blockIdx.x]);
     int lr = lrank0, rr = min(i0, ch.z) - lrank0;
-    const bool need_cb = T.child[0] >= 0 || T.child[1] >= 0;
+    const bool need_cb = child[0] >= 0 || child[1] >= 0;
 #pragma unroll
     for (int j = 0; j < ITEMS; j++) {
         if (t[j] < 0) continue;
@@ -642,7 +642,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_partition(const int4* __res
     // chunk meet in six words a side
 #pragma unroll
     for (int s = 0; s < 2; s++) {
-        if (T.child[s] < 0) continue;          // block-uniform
+        if (child[s] < 0) continue;            // block-uniform
 #pragma unroll
         for (int k = 0; k < 3; k++) {
             uint32_t lo = 0xFFFFFFFFu, hi = 0u;
@@ -663,7 +663,7 @@ __global__ void __launch_bounds__(SAH_THREADS) k_sah_partition(const int4* __res
     __syncthreads();
     if (threadIdx.x < 12) {
         const int s = threadIdx.x / 6, k = threadIdx.x % 6;
-        const int q = T.child[s];
+        const int q = s ? child[1] : child[0];
         const uint32_t v = s_cb[s][k];
         if (q >= 0 && v != (k < 3 ? 0xFFFFFFFFu : 0u)) {
             if (k < 3) atomicMin(&next[q].cb[k], v);
@@ -933,10 +933,8 @@ __device__ __forceinline__ void warp_split(BlockSmem& S, const SahRange& r, uint
     __syncwarp();   // the next range reuses the bins
 }
 
-__global__ void __launch_bounds__(SAH_THREADS) k_sah_block(const SahRange* __restrict__ blist,
-                                                           const int32_t* __restrict__ ord0,
-                                                           const int32_t* __restrict__ ord1,
-                                                           const float4* __restrict__ pbox,
+__global__ void __launch_bounds__(SAH_THREADS) k_sah_block(const SahRange* blist, const int32_t* ord0,
+                                                           const int32_t* ord1, const float4* pbox,
                                                            int32_t* __restrict__ order_final, Links L,
                                                            int32_t* counters) {
     extern __shared__ __align__(16) unsigned char sah_smem[];

@@ -222,7 +222,11 @@ namespace rtsdf {
 // to memory: it waits until the kernel before has finished and its writes are
 // visible (which has waited the same way, and so on back), and only then lets
 // the next one be launched, so that at most two kernels of a chain overlap and
-// none is started before all but its direct predecessor have ended.  Without
+// none is started before all but its direct predecessor have ended.  A chained
+// kernel therefore lives while its direct predecessor still writes: what that
+// one writes is read through plain loads only, never __ldg or a pointer that is
+// const and __restrict__ (the read-only path and its invariance to the compiler
+// hold for data that nothing changes while the kernel lives).  Without
 // the attribute, or as the first of a chain, the wait is over at once.  A
 // kernel that fills the GPU for long only waits (chain_wait()): the next one's
 // blocks would take places from its own.

@@ -54,8 +54,8 @@ void launch_pass(rtsdf_ctx* c, const uint32_t* in, uint32_t* out, int n, int k, 
 // z-blocked pass (dev::jfa_zblock_column): blocks of 32 x 4 threads in
 // (x, y), blockIdx.z = g k + rz.
 template <bool FINAL, int T, bool AHEAD, bool ZEDGE>
-__global__ void __launch_bounds__(128, 4) k_jfa_zblock(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
-                                                      int n, int k, float* __restrict__ coarse, float hc,
+__global__ void __launch_bounds__(128, 4) k_jfa_zblock(const uint32_t* in, uint32_t* __restrict__ out, int n,
+                                                      int k, float* __restrict__ coarse, float hc,
                                                       float beta_h) {
     chain_begin();
     const int x = blockIdx.x * 32 + threadIdx.x;
@@ -67,13 +67,13 @@ __global__ void __launch_bounds__(128, 4) k_jfa_zblock(const uint32_t* __restric
         const bool ex = __all_sync(0xFFFFFFFFu, x - k < 0 || x + k >= n);
         const bool ey = y - k < 0 || y + k >= n;
         if (x >= n || y >= n) return;
-        if (ex && ey) dev::jfa_zblock_column<FINAL, T, AHEAD, true, 2, 2>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
-        else if (ex) dev::jfa_zblock_column<FINAL, T, AHEAD, true, 2, 3>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
-        else if (ey) dev::jfa_zblock_column<FINAL, T, AHEAD, true, 3, 2>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
-        else dev::jfa_zblock_column<FINAL, T, AHEAD, true, 3, 3>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
+        if (ex && ey) dev::jfa_zblock_column<FINAL, T, AHEAD, false, true, 2, 2>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
+        else if (ex) dev::jfa_zblock_column<FINAL, T, AHEAD, false, true, 2, 3>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
+        else if (ey) dev::jfa_zblock_column<FINAL, T, AHEAD, false, true, 3, 2>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
+        else dev::jfa_zblock_column<FINAL, T, AHEAD, false, true, 3, 3>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
     } else {
         if (x >= n || y >= n) return;
-        dev::jfa_zblock_column<FINAL, T, AHEAD>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
+        dev::jfa_zblock_column<FINAL, T, AHEAD, false>(in, out, n, k, x, y, rz, g, coarse, hc, beta_h);
     }
 }
 

@@ -89,6 +89,8 @@ __device__ __forceinline__ void jfa_voxel(const uint32_t* __restrict__ in, uint3
 // coordinate on that axis (a duplicate of another candidate); a z-slice
 // outside the grid holds no seed.  Slices roll through registers: voxel t
 // needs slices t .. t + 2 only.
+// NC: read the input through the read-only path (only when nothing writes it
+// while the kernel lives: not in a chain, see chain_begin).
 // AHEAD hides a slice's load latency where few warps do (32^3: 12.0 -> 9.4 us,
 // 61^3: 28.4 -> 25.8); with the registers it takes, large grids are slower with
 // it (200^3: 629 -> 683 us).  Tried: keys as whole numbers in fp32, three
@@ -159,8 +161,8 @@ __device__ __forceinline__ uint32_t jfa_argmin(const uint32_t (*ss)[C], const in
     return kmin >= SEEDLESS_KEY_MIN ? SEED_EMPTY : vmin;
 }
 
-template <bool FINAL, int T, bool AHEAD, bool ZEDGE = false, int NX = 3, int NY = 3>
-__device__ __forceinline__ void jfa_zblock_column(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
+template <bool FINAL, int T, bool AHEAD, bool NC, bool ZEDGE = false, int NX = 3, int NY = 3>
+__device__ __forceinline__ void jfa_zblock_column(const uint32_t* in, uint32_t* __restrict__ out,
                                                   int n, int k, int x, int y, int rz, int g,
                                                   float* __restrict__ coarse, float hc, float beta_h) {
     constexpr int C = NX * NY;
@@ -189,6 +191,7 @@ __device__ __forceinline__ void jfa_zblock_column(const uint32_t* __restrict__ i
         ss[j][c] = sv;
         aa[j][c] = dp2a_lo_s_u(wxy, sv, (int)__dp4a(sv, sv, sv & 0x7F000000u));
     };
+    auto read = [](const uint32_t* p) { return NC ? __ldg(p) : *p; };
     auto load_slice = [&](int j) {
         const int z = rz + k * (T * g + j - 1);
         if (z >= 0 && z < n) {
@@ -196,7 +199,7 @@ __device__ __forceinline__ void jfa_zblock_column(const uint32_t* __restrict__ i
 #pragma unroll
             for (int iy = 0; iy < NY; iy++)
 #pragma unroll
-                for (int ix = 0; ix < NX; ix++) take(j, NX * iy + ix, __ldg(in + zo + ys[iy] + xs[ix]));
+                for (int ix = 0; ix < NX; ix++) take(j, NX * iy + ix, read(in + zo + ys[iy] + xs[ix]));
         } else {
 #pragma unroll
             for (int c = 0; c < C; c++) {
@@ -214,7 +217,7 @@ __device__ __forceinline__ void jfa_zblock_column(const uint32_t* __restrict__ i
 #pragma unroll
         for (int iy = 0; iy < NY; iy++)
 #pragma unroll
-            for (int ix = 0; ix < NX; ix++) nx[NX * iy + ix] = in_grid ? __ldg(p + (ys[iy] + xs[ix])) : SEED_EMPTY;
+            for (int ix = 0; ix < NX; ix++) nx[NX * iy + ix] = in_grid ? read(p + (ys[iy] + xs[ix])) : SEED_EMPTY;
     };
     auto take_slice = [&](int j) {
 #pragma unroll

@@ -68,7 +68,9 @@ struct Taps {
 // S at offset (dx, dy, dz) from the lower corner of the scene cube.  The fine
 // grid has n = 2 N >= 2 texels per axis, so a cell's upper neighbour is always
 // the next texel, and the eight taps are four rows of two.
-template <bool GRAD>
+// GRAD: also the taps and the gradient.  NC: read the grid through the
+// read-only path (not in a chained kernel, see chain_begin).
+template <bool GRAD, bool NC>
 __device__ __forceinline__ float sample(const ShadowArgs& a, float dx_, float dy_, float dz_, Taps* tp) {
     const int n = a.n;
     const float d[3] = {dx_, dy_, dz_};
@@ -92,7 +94,7 @@ __device__ __forceinline__ float sample(const ShadowArgs& a, float dx_, float dy
         const int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
         const float wx = dx ? fr[0] : 1.f - fr[0], wy = dy ? fr[1] : 1.f - fr[1], wz = dz ? fr[2] : 1.f - fr[2];
         const int off = dx + n * (dy + n * dz);
-        const float fv = __ldg(p + off);
+        const float fv = NC ? __ldg(p + off) : p[off];
         const float w = wx * wy * wz;
         val = fmaf(w, fv, val);
         if (GRAD) {
@@ -166,7 +168,7 @@ __global__ void __launch_bounds__(SHADOW_THREADS) k_shadow(ShadowArgs a, float* 
         const float qx = fmaf(t, a.Lx, ox), qy = fmaf(t, a.Ly, oy), qz = fmaf(t, a.Lz, oz);
         const float dx = __fsub_rn(qx, a.bx), dy = __fsub_rn(qy, a.by), dz = __fsub_rn(qz, a.bz);
         if (!inside(qx, qy, qz, dx, dy, dz)) break;
-        const float h = sample<false>(a, dx, dy, dz, nullptr);
+        const float h = sample<false, false>(a, dx, dy, dz, nullptr);
         if (h < a.eps) {
             res = 0.f;
             break;
@@ -212,7 +214,7 @@ __global__ void __launch_bounds__(128, 12) k_shadow_bwd(ShadowArgs a, const floa
             const float qx = fmaf(t, a.Lx, ox), qy = fmaf(t, a.Ly, oy), qz = fmaf(t, a.Lz, oz);
             const float dx = __fsub_rn(qx, a.bx), dy = __fsub_rn(qy, a.by), dz = __fsub_rn(qz, a.bz);
             if (!inside(qx, qy, qz, dx, dy, dz)) break;
-            const float h = sample<false>(a, dx, dy, dz, nullptr);
+            const float h = sample<false, true>(a, dx, dy, dz, nullptr);
             if (h < a.eps) {
                 term = true;
                 break;
@@ -258,7 +260,7 @@ __global__ void __launch_bounds__(128, 12) k_shadow_bwd(ShadowArgs a, const floa
                     Taps tp;
                     const float dx = __fsub_rn(fmaf(tj, a.Lx, ox), a.bx), dy = __fsub_rn(fmaf(tj, a.Ly, oy), a.by),
                                 dz = __fsub_rn(fmaf(tj, a.Lz, oz), a.bz);
-                    sample<true>(a, dx, dy, dz, &tp);
+                    sample<true, true>(a, dx, dy, dz, &tp);
 #pragma unroll
                     for (int c = 0; c < 8; c++) atomicAdd(dsdf + tp.idx[c], hbar * tp.w[c]);
                     const float qbx = hbar * tp.grad[0], qby = hbar * tp.grad[1], qbz = hbar * tp.grad[2];
@@ -315,7 +317,7 @@ __global__ void __launch_bounds__(128, 12) k_shadow_bwd(ShadowArgs a, const floa
 // jitter noise with TAA), static camera: the history is clamped to the
 // current frame's 3x3 neighbourhood range (clamped at the border) and
 // blended toward the current value in place, h = hc + blend (cur - hc).
-__global__ void __launch_bounds__(256) k_taa(const float* __restrict__ cur, float* __restrict__ hist, int w,
+__global__ void __launch_bounds__(256) k_taa(const float* cur, float* __restrict__ hist, int w,
                                              int h, float blend) {
     chain_begin();
     const int x = blockIdx.x * 32 + threadIdx.x;
@@ -328,13 +330,13 @@ __global__ void __launch_bounds__(256) k_taa(const float* __restrict__ cur, floa
 #pragma unroll
         for (int dx = -1; dx <= 1; dx++) {
             const int xx = min(max(x + dx, 0), w - 1);
-            const float v = __ldg(cur + (size_t)yy * w + xx);
+            const float v = cur[(size_t)yy * w + xx];
             mn = fminf(mn, v);
             mx = fmaxf(mx, v);
         }
     }
     const size_t i = (size_t)y * w + x;
-    const float c = __ldg(cur + i);
+    const float c = cur[i];
     const float hc = fminf(fmaxf(hist[i], mn), mx);
     hist[i] = fmaf(blend, __fsub_rn(c, hc), hc);
 }

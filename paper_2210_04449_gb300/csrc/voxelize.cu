@@ -23,7 +23,7 @@ namespace {
 
 using namespace dev;
 
-__global__ void k_quantise(const float* __restrict__ verts, int64_t nv, float bx, float by, float bz,
+__global__ void k_quantise(const float* verts, int64_t nv, float bx, float by, float bz,
                            float scale, int n, int32_t* __restrict__ q, uint32_t* err) {
     chain_begin();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -89,8 +89,7 @@ __global__ void __launch_bounds__(128) k_voxelize_small(const int32_t* __restric
 // block split the triangle's voxel box.
 __global__ void __launch_bounds__(256) k_voxelize_big(const int32_t* __restrict__ q,
                                                      const int32_t* __restrict__ tris,
-                                                     const int32_t* __restrict__ big_list,
-                                                     const uint32_t* __restrict__ big_count, int n,
+                                                     const int32_t* big_list, const uint32_t* big_count, int n,
                                                      uint32_t* __restrict__ seeds) {
     chain_begin();
     const uint32_t nb = *big_count;
