@@ -41,8 +41,13 @@ namespace {
 using namespace dev;
 
 constexpr int MAX_BATCH = 256;
-// minimum resident blocks per SM the compiler must allow (register budget
-// 65536 / (128 x this) per thread)
+// Resident blocks per SM of the pipeline launch: the register budget (65536 /
+// (128 x this) per thread) and, see FrameShared, the shared memory allow them.
+// With 7 (shared memory for the prefix and the tracer's state side by side), 64
+// scenes of 32^3 to 128^3 took 753 ms instead of 709 in one launch; the split
+// form, which held the tracer's state without tracing, voxelized in 1.42 instead
+// of 0.95 ms and masked in 1.18 instead of 1.11.  (Three scenes of 8^3 to 16^3:
+// 152 us with 7, 164 with 8, in the barriers.)
 #ifndef BATCH_BLOCKS_PER_SM
 #define BATCH_BLOCKS_PER_SM 8
 #endif
@@ -94,11 +99,10 @@ struct BatchArgs {
     uint32_t spins;
     unsigned long long* stamps;   // [8] global timer at the stage boundaries (block 0)
     BvhRef bvh;               // every scene's BVH in one array (child ids rebased)
-    int split;                // 1: the trace runs as a launch of its own after the pipeline launch
     int phase;                // split form: 1 = stages 0-2 (the jump flood follows as launches of its
-                              // own), 2 = stage 4 on; 0 = the whole frame in one launch
+                              // own), 2 = stage 4 (the trace follows); 0 = the whole frame in one launch
     const uint32_t* jfa_blocks;   // split jump flood: [max_passes][ns + 1] prefix over scenes of their blocks
-    unsigned long long* ray_prefix;   // [ns + 1] split form: ray prefix over scenes, written after the mask
+    unsigned long long* ray_prefix;   // [ns + 1] ray prefix over scenes, written after the mask
     uint32_t* trace_done;     // split trace: blocks done (the last one stamps the frame's end)
 };
 
@@ -122,7 +126,11 @@ __device__ __forceinline__ void stamp(const BatchArgs& b, int k) {
     if (blockIdx.x == 0 && threadIdx.x == 0) write_stamp(b, k);
 }
 
-__device__ bool grid_barrier(const BatchArgs& b) {
+// All blocks of the launch meet; `last` is run by one thread, of the block that
+// arrives last, before any block goes on (a fence first, if it reads what the
+// others wrote).
+template <class F>
+__device__ bool grid_barrier(const BatchArgs& b, F last) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -131,6 +139,7 @@ __device__ bool grid_barrier(const BatchArgs& b) {
         const uint32_t g0 = *gen;
         __threadfence();
         if (atomicAdd(b.bar_count, 1u) + 1u == gridDim.x) {
+            last();
             *b.bar_count = 0u;
             __threadfence();
             atomicAdd(b.bar_gen, 1u);
@@ -149,6 +158,9 @@ __device__ bool grid_barrier(const BatchArgs& b) {
     }
     __syncthreads();
     return s_ok != 0;
+}
+__device__ bool grid_barrier(const BatchArgs& b) {
+    return grid_barrier(b, [] {});
 }
 
 // Stages 1 and 2 of the batched frame, out of line: the 13-axis overlap
@@ -269,18 +281,14 @@ __global__ void __launch_bounds__(128, 4) k_batch_jfa(BatchArgs b, int p) {
     else dev::jfa_zblock_column<false, 8, false, true>(in, out, n, k, x, y, rz, g, coarse, d.hc, d.beta_h);
 }
 
-// Ray prefix over scenes (8 texel slots per masked voxel, `rays` rays
-// each), in shared memory; every thread of the block returns with it.
-__device__ __forceinline__ void batch_ray_prefix(const BatchArgs& b, unsigned long long* s_rp, int ns, int rays) {
-    if (threadIdx.x == 0) {
-        unsigned long long acc = 0;
-        for (int s = 0; s < ns; s++) {
-            s_rp[s] = acc;
-            acc += (unsigned long long)(*(volatile const uint32_t*)b.sc[s].t.count) * 8ull * (unsigned long long)rays;
-        }
-        s_rp[ns] = acc;
+// Ray prefix over scenes (8 texel slots per masked voxel, `rays` rays each).
+__device__ __forceinline__ void batch_ray_prefix(const BatchArgs& b, int ns, int rays) {
+    unsigned long long acc = 0;
+    for (int s = 0; s < ns; s++) {
+        b.ray_prefix[s] = acc;
+        acc += (unsigned long long)(*(volatile const uint32_t*)b.sc[s].t.count) * 8ull * (unsigned long long)rays;
     }
-    __syncthreads();
+    b.ray_prefix[ns] = acc;
 }
 
 // Stage 5: all scenes' rays from one dynamic counter, in units that stay
@@ -320,13 +328,32 @@ struct BatchUnits {
 };
 
 template <bool TEX>
-__device__ __forceinline__ void batch_trace_rays(const BatchArgs& b, const unsigned long long* s_rp, int ns) {
-    __shared__ BlockTrace s_trace;
-    BatchUnits src{b, s_rp, ns};
-    const uint32_t unit = unit_rays(s_rp[ns], (uint32_t)b.params->rays, (uint32_t)b.ray_chunk);
+__device__ __forceinline__ void batch_trace_rays(const BatchArgs& b, BlockTrace& s_trace) {
+    BatchUnits src{b, b.ray_prefix, b.ns};
+    const uint32_t unit = unit_rays(b.ray_prefix[b.ns], (uint32_t)b.params->rays, (uint32_t)b.ray_chunk);
     trace_units<false, TEX>(src, b.bvh, unit, b.refill_min, b.leaf_min, s_trace, nullptr);
 }
 
+// The pipeline's shared memory: the prefix over scenes of their voxels, and
+// once the mask is done with it, the tracer's state in its place.
+template <bool TRACE>
+struct FrameShared {
+    unsigned long long prefix[MAX_BATCH + 1];
+};
+template <>
+struct FrameShared<true> {
+    union {
+        unsigned long long prefix[MAX_BATCH + 1];
+        BlockTrace trace;
+    };
+};
+// 228 KB an SM, of which each block takes 1 KB more than it asks for
+static_assert(sizeof(FrameShared<true>) + 64 <= (228 * 1024) / BATCH_BLOCKS_PER_SM - 1024,
+              "the pipeline's blocks fit an SM's shared memory");
+
+// TRACE: the whole frame in one launch; else the split form's parts, which then
+// hold neither the tracer's shared memory nor its registers.
+template <bool TRACE>
 __global__ void __launch_bounds__(TRACE_THREADS, BATCH_BLOCKS_PER_SM) k_batch_frame(BatchArgs b) {
     const uint64_t tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     const uint64_t nthr = gridDim.x * (uint64_t)blockDim.x;
@@ -335,9 +362,8 @@ __global__ void __launch_bounds__(TRACE_THREADS, BATCH_BLOCKS_PER_SM) k_batch_fr
     __shared__ BatchParams P;
     const int ns = b.ns;
     if (b.phase != 2) stamp(b, 0);
-    // prefix over scenes: voxels in stages 0-4, rays in stages 5-6
-    __shared__ unsigned long long s_prefix[MAX_BATCH + 1];
-    unsigned long long* s_vp = s_prefix;
+    __shared__ FrameShared<TRACE> s_mem;
+    unsigned long long* s_vp = s_mem.prefix;
     if (threadIdx.x == 0) P = *b.params;
     for (int i = threadIdx.x; i <= ns; i += blockDim.x) s_vp[i] = b.vox_prefix[i];
     __syncthreads();
@@ -374,13 +400,14 @@ __global__ void __launch_bounds__(TRACE_THREADS, BATCH_BLOCKS_PER_SM) k_batch_fr
         batch_voxelize_big(b);
         if (!grid_barrier(b)) return;
         stamp(b, 3);
-        if (b.phase == 1) return;   // the jump flood follows as launches of its own (k_batch_jfa)
+        if (!TRACE) return;   // the jump flood follows as launches of its own (k_batch_jfa)
 
         // ---- stage 3: jump flooding, pass p of every scene that has one
-        for (int p = 0; p < b.max_passes; p++) {
-            batch_jfa_pass(b, s_vp, ns, p, tid, nthr);
-            if (!grid_barrier(b)) return;
-        }
+        if constexpr (TRACE)
+            for (int p = 0; p < b.max_passes; p++) {
+                batch_jfa_pass(b, s_vp, ns, p, tid, nthr);
+                if (!grid_barrier(b)) return;
+            }
     }   // stages 0-3
     // scenes without jump steps (N = 1): coarse value straight from the seed
     for (uint64_t s = tid; s < (uint64_t)ns; s += nthr) {
@@ -461,44 +488,40 @@ __global__ void __launch_bounds__(TRACE_THREADS, BATCH_BLOCKS_PER_SM) k_batch_fr
             }
         }
     }
-    if (!grid_barrier(b)) return;
+    // the tracer, here or as a launch of its own, reads the ray prefix from
+    // global memory: one scene's rays follow the other's
+    if (!grid_barrier(b, [&] {
+            __threadfence();
+            batch_ray_prefix(b, ns, P.rays);
+        }))
+        return;
     stamp(b, 5);
 
-    if (b.split) {
-        // the trace follows as a launch of its own; it reads the ray prefix
-        // from global memory
-        if (blockIdx.x == 0) {
-            batch_ray_prefix(b, s_prefix, ns, P.rays);
-            for (int i = threadIdx.x; i <= ns; i += blockDim.x) b.ray_prefix[i] = s_prefix[i];
-        }
-        return;
+    // ---- stage 5: trace all scenes' rays with dynamic fetch, Eq. 1 (stage 6) with it
+    if constexpr (TRACE) {
+        batch_trace_rays<false>(b, s_mem.trace);
+        if (!grid_barrier(b)) return;
+        stamp(b, 6);
+        stamp(b, 7);
     }
-
-    // ---- stage 5: trace all scenes' rays with dynamic fetch
-    unsigned long long* s_rp = s_prefix;
-    __syncthreads();   // every thread is done with the voxel prefix
-    batch_ray_prefix(b, s_rp, ns, P.rays);
-    batch_trace_rays<false>(b, s_rp, ns);
-    if (!grid_barrier(b)) return;
-    stamp(b, 6);
-    stamp(b, 7);
 }
 
 // Split form of stage 5: the trace as its own persistent launch, sized and
 // register-bounded like the per-scene tracer (its occupancy sets its speed:
 // the traversal hides latency with warps); it follows the pipeline launch on
-// the stream and skips its work when that launch gave up at a barrier.  (8 resident blocks, i.e. at most 64
-// registers, as for the per-scene tracer, and for the same measured reason:
-// 7 blocks cost that one 7 %, and 9 leave its stack too little shared
-// memory, 360 against 357 ms on 1M triangles.)
+// the stream and skips its work when that launch gave up at a barrier.  (8
+// resident blocks, i.e. at most 64 registers, as for the per-scene tracer, and
+// for the same measured reason: 7 blocks cost that one 7 %, and 9 leave its
+// stack too little shared memory, 360 against 357 ms on 1M triangles.)
 #ifndef BATCH_TRACE_BLOCKS_PER_SM
 #define BATCH_TRACE_BLOCKS_PER_SM 8
 #endif
 
 template <bool TEX>
 __global__ void __launch_bounds__(TRACE_THREADS, BATCH_TRACE_BLOCKS_PER_SM) k_batch_trace(BatchArgs b) {
+    __shared__ BlockTrace s_trace;
     if (*(volatile const uint32_t*)b.abort) return;
-    batch_trace_rays<TEX>(b, b.ray_prefix, b.ns);
+    batch_trace_rays<TEX>(b, s_trace);
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
@@ -801,14 +824,14 @@ cudaError_t launch_frame_kernel(rtsdf_batch* b) {
     a.bvh.tri = b->d_tri_all;
     a.bvh.nt = b->total_nt;
     a.bvh.err = b->d_ctr + 4;
-    a.split = b->split_trace;
     a.ray_prefix = b->d_ray_prefix;
     a.trace_done = b->d_ctr + 5;
     a.jfa_blocks = b->d_jfa_blocks;
     a.phase = b->split_trace ? 1 : 0;
     void* args[] = {&a};
     b->launches++;
-    cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_batch_frame, dim3(b->grid), dim3(TRACE_THREADS), args,
+    const void* frame = b->split_trace ? (const void*)k_batch_frame<false> : (const void*)k_batch_frame<true>;
+    cudaError_t e = cudaLaunchCooperativeKernel(frame, dim3(b->grid), dim3(TRACE_THREADS), args,
                                                 0, b->stream);
     if (e || !b->split_trace) return e;
     // split form: the jump flood as one launch per pass, the rest of the
@@ -821,8 +844,7 @@ cudaError_t launch_frame_kernel(rtsdf_batch* b) {
     }
     a.phase = 2;
     b->launches++;
-    e = cudaLaunchCooperativeKernel((const void*)k_batch_frame, dim3(b->grid), dim3(TRACE_THREADS), args, 0,
-                                    b->stream);
+    e = cudaLaunchCooperativeKernel(frame, dim3(b->grid), dim3(TRACE_THREADS), args, 0, b->stream);
     if (e) return e;
     b->launches++;
     if (a.bvh.wtex) k_batch_trace<true><<<b->trace_grid, TRACE_THREADS, 0, b->stream>>>(a);
@@ -830,10 +852,17 @@ cudaError_t launch_frame_kernel(rtsdf_batch* b) {
     return cudaGetLastError();
 }
 
+// Resident blocks per SM of the pipeline launch in the batch's form.
+cudaError_t frame_blocks(const rtsdf_batch* b, int* per_sm) {
+    return b->split_trace
+               ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_batch_frame<false>, TRACE_THREADS, 0)
+               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_batch_frame<true>, TRACE_THREADS, 0);
+}
+
 cudaError_t ensure_grid(rtsdf_batch* b) {
     int sms = 0, per_sm = 0;
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
-    if (!e) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_frame, TRACE_THREADS, 0);
+    if (!e) e = frame_blocks(b, &per_sm);
     if (e) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     const int use = (b->blocks_per_sm > 0 && b->blocks_per_sm < per_sm) ? b->blocks_per_sm : per_sm;
@@ -1217,9 +1246,8 @@ extern "C" rtsdf_status rtsdf_batch_autotune(rtsdf_batch_t b, float d_vox, int32
         }
     }
     int per_sm = 0;
-    if (st == RTSDF_OK &&
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_frame, TRACE_THREADS, 0) != cudaSuccess)
-        st = RTSDF_E_CUDA;
+    if (st == RTSDF_OK) st = rtsdf_batch_set_tuning(b, &cur);   // the form that was kept
+    if (st == RTSDF_OK && frame_blocks(b, &per_sm) != cudaSuccess) st = RTSDF_E_CUDA;
     for (int blocks = per_sm - 1; blocks >= per_sm - 2 && blocks >= 1 && st == RTSDF_OK; blocks--) {
         rtsdf_batch_tuning t = cur;
         t.blocks_per_sm = blocks;

@@ -266,3 +266,18 @@ def test_batch_follows_rebuilt_and_refitted_trees(use_graph, split, single):
     for rt in plain:
         rt.close()
     b.close()
+
+
+@pytest.mark.parametrize("split", [0, 1])
+def test_batch_pipeline_blocks_per_sm(split):
+    # the pipeline launch is bounded to registers for eight blocks per SM; its
+    # shared memory (the tracer's state in the single-launch form) must let
+    # eight in too
+    import torch
+    b = _make_batch(_workload()[:2])
+    b.set_tuning(split_trace=split, blocks_per_sm=0)
+    b.frame(2.0, 4, 0)
+    b.sync()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert b.stats()["grid"] >= 8 * sms
+    b.close()
