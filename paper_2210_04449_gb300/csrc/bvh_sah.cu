@@ -181,7 +181,9 @@ __device__ Choice axis_choose(const uint32_t* bins, int a, int lane) {
     float cost = CUDART_INF_F;
     if (lane < NB - 1 && pc > 0 && rc > 0)
         cost = half_area3(plo, phi) * (float)pc + half_area3(rlo, rhi) * (float)rc;
-    float bc = cost;
+    // a cost that is not a number (a vertex moved out of all range) is infinite:
+    // past it, the lanes would come to different splits
+    float bc = fminf(cost, CUDART_INF_F);
     int bl = lane;
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) {

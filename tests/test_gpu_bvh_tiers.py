@@ -70,3 +70,38 @@ def test_large_meshes(n):
     for builder in ("sah", "two_level"):
         for k, ref in got["lbvh"].items():
             assert np.array_equal(got[builder][k], ref), (builder, k)
+
+
+@pytest.mark.parametrize("builder", ["sah", "two_level"])
+@pytest.mark.parametrize("n", [700, 5000])
+def test_moves_out_of_all_range(builder, n):
+    # a move to NaN, to infinity or so far that areas overflow is an error at
+    # the next sync, and a build before it still makes a valid tree: the splits
+    # of ranges that hold such triangles, alone or among others, are the same
+    # for every lane
+    from paper_2210_04449_gb300 import RTSDF, RtsdfError
+    v = _soup(n).reshape(-1, 3).astype(np.float32)
+    t = np.arange(3 * n, dtype=np.int32).reshape(-1, 3)
+    obj = (np.arange(3 * n, dtype=np.int32) // 3) % 50
+    rt = RTSDF(8, seed=2)
+    rt.set_bvh_builder(builder)
+    rt.upload_mesh(v, t)
+    rt.set_objects(obj, 50)
+    by = np.zeros((50, 3), np.float32)
+    by[::7, 0] = np.nan
+    by[3] = np.inf
+    by[11, 1], by[12, 2], by[13] = 3e38, -3e38, 1e25
+    rt.move_objects(by)
+    rt.build_bvh()
+    ch, lt, root = rt.bvh_topology()
+    _check_tree(ch, lt, root, n, in_order=builder == "sah")
+    with pytest.raises(RtsdfError) as ei:
+        rt.sync()
+    assert ei.value.name == "RTSDF_E_MESH"
+    rt.upload_mesh(v, t)
+    rt.build_bvh()
+    rt.update(2.0, 8, 0)
+    rt.sync()
+    pipe = oracle.FinePipeline(np.zeros(3, np.float32), 1.0, 8, 0.5, 2.0, 1.0, 2, accel="bvh")
+    pipe.frame(v, t, 0, 8)
+    assert np.array_equal(rt.grids()["accum"].cpu().numpy().astype(np.float64), pipe.u)
