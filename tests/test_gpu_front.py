@@ -22,6 +22,18 @@ def _triangles(n):
     return v.reshape(-1, 3), np.arange(3 * n, dtype=np.int32).reshape(-1, 3)
 
 
+def _unit(rt, R, chunk, blocks):
+    """Rays of a unit: doubled from one texel's (32 at least) up to the chunk,
+    512 rays and 32 texels, while every warp of the grid gets two units."""
+    import torch
+    total = rt.masked_count() * 8 * R
+    warps = torch.cuda.get_device_properties(0).multi_processor_count * blocks * 4
+    u, most = max(R, 32), min(chunk, 512, 32 * R)
+    while 2 * u <= most and 2 * u * 2 * warps <= total:
+        u *= 2
+    return u
+
+
 SCENES = {
     "one": lambda: _triangles(1),
     "two": lambda: _triangles(2),
@@ -31,15 +43,8 @@ SCENES = {
 }
 
 
-@pytest.mark.parametrize("scene, nc, R, chunk", [
-    ("one", 7, 4, 1024), ("two", 7, 1, 32), ("stacked", 9, 2, 64), ("stacked", 9, 64, 4096),
-    ("soup", 11, 1, 1024), ("soup", 11, 16, 32), ("room", 13, 8, 256), ("room", 21, 32, 1024), ("room", 5, 1024, 64),
-])
-def test_units_and_fronts_match_the_oracle(scene, nc, R, chunk):
-    from paper_2210_04449_gb300 import RTSDF
+def _match(rt, scene, nc, R):
     verts, tris = SCENES[scene]()
-    rt = RTSDF(nc, seed=7)
-    rt.set_tuning(ray_chunk=chunk)
     rt.upload_mesh(verts, tris)
     rt.build_bvh()
     pipe = oracle.FinePipeline(BMIN, 1.0, nc, 0.5, 2.0, 1.0, 7, accel="bvh")
@@ -51,6 +56,52 @@ def test_units_and_fronts_match_the_oracle(scene, nc, R, chunk):
     cnt = g["counts"].cpu().numpy().astype(np.int64)
     assert np.array_equal(g["accum"].cpu().numpy().astype(np.float64), pipe.u)
     assert np.array_equal(cnt & 0xFFFF, pipe.nF) and np.array_equal(cnt >> 16, pipe.nB)
+
+
+# (a full grid has more warps than these frames have units: the smallest ones,
+# of 32 rays or one texel, up to 128 in the last but one)
+@pytest.mark.parametrize("scene, nc, R, chunk", [
+    ("one", 7, 4, 1024), ("two", 7, 1, 32), ("stacked", 9, 2, 64), ("stacked", 9, 64, 4096),
+    ("soup", 11, 1, 1024), ("soup", 11, 16, 32), ("room", 13, 8, 256), ("room", 21, 32, 1024), ("room", 5, 1024, 64),
+])
+def test_units_and_fronts_match_the_oracle(scene, nc, R, chunk):
+    from paper_2210_04449_gb300 import RTSDF
+    rt = RTSDF(nc, seed=7)
+    rt.set_tuning(ray_chunk=chunk)
+    _match(rt, scene, nc, R)
+
+
+@pytest.mark.parametrize("scene, nc, R, chunk, unit", [
+    ("soup", 11, 16, 1024, 128), ("room", 28, 4, 1024, 128), ("room", 21, 32, 256, 256), ("room", 24, 16, 1024, 512),
+    ("room", 21, 32, 1024, 512), ("stacked", 20, 64, 4096, 512),
+])
+def test_units_of_many_texels_match_the_oracle(scene, nc, R, chunk, unit):
+    """One block per SM, so that units grow: 8 to 32 texels each, with fronts
+    of 40 (below 256 rays) and 64 entries."""
+    from paper_2210_04449_gb300 import RTSDF
+    rt = RTSDF(nc, seed=7)
+    rt.set_tuning(ray_chunk=chunk, trace_blocks_per_sm=1)
+    _match(rt, scene, nc, R)
+    assert _unit(rt, R, chunk, 1) == unit
+
+
+def test_vote_does_not_depend_on_the_unit():
+    """A full grid: units of one texel against units of 512 rays."""
+    from paper_2210_04449_gb300 import RTSDF
+    m = S.room_scene(3, n_objects=30, n_spheres=12, subdiv=2)
+    out = []
+    for chunk in (32, 1024):
+        rt = RTSDF(56, seed=3)
+        rt.set_tuning(ray_chunk=chunk)
+        rt.upload_mesh(m.verts, m.tris)
+        rt.build_bvh()
+        for t in range(2):
+            rt.update(2.0, 64, t)
+        rt.sync()
+        assert _unit(rt, 64, chunk, 8) == (64 if chunk == 32 else 512)
+        out.append({k: rt.grids()[k].cpu().numpy().copy() for k in ("accum", "counts", "fine")})
+    for k in out[0]:
+        assert np.array_equal(out[0][k], out[1][k]), k
 
 
 def test_nearest_face_does_not_depend_on_the_unit():
