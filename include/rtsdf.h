@@ -358,9 +358,11 @@ rtsdf_status rtsdf_jfa_noalloc(const uint32_t* seeds_in, uint32_t* seeds_out, fl
  * pipeline of Sec. 2.1-2.2 (voxelize, jump flood, mask, trace, Eq. 1) for
  * every scene in one persistent cooperative kernel launch, replayed from a
  * CUDA graph; with split_trace = 1 that launch stops after the mask and the
- * trace of every scene follows as a launch of its own in the same graph.  Each scene's result equals a plain
- * per-scene frame (same kernels' arithmetic, same rays).  Scenes must be
- * static within the batch (no pending rtsdf_move_objects).
+ * trace of every scene follows as a launch of its own in the same graph.
+ * Each scene's result equals a plain per-scene frame (same kernels'
+ * arithmetic, same rays).  Scenes must be static within a frame (no pending
+ * rtsdf_move_objects); a mesh uploaded or a BVH built or refitted between
+ * frames is followed.
  * ------------------------------------------------------------------------ */
 typedef struct rtsdf_batch* rtsdf_batch_t;
 
@@ -388,7 +390,8 @@ typedef struct {
     /* stage times of the last frame, ms (global timer read at the stage
        barriers; with split_trace, trace runs from the end of the pipeline
        launch to the end of the last trace block): clear, voxelize, large
-       triangles, jump flood, mask, trace (with Eq. 1), and 0 */
+       triangles, jump flood, mask, trace (with Eq. 1); the last is
+       reserved and 0 */
     float stage_ms[7];
 } rtsdf_batch_info;
 

@@ -390,6 +390,7 @@ class RTSDFBatch:
         s = _abi.BatchInfo()
         call("rtsdf_batch_stats", self._h, ctypes.byref(s))
         out = {k: getattr(s, k) for k, _ in _abi.BatchInfo._fields_ if k != "stage_ms"}
+        # (the trace stage applies Eq. 1: "finalize" is a reserved slot and 0)
         names = ("clear", "voxelize", "voxelize_large", "jfa", "mask", "trace", "finalize")
         out["stage_ms"] = {n: round(float(s.stage_ms[i]), 4) for i, n in enumerate(names)}
         return out

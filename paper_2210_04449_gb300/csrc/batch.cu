@@ -97,7 +97,7 @@ struct BatchArgs {
     int ray_chunk;
     int leaf_min;
     uint32_t spins;
-    unsigned long long* stamps;   // [8] global timer at the stage boundaries (block 0)
+    unsigned long long* stamps;   // [7] global timer at the stage boundaries (block 0)
     BvhRef bvh;               // every scene's BVH in one array (child ids rebased)
     int phase;                // split form: 1 = stages 0-2 (the jump flood follows as launches of its
                               // own), 2 = stage 4 (the trace follows); 0 = the whole frame in one launch
@@ -497,12 +497,11 @@ __global__ void __launch_bounds__(TRACE_THREADS, BATCH_BLOCKS_PER_SM) k_batch_fr
         return;
     stamp(b, 5);
 
-    // ---- stage 5: trace all scenes' rays with dynamic fetch, Eq. 1 (stage 6) with it
+    // ---- stage 5: trace all scenes' rays with dynamic fetch, and Eq. 1
     if constexpr (TRACE) {
         batch_trace_rays<false>(b, s_mem.trace);
         if (!grid_barrier(b)) return;
         stamp(b, 6);
-        stamp(b, 7);
     }
 }
 
@@ -525,10 +524,7 @@ __global__ void __launch_bounds__(TRACE_THREADS, BATCH_TRACE_BLOCKS_PER_SM) k_ba
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(b.trace_done, 1u) == gridDim.x - 1) {   // the last block out
-            write_stamp(b, 6);
-            write_stamp(b, 7);
-        }
+        if (atomicAdd(b.trace_done, 1u) == gridDim.x - 1) write_stamp(b, 6);   // the last block out
     }
 }
 
@@ -915,8 +911,8 @@ rtsdf_status rtsdf_batch_create(const rtsdf_config* cfgs, int32_t n, rtsdf_batch
         if (!e) e = cudaMemset(b->d_ctr, 0, sizeof(uint32_t) * 8);
         if (!e) e = cudaMalloc(&b->d_next_ray, sizeof(unsigned long long));
         if (!e) e = cudaMalloc(&b->d_ray_prefix, sizeof(unsigned long long) * (MAX_BATCH + 1));
-        if (!e) e = cudaMalloc(&b->d_stamps, sizeof(unsigned long long) * 8);
-        if (!e) e = cudaMemset(b->d_stamps, 0, sizeof(unsigned long long) * 8);
+        if (!e) e = cudaMalloc(&b->d_stamps, sizeof(unsigned long long) * 7);
+        if (!e) e = cudaMemset(b->d_stamps, 0, sizeof(unsigned long long) * 7);
         if (!e) e = cudaMalloc(&b->d_params, sizeof(BatchParams));
         if (!e) e = cudaMallocHost(&b->h_params, sizeof(BatchParams));
         if (!e) e = cudaEventCreate(&b->ev0);
@@ -1097,9 +1093,9 @@ rtsdf_status rtsdf_batch_stats(rtsdf_batch_t b, rtsdf_batch_info* out) {
     float ms = -1.f;
     if (b->frames > 0 && cudaEventElapsedTime(&ms, b->ev0, b->ev1) != cudaSuccess) ms = -1.f;
     out->last_frame_ms = ms;
-    unsigned long long st[8];
+    unsigned long long st[7];
     if (cudaMemcpy(st, b->d_stamps, sizeof(st), cudaMemcpyDeviceToHost) == cudaSuccess)
-        for (int k = 0; k < 7; k++) out->stage_ms[k] = st[k + 1] >= st[k] ? (float)((st[k + 1] - st[k]) * 1e-6) : 0.f;
+        for (int k = 0; k < 6; k++) out->stage_ms[k] = st[k + 1] >= st[k] ? (float)((st[k + 1] - st[k]) * 1e-6) : 0.f;
     return RTSDF_OK;
 }
 

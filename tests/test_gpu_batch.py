@@ -61,8 +61,8 @@ def _make_batch(items):
 
 @pytest.mark.parametrize("use_graph,split", [(1, 0), (0, 0), (1, 1), (0, 1)])
 def test_batch_equals_sequential(use_graph, split):
-    # split = 1: the trace and the Eq. 1 finalize run as launches of their
-    # own after the pipeline launch; the grids must not change
+    # split = 1: the trace (with Eq. 1) runs as a launch of its own after the
+    # pipeline launch; the grids must not change
     items = _workload()
     d, R, frames = 2.0, 8, [0, 1, 2]
     b = _make_batch(items)
@@ -85,8 +85,8 @@ def test_batch_equals_sequential(use_graph, split):
 
 @pytest.mark.parametrize("split", [0, 1])
 def test_batch_barrier_timeout_reported_then_recovers(split):
-    # with split = 1 the trace and finalize launches see the abort flag and
-    # skip their work
+    # with split = 1 the flood's and the trace's launches see the abort flag
+    # and skip their work
     from paper_2210_04449_gb300 import RtsdfError
     items = _workload()
     d, R = 2.0, 4
