@@ -46,7 +46,6 @@ constexpr int SAH_THREADS = 256;
 constexpr int SAH_ITEMS = SAH_CH / SAH_THREADS;
 constexpr int SAH_WARPS = SAH_THREADS / 32;
 constexpr int WARP_MAX = 32;                  // largest range of the exact warp build
-constexpr int BLK_STACK = 48;                 // disjoint ranges > 32 in 1024: at most 31
 // Largest range of the block tier that one warp bins and splits, so that the
 // ranges of a level are split side by side and without block barriers (which
 // bound the tier: 4.5 of its stalls per issue).  Whole build with 256 against
@@ -55,6 +54,7 @@ constexpr int BLK_STACK = 48;                 // disjoint ranges > 32 in 1024: a
 // ranges from a list as they come, without rounds, were slower: 520 us at 2.2k.
 constexpr int MID_MAX = 256;
 constexpr int MID_CAP = 32;                   // disjoint ranges > 32 in 1024: at most 31
+constexpr int BLK_STACK = SAH_CH / MID_MAX;   // disjoint ranges > MID_MAX in SAH_CH: at most 3
 constexpr int WLIST_CAP = SAH_CH / 2;         // disjoint ranges >= 2 in 1024
 constexpr unsigned FULL = 0xFFFFFFFFu;
 

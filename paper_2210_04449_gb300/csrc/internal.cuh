@@ -67,7 +67,7 @@ struct Bvh {
     cudaTextureObject_t wtex = 0;  // the wide nodes as int4 texels (0: none; see make_int4_texture)
     float* nbox = nullptr;         // [nt - 1][6] box of every binary node
     float* lbox = nullptr;         // [nt][6] padded box of every leaf
-    float4* tri = nullptr;         // [3 nt] per leaf: (v0, orig idx bits), (e1, 0), (e2, 0)
+    float4* tri = nullptr;         // [TRI_F4 nt] per leaf: (v0, orig idx bits), (e1, 0), (e2, 0), pad
     int32_t* leaf_tri = nullptr;   // [nt] original triangle index of each leaf
     int32_t* leaf_parent = nullptr;// [nt]
     uint32_t* flags = nullptr;     // [nt] bottom-up visit counters

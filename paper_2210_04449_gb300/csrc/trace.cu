@@ -66,7 +66,7 @@ struct SceneUnits {
 template <bool COUNT, bool TEX>
 __global__ void __launch_bounds__(TRACE_THREADS, TRACE_MIN_BLOCKS) k_trace(TraceArgs a) {
     __shared__ BlockTrace s_trace;
-    __shared__ TraceArgs s_args;   // for the parts that are called
+    __shared__ TraceArgs s_args;   // what the unit source reads at refills
     chain_wait();
     if (threadIdx.x == 0) s_args = a;
     __syncthreads();

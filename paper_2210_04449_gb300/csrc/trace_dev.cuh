@@ -173,14 +173,6 @@ struct Stack {
     }
 };
 
-// Traversal in two phases.  With one triangle per leaf, a warp in which
-// every lane takes either a node step or a leaf step would pay both paths on
-// almost every iteration.  So a lane that reaches a leaf parks it (one per
-// lane) and keeps entering internal nodes; the warp runs the leaf phase only
-// when enough lanes hold a parked leaf or some cannot continue.  The order of
-// triangle tests does not change the closest hit (every triangle whose box
-// the ray meets is tested unless its entry distance exceeds the best hit).
-
 // Pop the next entry that can still hold a hit at distance <= bt, parking
 // leaves while the lane's slot is free; stops at an internal node, at a leaf
 // behind the parked one, or with the stack (and what lies below it) empty
