@@ -50,18 +50,18 @@ FLOP_PER_TEST = 30
 INST_PER_RAY = {
     # ncu --metrics smsp__inst_executed.sum,gpu__time_duration.sum,dram__bytes_read.sum,dram__bytes_write.sum
     # -k regex:k_trace -c 1 on "bench.py --steps 2 --warmup 1 --no-cpu-baseline --no-batch --no-variant
-    # --no-configs" (1 pass; the first frame's launch, 349.43 ms): 308,462,238,999 warp instructions over
+    # --no-configs" (1 pass; the first frame's launch, 349.67 ms): 308,463,217,306 warp instructions over
     # 2,557,074 masked voxels x 8 texels x 64 rays = 1,309,221,888 rays
-    "d8df5449bd0b4eca": 235.61,
+    "48db0fe3125046c6": 235.61,
 }
 
 # DRAM bytes per launch of the tracer, from an ncu capture (profiles/), keyed
 # by the sha256 of the sources it was measured on (the kernel and the BVH
 # builders, whose tree it walks); reported as null once any of them changes.
 TRAFFIC = {
-    # the same capture as INST_PER_RAY above (first k_trace<0, 1> launch, SAH tree): 17.93 GB read +
-    # 936.23 MB written (the accumulator, counts and fine SDF of the traced texels)
-    "d8df5449bd0b4eca": 17.93e9 + 936.23e6,
+    # the same capture as INST_PER_RAY above (first k_trace<0, 1> launch, SAH tree): 17.92 GB read +
+    # 934.32 MB written (the accumulator, counts and fine SDF of the traced texels)
+    "48db0fe3125046c6": 17.92e9 + 934.32e6,
 }
 TRAFFIC_SOURCES = ("trace.cu", "trace_dev.cuh", "front_dev.cuh", "bvh.cu", "bvh_sah.cu")
 
