@@ -269,6 +269,43 @@ def test_batch_follows_rebuilt_and_refitted_trees(use_graph, split, single):
 
 
 @pytest.mark.parametrize("split", [0, 1])
+def test_batch_follows_two_level_refits(split):
+    # a two-level refit collapses the tree anew: the number of its 4-wide nodes
+    # may change, also in the last scene, where no later offset shows it
+    from paper_2210_04449_gb300 import RTSDF, RTSDFBatch
+    d, R = 2.0, 8
+    meshes = [S.animated_scene(k, n_objects=15, n_lon=12, n_lat=7) for k in (4, 5)]
+    b = RTSDFBatch([dict(coarse_n=24, seed=k) for k in range(2)])
+    b.set_tuning(split_trace=split)
+    plain = [RTSDF(24, seed=k) for k in range(2)]
+    for rts in (b.scenes, plain):
+        for rt, m in zip(rts, meshes):
+            rt.set_bvh_builder("two_level")
+            rt.upload_mesh(m.verts, m.tris)
+            rt.set_objects(m.vert_object, m.n_objects)
+            rt.set_reset(False)
+            rt.build_bvh()
+    rng = np.random.default_rng(2)
+    for f in range(4):
+        b.frame(d, R, f)
+        b.sync()
+        for sc, rt in zip(b.scenes, plain):
+            rt.update(d, R, f)
+            rt.sync()
+            got, want = _grids(sc), _grids(rt)
+            for k in ("accum", "counts", "fine", "masked"):
+                assert np.array_equal(got[k], want[k]), (f, k)
+        for i, m in enumerate(meshes):
+            by = rng.uniform(-0.02, 0.02, (m.n_objects, 3)).astype(np.float32)
+            for rt in (b.scenes[i], plain[i]):
+                rt.move_objects(by)
+                rt.build_bvh(refit=True)
+    for rt in plain:
+        rt.close()
+    b.close()
+
+
+@pytest.mark.parametrize("split", [0, 1])
 def test_batch_pipeline_blocks_per_sm(split):
     # the pipeline launch is bounded to registers for eight blocks per SM; its
     # shared memory (the tracer's state in the single-launch form) must let
